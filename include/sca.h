@@ -34,6 +34,14 @@
  *  - Arrays of N = L*L sites are float64 in site order i = x*L + y.
  *  - A context is not thread-safe; use one per thread.  A server is safe for
  *    concurrent sca_submit / sca_poll from several threads.
+ *  - Elimination.  Every evaluation eliminates all 2 n_omega blocks A_{n,sigma} exactly.  From
+ *    L = 8 up, and while pi T >= 0.03 |t| (for a density of states: eta >= 0.03 |t|), it goes
+ *    through the lattice's sparsity: nested dissection of the torus, then the entries of
+ *    A^{-1} inside the fronts, in float64 (SCA_PREC_FP64) or double-float (48 bits, the other
+ *    three).  Below that line, for smaller lattices, and where the caller asks for it
+ *    (sca_set_pivoting, sca_set_panel_precision, sca_profile_enable(ctx, 1), or one of the
+ *    dense elimination's environment switches set when the context is created), every block is
+ *    eliminated as a dense matrix in the context's precision ("the dense elimination" below).
  *  - Blocks are numbered b = 2n + s with s = 0 for sigma = +1 (up) and s = 1
  *    for sigma = -1 (down).
  */
@@ -63,7 +71,8 @@ typedef enum {
   SCA_ENOSTATE = 9     /* call order: e.g. sca_adam_step before sca_adam_init */
 } sca_status;
 
-/* Arithmetic of the dense contractions.  FP64: everything in float64.
+/* Arithmetic of the dense elimination's contractions (the nested elimination computes in float64
+ * for SCA_PREC_FP64 and in double-float for the other three).  FP64: everything in float64.
  * FP32: blocks stored as complex64, CUDA-core float32 contractions.
  * 3XTF32: complex64 blocks, contractions on tcgen05 tensor cores in split
  * TF32 (hi*hi + hi*lo + lo*hi, hi = the value with 13 low mantissa bits cleared) with
@@ -123,14 +132,13 @@ sca_status sca_workspace_bytes(const sca_params* params, uint64_t* bytes);
  * it.  Errors: SCA_EINVAL, SCA_ECUDA. */
 sca_status sca_set_site_energy(sca_ctx* ctx, const double* eps_extra_host);
 
-/* Omega(phi) for a host field phi (N doubles).  Runs the blocked pivoted LU
- * of every block (Eq. 2; no inverse).  Errors: SCA_EINVAL, SCA_ENONFINITE,
- * SCA_ECUDA. */
+/* Omega(phi) for a host field phi (N doubles): elimination of every block
+ * (Eq. 2; no inverse).  Errors: SCA_EINVAL, SCA_ENONFINITE, SCA_ECUDA. */
 sca_status sca_potential(sca_ctx* ctx, const double* phi_host, double* omega);
 
-/* Omega(phi) and its gradient (grad: N host doubles).  Runs the blocked
- * Gauss-Jordan inversion of every block, whose pivots are those of the LU
- * (same ln|det|) and whose result is G = A^{-1}.  Errors as sca_potential. */
+/* Omega(phi) and its gradient (grad: N host doubles) from the diagonal of
+ * G = A^{-1} of every block (dense elimination: blocked Gauss-Jordan inversion,
+ * whose pivots are those of the LU).  Errors as sca_potential. */
 sca_status sca_grad(sca_ctx* ctx, const double* phi_host, double* omega, double* grad);
 
 /* Device-pointer variants.  d_phi: N doubles; d_omega: 1 double; d_grad: N
@@ -143,10 +151,10 @@ sca_status sca_grad_dev(sca_ctx* ctx, const double* d_phi, double* d_omega, doub
                         void* stream);
 
 /* Autograd split (device pointers, asynchronous on `stream`).
- * sca_forward_dev: Omega(phi) through the blocked Gauss-Jordan inversion of every block; the
- * inverses stay resident in the context's workspace.
- * sca_backward_dev: the adjoint stage from those resident inverses: the diagonal of
- * G = A^{-1} (refined in float64 for the reduced precisions) reduced into
+ * sca_forward_dev: Omega(phi) through the elimination of every block; the eliminated fronts (or
+ * dense inverses) stay resident in the context's workspace.
+ * sca_backward_dev: the adjoint stage from what is resident: the diagonal of
+ * G = A^{-1} (dense elimination in the reduced precisions: refined in float64) reduced into
  * d_grad = dOmega/dphi.  It must follow a sca_forward_dev with the same d_phi contents and no
  * other call on the context in between; it returns SCA_ENOSTATE otherwise, or when the
  * workspace is chunked (not every block resident). */
@@ -304,8 +312,8 @@ sca_status sca_set_wait_limit(sca_ctx* ctx, int64_t cycles);
  * broadening.  rho_out (host, 2 n_w doubles): spin up (sigma = +1) at [0, n_w), spin down at
  * [n_w, 2 n_w).  The resolvents go through the same batched elimination as the gradient, in
  * batches of n_omega frequencies (the context's block slots), with partial pivoting unless
- * eta > 4|t| or the context is set to SCA_PIVOT_NONE; the mixed precisions take Im G_ii from
- * the float32 inverse without refinement.  Invalidates the inverses kept for
+ * eta > 4|t| or the context is set to SCA_PIVOT_NONE (dense elimination, eta < 0.03 |t|: the
+ * mixed precisions take Im G_ii from the float32 inverse without refinement).  Invalidates the inverses kept for
  * sca_backward_dev.  SCA_EINVAL for bad arguments, SCA_ENONFINITE for a singular resolvent. */
 sca_status sca_dos(sca_ctx* ctx, const double* phi_host, const double* w_host, int32_t n_w,
                    double eta, double* rho_out);
@@ -330,12 +338,14 @@ sca_status sca_metropolis_init(sca_ctx* ctx, const double* phi0_host, double del
 sca_status sca_metropolis_step(sca_ctx* ctx, int32_t n_steps, double* omega_trace,
                                uint8_t* accepted, double* omega, int64_t* accepted_total);
 
-/* Pivoting of the batched elimination of the A_{n,sigma} (Sec. II, Eq. 2).
- *   SCA_PIVOT_PARTIAL (default): partial pivoting for the blocks whose column diagonal
+/* Pivoting of the elimination of the A_{n,sigma} (Sec. II, Eq. 2).  A new context takes the nested
+ * elimination where it applies (no interchanges: -i A and all its Schur complements have the
+ * Hermitian part omega_n I > 0) and SCA_PIVOT_PARTIAL elsewhere.
+ *   SCA_PIVOT_PARTIAL: the dense elimination, with partial pivoting for the blocks whose column diagonal
  *     dominance is not guaranteed (omega_n <= 4|t|); the remaining blocks provably keep their
  *     diagonal pivots and skip the search.
- *   SCA_PIVOT_NONE: every block is eliminated without interchanges, as a complex-symmetric
- *     (LDL^T-type) elimination that updates one triangle on the tensor-core path.  The paper
+ *   SCA_PIVOT_NONE: every block is eliminated without interchanges: nested where it applies,
+ *     elsewhere as a dense complex-symmetric (LDL^T-type) elimination that updates one triangle on the tensor-core path.  The paper
  *     has no such variant.  -i A_{n,sigma} has Hermitian part omega_n I > 0, so every leading
  *     principal minor is nonzero and the elimination exists; its growth has no a-priori bound
  *     and rises as omega_n falls (the largest growth met in tests is below 10, down to
@@ -348,11 +358,13 @@ sca_status sca_set_pivoting(sca_ctx* ctx, int32_t mode);
  * the interchanges with U12 and the rest-of-panel update) on the reduced-precision paths:
  * SCA_PREC_FP32 (default: the blocks' compute type) or SCA_PREC_FP64 (float64 arithmetic on
  * the float32 blocks; the doubled shared-memory panel narrows the sub-panels, e.g. to 4
- * columns at N = 1600).  The pivot-block inverses and the contractions are unchanged.  Float64
- * contexts accept only SCA_PREC_FP64.  Applies from the next call; SCA_EINVAL otherwise. */
+ * columns at N = 1600) takes the dense elimination.  The pivot-block inverses and the
+ * contractions are unchanged.  Float64 contexts accept only SCA_PREC_FP64.  Applies from the
+ * next call; SCA_EINVAL otherwise. */
 sca_status sca_set_panel_precision(sca_ctx* ctx, int32_t prec);
 
-/* SM partitions for the two block groups (driver green contexts).  The pivoted group (the
+/* SM partitions for the two block groups of the dense elimination (driver green contexts; the
+ * nested elimination has one group and takes every SM).  The pivoted group (the
  * lowest frequencies, a chain of short dependent launches) and the dominant group (bandwidth-
  * bound launches that fill every SM they reach) run side by side on one GPU; with a
  * partition, every launch of the dominant group stays on the SMs outside a set of
@@ -390,8 +402,10 @@ sca_status sca_sm_partition(sca_ctx* ctx, int32_t* pivoted_sms, int32_t* dominan
  * kernels above, so they are not part of any sum), 13 update of the rest of a pivoted outer
  * panel after each sub-panel, 14 rank-nb factors of the pivoted group, 15 the first update of a
  * merged pair of elimination steps of the dominant blocks (only the second step's row and column
- * strips; the merged update of the rest is kind 5).  Enabling resets the
- * counters.  Timing adds a small host overhead per launch; keep it off when measuring
+ * strips; the merged update of the rest is kind 5), 16 and 17 one tree level of the nested
+ * elimination and of its diag(G).  enable = 1 times the dense elimination, which the context then
+ * takes (kinds 0 to 15 are its kernels); enable = 2 times whatever the context takes without
+ * profiling.  Enabling resets the counters.  Timing adds a small host overhead per launch; keep it off when measuring
  * throughput.  With the environment variable SCA_PROFILE_TRACE set to a file name, each
  * synchronisation also appends the launches it collected to that file, one line each:
  * kind name, stream index (order of first use), start and duration in ms from the first. */

@@ -219,7 +219,7 @@ class Context:
         return om, g
 
     def forward_dev(self, phi_t, omega_t) -> int:
-        """Omega via the inversion; returns the generation whose inverses stay resident."""
+        """Omega via the elimination; returns the generation whose fronts stay resident."""
         gen = self._bump()
         check(_lib.lib().sca_forward_dev(self._h, ctypes.c_void_p(phi_t.data_ptr()),
                                          ctypes.c_void_p(omega_t.data_ptr()), self._stream()))
@@ -239,7 +239,7 @@ class Context:
     # ---- streams and per-kernel timing
     KINDS = ["assemble", "panel", "swap", "trinv", "prep", "update", "refine", "reduce", "diag",
              "update_piv", "fused", "span_pivoted", "span_dominant", "panel_update", "prep_piv",
-             "update_cross"]
+             "update_cross", "nest_up", "nest_down"]
 
     def set_stream(self, stream=None):
         """Enqueue on a torch.cuda.Stream (or raw handle); None restores the own stream."""
@@ -251,8 +251,9 @@ class Context:
         check(_lib.lib().sca_set_wait_limit(self._h, int(cycles)))
 
     def set_pivoting(self, mode: str = "partial"):
-        """'partial': partial pivoting where diagonal dominance is not guaranteed (default);
-        'none': every block eliminated without interchanges (complex-symmetric elimination)."""
+        """'partial': dense elimination, partial pivoting where diagonal dominance is not
+        guaranteed; 'none': no interchanges (nested elimination where it applies, as in a new
+        context; else a dense complex-symmetric elimination)."""
         modes = {"partial": 0, "none": 1}
         if mode not in modes:
             raise ValueError(f"pivoting mode must be one of {sorted(modes)}")
@@ -283,8 +284,10 @@ class Context:
         check(_lib.lib().sca_sm_partition(self._h, ctypes.byref(p), ctypes.byref(d)))
         return p.value, d.value
 
-    def profile(self, enable: bool = True):
-        check(_lib.lib().sca_profile_enable(self._h, 1 if enable else 0))
+    def profile(self, enable: bool | int = True):
+        """True: time the dense elimination's kernels, which the context then takes; 2: time
+        whatever it takes without profiling; False: off."""
+        check(_lib.lib().sca_profile_enable(self._h, int(enable)))
 
     def profile_read(self) -> dict:
         out = {}

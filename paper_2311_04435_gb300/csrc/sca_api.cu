@@ -110,6 +110,23 @@ static sca_status validate_adam(const sca_adam* a) {
   return SCA_OK;
 }
 
+// The environment switches of the dense elimination (its comparison paths and tile sizes): a
+// context created with one of them set takes that elimination, which they are about.
+static bool dense_switch_set() {
+  static const char* const names[] = {"SCA_PIVOT_ALL",    "SCA_SYM",          "SCA_REFINE_LOWER",
+                                      "SCA_TINV_BLOCKED", "SCA_PIVOTED_FIRST", "SCA_FUSED_SWAP",
+                                      "SCA_DIAG_TC",      "SCA_PAIR",          "SCA_NB",
+                                      "SCA_ALT_POLICY",   "SCA_SM_RESERVE"};
+  for (const char* n : names)
+    if (std::getenv(n)) return true;
+  return false;
+}
+
+bool nested_now(const Engine& e) {
+  if (!e.nest || e.dense_only || (e.prof && e.prof->on && e.prof->dense)) return false;
+  return e.dos_mode ? nested_rule(e.p.t, e.dos_eta, e.dos_eta) : e.nest_rule;
+}
+
 static size_t round_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 sca_status plan(const sca_params& p, Engine& e) {
@@ -173,6 +190,8 @@ sca_status plan(const sca_params& p, Engine& e) {
   e.pair = e.tc && e.nb == 128 && e.N > e.nb && e.B > e.piv_blocks;
   if (const char* v = std::getenv("SCA_PAIR"))
     if (std::atoi(v) == 0) e.pair = false;
+  e.nest_rule = nested_rule(p.t, M_PI * p.T, (2.0 * p.n_omega - 1.0) * M_PI * p.T);
+  e.dense_only = dense_switch_set();
   size_t bytes = 0;
   bytes += (size_t)e.chunk * e.mat_stride * S;           // blocks
   bytes += 2 * (size_t)e.chunk * e.fw_mat * S;            // F, W
@@ -205,9 +224,15 @@ sca_status allocate(Engine& e) {
   sca_status st;
 #define SCA_ALLOC(ptr, bytes, what) \
   if ((st = dev_alloc(&(ptr), (bytes), e, what)) != SCA_OK) return st;
-  SCA_ALLOC(e.M, (size_t)e.chunk * e.mat_stride * S, "blocks");
-  SCA_ALLOC(e.F, (size_t)e.chunk * e.fw_mat * S, "F");
-  SCA_ALLOC(e.W, (size_t)e.chunk * e.fw_mat * S, "W");
+  // Blocks, F and W in one allocation.  The nested elimination's fronts take the blocks' place;
+  // at 8 x 8 sites they need more than the float32 blocks and run into F and W, which hold no
+  // zero padding there (one elimination step: the whole block is its pivot block).
+  const size_t mbytes = round_up((size_t)e.chunk * e.mat_stride * S, 1024);
+  const size_t fbytes = round_up((size_t)e.chunk * e.fw_mat * S, 1024);
+  e.block_room = e.N <= e.nb ? mbytes + 2 * fbytes : mbytes;
+  SCA_ALLOC(e.M, mbytes + 2 * fbytes, "blocks, F and W");
+  e.F = static_cast<char*>(e.M) + mbytes;
+  e.W = static_cast<char*>(e.F) + fbytes;
   SCA_ALLOC(e.Tinv, (size_t)e.chunk * 2 * e.nb * e.nb * 2 * S, "Tinv");
   SCA_ALLOC(e.adiag, (size_t)e.chunk * e.N * 2 * sizeof(float), "diagonal table");
   SCA_ALLOC(e.piv, (size_t)e.chunk * e.N * sizeof(int), "piv");
@@ -245,6 +270,7 @@ sca_status allocate(Engine& e) {
   if (e.tc && (st = tc_prepare(e)) != SCA_OK) { release(e); return st; }
 #undef SCA_ALLOC
   if ((st = fused_prepare(e)) != SCA_OK) { release(e); return st; }
+  if ((st = nested_prepare(e)) != SCA_OK) { release(e); return st; }
   if (e.tc && e.piv_blocks > 0) {
     // SMs kept free for the pivoted group (SCA_SM_RESERVE overrides the default)
     int r = e.N > 2048 ? kLargeNSmReserve : kDefaultSmReserve;
@@ -327,7 +353,7 @@ void prof_end(Engine& e, int kind, cudaStream_t s) {
 static const char* const kKindNames[kKinds] = {
     "assemble", "panel", "swap", "trinv", "prep", "update", "refine", "reduce", "diag",
     "update_piv", "fused", "span_pivoted", "span_dominant", "panel_update", "prep_piv",
-    "update_cross"};
+    "update_cross", "nest_up", "nest_down"};
 
 void prof_collect(Engine& e) {
   Profiler* p = e.prof;
@@ -373,6 +399,7 @@ void release(Engine& e) {
   prof_free(e);
   tc_release(e);
   fused_release(e);
+  nested_release(e);
   partition_release(e);
   if (e.ev_join2) cudaEventDestroy(e.ev_join2);
   e.ev_join2 = nullptr;
@@ -384,7 +411,7 @@ void release(Engine& e) {
   if (e.ev_aux1) cudaEventDestroy(e.ev_aux1);
   e.side = e.aux = nullptr;
   e.ev_fork = e.ev_join = e.ev_aux0 = e.ev_aux1 = nullptr;
-  void* ptrs[] = {e.M, e.F, e.W, e.F2, e.W2, e.Tinv, e.tt, e.adiag, e.piv, e.perm, e.flags, e.ld,
+  void* ptrs[] = {e.M, e.F2, e.W2, e.Tinv, e.tt, e.adiag, e.piv, e.perm, e.flags, e.ld,
                   e.d_z, e.tr, e.gd, e.eps_extra, e.d_phi, e.d_m, e.d_v, e.d_g, e.d_status,
                   e.d_omega};
   for (void* q : ptrs)
@@ -629,6 +656,7 @@ sca_status sca_dos(sca_ctx* c, const double* phi_host, const double* w_host, int
   const double thr = 4.0 * std::fabs(e.p.t) * (1.0 + 1e-3);
   e.piv_blocks = (e.nopiv || eta > thr) ? 0 : e.B;
   e.dos_mode = true;
+  e.dos_eta = eta;
   for (int32_t k0 = 0; k0 < n_w && st == SCA_OK; k0 += half) {
     const int cnt = std::min<int>(half, n_w - k0);
     for (int n = 0; n < half; ++n) {  // a short last batch repeats its last frequency
@@ -904,6 +932,7 @@ sca_status sca_set_pivoting(sca_ctx* c, int32_t mode) {
   }
   c->e.piv_blocks = (mode == SCA_PIVOT_NONE) ? 0 : c->e.piv_planned;
   c->e.nopiv = (mode == SCA_PIVOT_NONE);
+  c->e.dense_only = mode == SCA_PIVOT_PARTIAL || dense_switch_set();
   return SCA_OK;
 }
 
@@ -915,6 +944,7 @@ sca_status sca_set_panel_precision(sca_ctx* c, int32_t prec) {
     return SCA_EINVAL;
   }
   c->e.panel_fp64 = !c->e.fp64 && prec == SCA_PREC_FP64;
+  if (c->e.panel_fp64) c->e.dense_only = true;
   return SCA_OK;
 }
 
@@ -956,6 +986,7 @@ sca_status sca_profile_enable(sca_ctx* c, int32_t enable) {
   cudaStreamSynchronize(c->stream);
   prof_collect(c->e);
   c->e.prof->on = enable != 0;
+  c->e.prof->dense = enable != 2;
   for (int k = 0; k < kKinds; ++k) { c->e.prof->ms[k] = 0.0; c->e.prof->n[k] = 0; }
   return SCA_OK;
 }

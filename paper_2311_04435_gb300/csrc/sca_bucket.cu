@@ -130,6 +130,7 @@ sca_status bucket_req_init(Bucket* b, BucketReq* r, const sca_params& p, const s
   r->step = 0;
   r->nb = 2 * p.n_omega;
   r->npiv = pivoted_count(p);
+  r->nested = nested_rule(p.t, M_PI * p.T, (2.0 * p.n_omega - 1.0) * M_PI * p.T);
   r->delta_eff = (p.ionic == SCA_IONIC_HALF) ? 0.5 * p.delta : p.delta;
   cudaError_t err = cudaMalloc((void**)&r->d, sizeof(double) * (4 * (size_t)N + 8));
   if (err != cudaSuccess) { r->d = nullptr; return cuda_fail(err, "request state"); }
@@ -146,7 +147,7 @@ void bucket_req_release(BucketReq* r) {
   r->d = nullptr;
 }
 
-sca_status bucket_run(Bucket* b, BucketReq* const* reqs, int n, int nsteps, bool adam) {
+sca_status bucket_run(Bucket* b, BucketReq* const* requests, int n, int nsteps, bool adam) {
   NvtxRange range("sca.bucket_run");
   Engine& e = b->ctx->e;
   cudaStream_t s = b->ctx->stream;
@@ -155,6 +156,10 @@ sca_status bucket_run(Bucket* b, BucketReq* const* reqs, int n, int nsteps, bool
   // the staging buffers of the previous call are free once its copies have run
   cudaError_t err = cudaStreamSynchronize(s);
   if (err != cudaSuccess) return cuda_fail(err, "bucket run");
+  // A request takes the elimination it takes alone (nested where its frequencies admit it), so
+  // the passes are formed of one kind each.
+  std::vector<BucketReq*> reqs(requests, requests + n);
+  std::stable_partition(reqs.begin(), reqs.end(), [](const BucketReq* r) { return r->nested; });
   // passes: requests in order while their blocks fit the slots
   std::vector<int> first, count;
   for (int i = 0, used = 0; i < n; ++i) {
@@ -162,7 +167,8 @@ sca_status bucket_run(Bucket* b, BucketReq* const* reqs, int n, int nsteps, bool
       set_error("request has more blocks than its size bucket");
       return SCA_EINVAL;
     }
-    if (first.empty() || used + reqs[i]->nb > b->cap || count.back() == b->rmax) {
+    if (first.empty() || used + reqs[i]->nb > b->cap || count.back() == b->rmax ||
+        reqs[i]->nested != reqs[i - 1]->nested) {
       first.push_back(i);
       count.push_back(0);
       used = 0;
@@ -236,6 +242,7 @@ sca_status bucket_run(Bucket* b, BucketReq* const* reqs, int n, int nsteps, bool
     for (int p = 0; p < P && st == SCA_OK; ++p) {
       e.B = ntot[p];
       e.piv_blocks = npiv[p];
+      e.nest_rule = reqs[first[p]]->nested;
       e.bd = b->d_bd + (size_t)p * b->cap;
       st = run_blocks(e, reqs[first[p]]->d, true, s);
       if (st == SCA_OK)

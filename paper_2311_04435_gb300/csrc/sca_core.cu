@@ -3216,6 +3216,9 @@ sca_status run_blocks(Engine& e, const double* d_phi, bool want_grad, cudaStream
                       bool refine_stage) {
   NvtxRange range(want_grad ? "sca.blocks(inverse)" : "sca.blocks(log-det)");
   sca_status st;
+  e.fronts_kept = nested_now(e);
+  if (e.fronts_kept)
+    return run_nested(e, make_lattice(e, d_phi), true, want_grad && (refine_stage || e.dos_mode), s);
   if (e.fp64) {
     if ((st = set_smem_limits<double, double>()) != SCA_OK) return st;
     return run_blocks_t<double, double>(e, d_phi, want_grad, refine_stage, s);
@@ -3230,6 +3233,7 @@ sca_status run_refine_resident(Engine& e, const double* d_phi, cudaStream_t s) {
     return SCA_ENOSTATE;
   }
   const Lattice la = make_lattice(e, d_phi);
+  if (e.fronts_kept) return run_nested(e, la, false, true, s);
   if (e.fp64) return launch_refine<double>(e, la, 0, 0, e.B, s);
   return launch_refine<float>(e, la, 0, 0, e.B, s);
 }

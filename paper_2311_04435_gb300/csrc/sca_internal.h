@@ -65,6 +65,8 @@ struct AdamStep {
 };
 
 struct BlockDesc;  // per-slot physics (sca_device.cuh)
+struct Lattice;
+struct Nested;     // the nested elimination's tables and launch plan (sca_nested.cu)
 
 // One request of a shared pass (size-bucket batching): its device state and blocks.
 struct ReqDesc {
@@ -99,6 +101,7 @@ struct Engine {
   size_t plane_stride = 0, mat_stride = 0;  // elements
   size_t fw_plane = 0, fw_mat = 0;          // F / W panel strides (elements)
 
+  size_t block_room = 0;    // bytes from M on that the nested elimination's fronts may use
   void* M = nullptr;        // chunk blocks
   void* F = nullptr;        // chunk x 2 planes x N x nb (x2 hi/lo for tc)
   void* W = nullptr;        // same, W^T
@@ -128,6 +131,14 @@ struct Engine {
   double* d_status = nullptr;   // 8 doubles
   double* d_omega = nullptr;    // 1 double scratch
   double* h_status = nullptr;   // pinned 8 doubles
+  // nested elimination (sca_nested.cu): its fronts use M.  nest_rule: the smallest omega_n
+  // admits it; dense_only: the caller or an environment switch chose the dense elimination's
+  // options; fronts_kept: the last pass left fronts (not dense inverses) in M.
+  Nested* nest = nullptr;
+  bool nest_rule = false;
+  bool dense_only = false;
+  bool fronts_kept = false;
+  double dos_eta = 0.0;
   void* tmap = nullptr;         // host-side tensor-map storage (tc path)
   size_t bytes = 0;
   struct Profiler* prof = nullptr;  // per-kernel event timing (sca_profile_enable)
@@ -176,12 +187,15 @@ enum KernelKind {
   kPanelUpd,   // pivoted group: update of the rest of the outer panel after a sub-panel
   kPrepPiv,    // pivoted group: rank-nb factors
   kUpdateCross,  // merged two-step update: the first step's update of the second step's strips
+  kNestUp,     // nested elimination, one level of fronts
+  kNestDown,   // nested elimination, one level of diag(G)
   kKinds
 };
 
 // Event bracketing of launches while profiling is on (no-ops otherwise).
 struct Profiler {
   bool on = false;
+  bool dense = false;  // time the dense elimination's kernels (evaluations take that path)
   double ms[kKinds] = {};
   uint64_t n[kKinds] = {};
   struct Rec { int kind; cudaEvent_t a, b; cudaStream_t s; };
@@ -221,6 +235,21 @@ sca_status run_refine_resident(Engine& e, const double* d_phi, cudaStream_t s);
 
 sca_status run_reduce(Engine& e, const double* d_phi, double* d_omega, double* d_grad,
                       const AdamStep* adam, cudaStream_t s);
+
+// Nested elimination (sca_nested.cu).  Its rounding errors can grow by powers of |t| / Im z, so
+// contexts whose smallest omega_n, and densities of states whose eta, lie below
+// kNestedMinImag |t| take the pivoted dense elimination.  Where the line lies: in float64 on
+// 100..400 sites with disorder, gradients are as close to the exact ones as the dense path's down
+// to T = 0.01 (omega_0 = 0.031), densities of states down to eta = 0.02 (8.2e-14 against 7.9e-14);
+// at eta = 0.01 the nested error is 1.7 times the dense one (1.8e-13 against 1.1e-13).  The other
+// limits keep double-float squares inside float32's range.
+constexpr double kNestedMinImag = 0.03;
+bool nested_rule(double t, double imag_min, double imag_max);
+sca_status nested_prepare(Engine& e);  // tables (leaves e.nest null where it does not apply)
+void nested_release(Engine& e);
+bool nested_now(const Engine& e);      // whether the next evaluation takes it
+// up: eliminate (ld); down: diag(G) from the fronts left in M by a preceding `up`.
+sca_status run_nested(Engine& e, const Lattice& la, bool up, bool down, cudaStream_t s);
 
 // Assembled blocks (for sca_debug_assemble).
 sca_status run_assemble_only(Engine& e, const double* d_phi, int b0, int count, cudaStream_t s);
@@ -275,6 +304,7 @@ struct BucketReq {
   sca_adam a{};
   int32_t step = 0;
   int nb = 0, npiv = 0;
+  bool nested = false;  // its frequencies admit the nested elimination
   double delta_eff = 0.0;
   double* d = nullptr;
 };
