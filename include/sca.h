@@ -402,8 +402,8 @@ sca_status sca_sm_partition(sca_ctx* ctx, int32_t* pivoted_sms, int32_t* dominan
  * kernels above, so they are not part of any sum), 13 update of the rest of a pivoted outer
  * panel after each sub-panel, 14 rank-nb factors of the pivoted group, 15 the first update of a
  * merged pair of elimination steps of the dominant blocks (only the second step's row and column
- * strips; the merged update of the rest is kind 5), 16 and 17 one tree level of the nested
- * elimination and of its diag(G).  enable = 1 times the dense elimination, which the context then
+ * strips; the merged update of the rest is kind 5), 16 the nested elimination (with its diag(G) where one
+ * launch does both), 17 its diag(G) from resident fronts.  enable = 1 times the dense elimination, which the context then
  * takes (kinds 0 to 15 are its kernels); enable = 2 times whatever the context takes without
  * profiling.  Enabling resets the counters.  Timing adds a small host overhead per launch; keep it off when measuring
  * throughput.  With the environment variable SCA_PROFILE_TRACE set to a file name, each

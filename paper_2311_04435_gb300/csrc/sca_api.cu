@@ -154,6 +154,7 @@ sca_status plan(const sca_params& p, Engine& e) {
   const double thr = 4.0 * std::fabs(p.t) * (1.0 + 1e-3);
   while (n_piv < p.n_omega && (2.0 * n_piv + 1.0) * M_PI * p.T <= thr) ++n_piv;
   e.piv_blocks = 2 * n_piv;
+  e.nest_dense = e.piv_blocks;
   if (const char* v = std::getenv("SCA_PIVOT_ALL"))
     if (std::atoi(v) != 0) e.piv_blocks = e.B;
   e.piv_planned = e.piv_blocks;
@@ -657,6 +658,8 @@ sca_status sca_dos(sca_ctx* c, const double* phi_host, const double* w_host, int
   e.piv_blocks = (e.nopiv || eta > thr) ? 0 : e.B;
   e.dos_mode = true;
   e.dos_eta = eta;
+  const int dense_saved = e.nest_dense;
+  e.nest_dense = eta > thr ? 0 : e.B;
   for (int32_t k0 = 0; k0 < n_w && st == SCA_OK; k0 += half) {
     const int cnt = std::min<int>(half, n_w - k0);
     for (int n = 0; n < half; ++n) {  // a short last batch repeats its last frequency
@@ -685,6 +688,7 @@ sca_status sca_dos(sca_ctx* c, const double* phi_host, const double* w_host, int
     }
   }
   e.dos_mode = false;
+  e.nest_dense = dense_saved;
   e.piv_blocks = saved;
   return st;
 }

@@ -237,11 +237,12 @@ sca_status bucket_run(Bucket* b, BucketReq* const* requests, int n, int nsteps, 
   err = cudaMemcpyAsync(b->d_req, b->h_req, sizeof(ReqDesc) * (size_t)P * b->steps * b->rmax,
                         cudaMemcpyHostToDevice, s);
   if (err != cudaSuccess) return cuda_fail(err, "bucket tables upload");
-  const int B0 = e.B, piv0 = e.piv_blocks;
+  const int B0 = e.B, piv0 = e.piv_blocks, dense0 = e.nest_dense;
   for (int sidx = 0; sidx < nsteps && st == SCA_OK; ++sidx)
     for (int p = 0; p < P && st == SCA_OK; ++p) {
       e.B = ntot[p];
       e.piv_blocks = npiv[p];
+      e.nest_dense = npiv[p];
       e.nest_rule = reqs[first[p]]->nested;
       e.bd = b->d_bd + (size_t)p * b->cap;
       st = run_blocks(e, reqs[first[p]]->d, true, s);
@@ -250,6 +251,7 @@ sca_status bucket_run(Bucket* b, BucketReq* const* requests, int n, int nsteps, 
     }
   e.B = B0;
   e.piv_blocks = piv0;
+  e.nest_dense = dense0;
   e.bd = nullptr;
   if (st != SCA_OK) return st;
   if (adam)

@@ -136,6 +136,7 @@ struct Engine {
   // options; fronts_kept: the last pass left fronts (not dense inverses) in M.
   Nested* nest = nullptr;
   bool nest_rule = false;
+  int nest_dense = 0;       // leading blocks without column dominance (dense leaves)
   bool dense_only = false;
   bool fronts_kept = false;
   double dos_eta = 0.0;

@@ -16,22 +16,34 @@
 // No pivot is searched for: -i A has the Hermitian part (Im z) I with Im z = w_n > 0 (eta for a
 // density of states), and so has every Schur complement and every leading block of one; each
 // pivot is at least Im z in modulus.  Rounding errors grow by powers of |t| / Im z, which is why
-// callers with Im z below kMinImag |t| take the pivoted dense elimination (nested_rule).
+// callers with Im z below kNestedMinImag |t| take the pivoted dense elimination (nested_rule).
 //
 // Arithmetic: float64, or on the reduced-precision paths double-float (an unevaluated sum of two
 // float32, 48 bits): products exact by FMA, sums by two-sums, 12 float32 instructions per real
 // multiply-add.  This GPU does 64 float32 FMAs in the time of one float64 FMA, so double-float is
 // 5 times as fast as float64 and keeps 24 bits more than the float32 blocks of the dense paths.
 //
-// Work split: one CTA per (node, block), one launch per tree level and direction, fronts in
-// global memory (a block's fronts take 3.2 MB at N = 1600), the current panel of at most 20 pivot
-// rows and its X in shared memory.  Both number types are bound by their arithmetic: a panel of w
-// rows does w / 2 multiply-adds per front entry that it reads and writes.
+// Work split: a group of threads per front (a warp for the smallest, 256 or 512 threads for the
+// largest), fronts in global memory (a block's take 3.2 MB at N = 1600), the current panel of at
+// most 20 pivot rows and its X in shared memory.  Up to one block per SM the whole elimination is
+// one launch, a CTA of 512 threads per block or a cluster of them, with a barrier per tree level;
+// more blocks take one launch per level and direction, spread over the chip, and the blocks with
+// dense leaves run beside the others on a second stream.  Microseconds per gradient, one launch
+// against one per level: 16x16 with 64 blocks 176 / 254, 24x24 with 128 578 / 687, 32x32 with 128
+// 1100 / 1217, 64x64 with 128 7850 / 8281; 20x20 with 512 blocks 1313 / 1150, float64 2892 / 2429,
+// 40x40 with 256 5766 / 3570.  An entry's arithmetic is the same in every split: results do not
+// depend on it.
+//
+// What bounds it: float64, the float64 pipe (80 % active at 20x20: 2.1 times the instructions that
+// the products alone need, for lanes that idle at the edges of small fronts); double-float, issue
+// (IPC 2.1 of 4 with 16 warps per SM) and the dependent chain of a panel's pivots, some 1800
+// cycles per pivot, which other fronts' products overlap only in part.
 #include <cuda_runtime.h>
 
 #include <algorithm>
 #include <cmath>
 #include <new>
+#include <type_traits>
 #include <vector>
 
 #include "sca_device.cuh"
@@ -74,6 +86,8 @@ __device__ __forceinline__ void zset(Zf& z, double re, double im) {
   const dsf a = ds_of(re), b = ds_of(im);
   z = {a.h, a.l, b.h, b.l};
 }
+__device__ __forceinline__ void zset0(Zd& z) { z = {0.0, 0.0}; }
+__device__ __forceinline__ void zset0(Zf& z) { z = {0.f, 0.f, 0.f, 0.f}; }
 __device__ __forceinline__ double zre(Zd z) { return z.re; }
 __device__ __forceinline__ double zim(Zd z) { return z.im; }
 __device__ __forceinline__ double zre(Zf z) { return (double)z.rh + (double)z.rl; }
@@ -84,6 +98,20 @@ __device__ __forceinline__ Zd zadd(Zd a, Zd b) { return {a.re + b.re, a.im + b.i
 __device__ __forceinline__ Zf zadd(Zf a, Zf b) {
   const dsf r = ds_add({a.rh, a.rl}, {b.rh, b.rl}), i = ds_add({a.ih, a.il}, {b.ih, b.il});
   return {r.h, r.l, i.h, i.l};
+}
+
+__device__ __forceinline__ Zd zsel(bool c, Zd a, Zd b) {
+  return {c ? a.re : b.re, c ? a.im : b.im};
+}
+__device__ __forceinline__ Zf zsel(bool c, Zf a, Zf b) {
+  return {c ? a.rh : b.rh, c ? a.rl : b.rl, c ? a.ih : b.ih, c ? a.il : b.il};
+}
+__device__ __forceinline__ Zd zshfl_xor(Zd z, int off) {
+  return {__shfl_xor_sync(0xffffffffu, z.re, off), __shfl_xor_sync(0xffffffffu, z.im, off)};
+}
+__device__ __forceinline__ Zf zshfl_xor(Zf z, int off) {
+  return {__shfl_xor_sync(0xffffffffu, z.rh, off), __shfl_xor_sync(0xffffffffu, z.rl, off),
+          __shfl_xor_sync(0xffffffffu, z.ih, off), __shfl_xor_sync(0xffffffffu, z.il, off)};
 }
 
 __device__ __forceinline__ void acc_of(Ad& a, Zd z) { a = {z.re, z.im}; }
@@ -125,16 +153,28 @@ __device__ __forceinline__ Z zmul(Z a, Z b) {
   mac(s, a, b);
   return acc_get(s);
 }
-__device__ __forceinline__ Zd zinv(Zd z) {
-  const double d = 1.0 / (z.re * z.re + z.im * z.im);
+// 1 / z, and |z|^2 in float64.
+__device__ __forceinline__ Zd zinv(Zd z, double* mag2 = nullptr) {
+  const double m = z.re * z.re + z.im * z.im;
+  const float mf = (float)m;
+  double d;
+  if (mf > 1e-37f && mf < 1e37f) {  // float32 reciprocal and two Newton steps: 6 float64
+    d = (double)__frcp_rn(mf);      // instructions where a division takes some 15
+    d = fma(d, fma(-m, d, 1.0), d);
+    d = fma(d, fma(-m, d, 1.0), d);
+  } else {
+    d = 1.0 / m;
+  }
+  if (mag2) *mag2 = m;
   return {z.re * d, -z.im * d};
 }
-__device__ __forceinline__ Zf zinv(Zf z) {
+__device__ __forceinline__ Zf zinv(Zf z, double* mag2 = nullptr) {
   float s = 0.f, c = 0.f;
   mac1(s, c, z.rh, z.rl, z.rh, z.rl);
   mac1(s, c, z.ih, z.il, z.ih, z.il);
   const dsf d = two_sum(s, c);
-  const float q = 1.0f / d.h;  // then one Newton step: q + q (1 - d q)
+  if (mag2) *mag2 = (double)d.h + (double)d.l;
+  const float q = __frcp_rn(d.h);  // then one Newton step: q + q (1 - d q)
   float e = fmaf(-q, d.h, 1.0f);
   e = fmaf(-q, d.l, e);
   const float ql = __fmul_rn(q, e);
@@ -145,386 +185,657 @@ __device__ __forceinline__ Zf zinv(Zf z) {
   return {r.h, r.l, i.h, i.l};
 }
 
+// A product of moduli squared as mantissa in [1, 2) and exponent: a node's share of |det A|^2.
+// One logarithm per node at the root instead of one per pivot (a float64 logarithm costs about
+// 40 instructions of the slowest pipe of this GPU).
+struct alignas(16) Det {
+  double mant;
+  int exp, pad;
+};
+__device__ __forceinline__ void det_norm(double& m, int& e) {
+  if (m < 0x1p-1000) {  // subnormal range
+    m *= 0x1p200;
+    e -= 200;
+  }
+  const int hi = __double2hiint(m);
+  e += ((hi >> 20) & 0x7ff) - 1023;
+  m = __hiloint2double((hi & 0x800fffff) | 0x3ff00000, __double2loint(m));
+}
+// Product over the warp's lanes of m2 (1.0 where a lane has none), in a fixed order, times
+// (mant, exp); flags non-positive or non-finite moduli.
+__device__ __forceinline__ void det_mul(double m2, double& mant, int& exp, int* flags) {
+  if (!(m2 > 0.0 && isfinite(m2))) {
+    atomicOr(flags, 1);
+    m2 = 1.0;
+  }
+  int e = 0;
+  det_norm(m2, e);
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+    m2 *= __shfl_xor_sync(0xffffffffu, m2, off);
+    e += __shfl_xor_sync(0xffffffffu, e, off);
+  }
+  mant *= m2;
+  exp += e;
+  det_norm(mant, exp);
+}
+
 // ------------------------------------------------------------------ kernels
+constexpr int kRows = nested::kRows;    // rows of a thread's output tile at most
+constexpr int kSlots = nested::kSlots;  // entries of a pivots' block that a thread holds at most
+
+// How one level's fronts are worked on: `group` threads per front, each group with `smem` bytes.
+struct LevelPlan {
+  int first, count, group, smem;
+};
+
 template <typename Z>
 struct NestArgs {
   const Node* nodes;     // the two forms of the tree, nnodes each: closed-form, dense leaves
   const int16_t* tab;
   Z* fronts;             // fronts of the pass's blocks, `stride` entries apart
   long long stride;
-  double* ldp;           // [block of the pass][node]: the node's share of ln|det A|
-  int nnodes;
+  Det* det;              // [block of the pass][node]: the node's share of |det A|^2
+  int nnodes, nlevels;
   int b0;                // block of the pass's first slot
+  int csize;             // CTAs per block
+  int ndense;            // leading slots of the pass that take the dense leaves
+  int k0, k1;            // phases: [0, nlevels) up from the leaves, [nlevels, 2 nlevels) down
   Lattice la;
   double* ld;            // ln|det A_b|
   double* gd;            // [b][site]: sigma Re G_ii (or Im G_ii where zshift is set)
   int* flags;
+  LevelPlan lv[2][nested::kMaxLevels];  // by form; root first
 };
 
-// The nodes of the form that a block with shift imaginary part zi takes: dense leaves unless its
-// columns are diagonally dominant (the line of the dense elimination's pivoted group).
-template <typename Z>
-__device__ __forceinline__ const Node* tree_of(const NestArgs<Z>& a, double t, double zi) {
-  return a.nodes + (zi > 4.0 * fabs(t) * (1.0 + 1e-3) ? 0 : a.nnodes);
-}
-
+// Whether two sites, packed as 256 x + y, are neighbours.
 __device__ __forceinline__ bool adjacent(int L, int a, int b) {
-  const int dx = abs(a / L - b / L), dy = abs(a % L - b % L);
+  const int dx = abs((a >> 8) - (b >> 8)), dy = abs((a & 255) - (b & 255));
   return (dx == 0 && (dy == 1 || dy == L - 1)) || (dy == 0 && (dx == 1 || dx == L - 1));
 }
 
 // Entry (hi, lo) of a front before its own elimination, hi >= lo: A's entry where lo is a pivot
 // (entries between boundary sites belong to an ancestor), the children's Schur complements, and
-// in a leaf the closed-form elimination of the blacks next to both sites (bt = t^2 / a_b).
+// in a leaf the closed-form elimination of the blacks next to both sites (bt = -t^2 / a_b).
 template <typename Z>
 struct Front {
   int L;
-  double t;
   const Z* c[2];        // children's Schur complements (their boundary parts), row stride cm
   int cm[2];
   int p, leaf;
-  const int16_t *site, *cmap0, *cmap1, *adj;
-  const Z* bt;
-  const Z* diag;        // A_ii of the pivots
+  int site, cmap0, cmap1, adj;  // shared-memory offsets of the index maps,
+  int bt, diag;                 // of the blacks' terms, of A_ii of the pivots followed by t
   __device__ __forceinline__ Z at(int hi, int lo) const {
+    extern __shared__ __align__(16) unsigned char smem[];
+    auto tab = [&](int o, int i) { return (int)reinterpret_cast<const int16_t*>(smem + o)[i]; };
     Z v;
-    zset(v, 0.0, 0.0);
+    zset0(v);
     if (leaf) {
-      for (int x = 0; x < 4; ++x) {
-        const int b = adj[4 * hi + x];
-        if (b < 0) break;
-#pragma unroll
-        for (int y = 0; y < 4; ++y)
-          if (adj[4 * lo + y] == b) v = zadd(v, zneg(bt[b]));
-      }
-    } else {
-      if (c[0]) {
-        const int i = cmap0[hi], j = cmap0[lo];
-        if (i >= 0 && j >= 0) v = c[0][(size_t)i * cm[0] + j];
-      }
-      if (c[1]) {
-        const int i = cmap1[hi], j = cmap1[lo];
-        if (i >= 0 && j >= 0) v = zadd(v, c[1][(size_t)i * cm[1] + j]);
-      }
+      for (int both = tab(adj, hi) & tab(adj, lo); both; both &= both - 1)
+        v = zadd(v, reinterpret_cast<const Z*>(smem + bt)[__ffs(both) - 1]);
+    } else if (c[0]) {  // (a node with children has two)
+      const int i = tab(cmap0, hi), j = tab(cmap0, lo), k = tab(cmap1, hi), l = tab(cmap1, lo);
+      Z x;
+      zset0(x);
+      const Z *c0 = c[0], *c1 = c[1];
+      __builtin_assume(__isGlobal(c0));
+      __builtin_assume(__isGlobal(c1));
+      if (i >= 0 && j >= 0) v = c0[i * cm[0] + j];
+      if (k >= 0 && l >= 0) x = c1[k * cm[1] + l];
+      v = zadd(v, x);
     }
     if (lo < p) {
-      if (hi == lo) {
-        v = zadd(v, diag[lo]);
-      } else if (adjacent(L, site[hi], site[lo])) {
-        Z b;
-        zset(b, t, 0.0);
-        v = zadd(v, b);
-      }
+      if (hi == lo)
+        v = zadd(v, reinterpret_cast<const Z*>(smem + diag)[lo]);
+      else if (adjacent(L, tab(site, hi), tab(site, lo)))
+        v = zadd(v, reinterpret_cast<const Z*>(smem + diag)[p]);
     }
     return v;
   }
 };
 
-// One node of one block, up: see the file comment.  Shared memory: the panel's rows A (w x the
-// rest of the front), X, the leaf's blacks, the pivots' diagonal and the index maps.
-template <typename Z, int NT>
-__global__ void __launch_bounds__(NT) k_nest_up(NestArgs<Z> a, int first) {
+// Row and column of entry e of a lower triangle stored row after row.
+__device__ __forceinline__ void triangle(int e, int& i, int& j) {
+  i = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);
+  if ((i + 1) * (i + 2) / 2 <= e) ++i;
+  if (i * (i + 1) / 2 > e) --i;
+  j = e - i * (i + 1) / 2;
+}
+
+// Block of KR rows and column of task e where row block b has KR (b + 1) columns.
+template <int KR>
+__device__ __forceinline__ void row_block(int e, int& b, int& j) {
+  b = (int)((sqrtf((8.0f / KR) * (float)e + 1.0f) - 1.0f) * 0.5f);
+  if (KR * (b + 1) * (b + 2) / 2 <= e) ++b;
+  if (KR * b * (b + 1) / 2 > e) --b;
+  j = e - KR * b * (b + 1) / 2;
+}
+
+// The threads that work on one front: `size` of them (a power of two, a whole warp at least) with
+// a barrier of their own.
+struct Group {
+  int size, tid, bar;
+  __device__ __forceinline__ void sync() const {
+    if (size == 32)
+      __syncwarp();
+    else
+      asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(size) : "memory");
+  }
+};
+
+// Offset of a pointer into the CTA's dynamic shared memory.
+__device__ __forceinline__ int off(const void* p) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  return (int)(static_cast<const unsigned char*>(p) - smem);
+}
+
+// What the fronts of one block share.
+template <typename Z>
+struct Block {
+  const Node* nodes;
+  const int16_t* tab;
+  Z* fronts;
+  Det* det;
+  double* gd;
+  int* flags;
+  Lattice la;
+  double zr, zi;
+  int sg;
+};
+
+// The functions below are calls of their own, with offsets into shared memory instead of pointers:
+// inlined into one kernel they spill, and through a call a pointer would lose its address space.
+// Their inner loops have no branch per row, which would split them into blocks of two dependent
+// chains each; rows past the end repeat the last one and are dropped.
+
+// -F11^{-1} by w Gauss-Jordan steps, diagonal pivots in order: thread (g, j) holds the entries
+// (g, j), (g + G, j), ... of the w x w block, S of them, G = size / w.  A step needs the pivot's
+// row, its column and its reciprocal; their owners write them to shared memory as soon as they
+// have them (two buffers, one barrier per step).  The result replaces F11, negated, and goes to
+// the front.
+template <typename Z, int S>
+__device__ __noinline__ void invert(const Group gr, int w, int F11o, int rowo, int colo,
+                                    int mago, Z* Fo, int m) {
+  using Acc = typename AccOf<Z>::type;
+  extern __shared__ __align__(16) unsigned char smem[];
+  Z* F11 = reinterpret_cast<Z*>(smem + F11o);
+  Z* rowb = reinterpret_cast<Z*>(smem + rowo);
+  Z* colb = reinterpret_cast<Z*>(smem + colo);
+  double* mag = reinterpret_cast<double*>(smem + mago);
+  __builtin_assume(__isGlobal(Fo));
+  const int G = min(w, gr.size / w), g = gr.tid / w, j = gr.tid - g * w;
+  const bool on = g < G;
+  Z reg[S];
+  int row[S];
+#pragma unroll
+  for (int s = 0; s < S; ++s) row[s] = min(g + s * G, w - 1);
+  if (on) {
+#pragma unroll
+    for (int s = 0; s < S; ++s) reg[s] = F11[row[s] * w + j];
+    if (g == 0) rowb[j] = reg[0];
+    if (j == 0) {
+#pragma unroll
+      for (int s = 0; s < S; ++s) colb[row[s]] = zneg(reg[s]);
+    }
+    if (gr.tid == 0) colb[w] = zinv(reg[0], mag);
+  }
+#pragma unroll 1
+  for (int c = 0; c < w; ++c) {
+    gr.sync();
+    const Z* rb = rowb + (c & 1) * w;
+    const Z* cb = colb + (c & 1) * (w + 1);
+    Z* rn = rowb + ((c + 1) & 1) * w;
+    Z* cn = colb + ((c + 1) & 1) * (w + 1);
+    if (on) {
+      const bool own = j == c;
+      const Z dinv = cb[w];
+      const Z u = zsel(own, dinv, zmul(rb[j], dinv));
+      Z zero;
+      zset0(zero);
+#pragma unroll
+      for (int s = 0; s < S; ++s) {
+        Acc x;
+        acc_of(x, zsel(own, zero, reg[s]));
+        mac(x, cb[row[s]], u);
+        reg[s] = zsel(row[s] == c, u, acc_get(x));
+      }
+      if (c + 1 < w && g == (c + 1) % G) {  // the next pivot's row
+        Z nr = reg[0];
+#pragma unroll
+        for (int s = 1; s < S; ++s) nr = zsel(row[s] == c + 1, reg[s], nr);
+        rn[j] = nr;
+        if (j == c + 1) cn[w] = zinv(nr, mag + j);
+      }
+      if (j == c + 1) {
+#pragma unroll
+        for (int s = 0; s < S; ++s) cn[row[s]] = zneg(reg[s]);
+      }
+    }
+  }
+  if (on) {
+#pragma unroll
+    for (int s = 0; s < S; ++s) {
+      F11[row[s] * w + j] = zneg(reg[s]);
+      Fo[(size_t)row[s] * m + j] = reg[s];
+    }
+  }
+}
+
+// Lower triangle of the rest, F22 - F12^T X: each thread one column and KR rows.  Neighbouring lanes
+// take neighbouring columns, so the front's rows, X and the children's rows are read and written
+// along them, and F12 is broadcast.
+template <typename Z, int KR>
+__device__ __noinline__ void update_rest(const Group gr, const Front<Z>& f, bool first, int at0,
+                                            int w, int r, int m, int Ao, int lda, int Xo, Z* R) {
+  using Acc = typename AccOf<Z>::type;
+  extern __shared__ __align__(16) unsigned char smem[];
+  const Z* A = reinterpret_cast<const Z*>(smem + Ao);
+  const Z* X = reinterpret_cast<const Z*>(smem + Xo);
+  __builtin_assume(__isGlobal(R));
+  const int nb = (r + KR - 1) / KR, tasks = KR * nb * (nb + 1) / 2;
+  for (int e = gr.tid; e < tasks; e += gr.size) {
+    int b, j;
+    row_block<KR>(e, b, j);
+    if (j >= r) continue;
+    const int i0 = b * KR;
+    Acc s[KR];
+#pragma unroll
+    for (int u = 0; u < KR; ++u) s[u] = Acc{};
+    const Z *Ai = A + i0, *Xj = X + j;
+#pragma unroll 2
+    for (int k = 0; k < w; ++k) {
+      const Z x = *Xj;
+#pragma unroll
+      for (int u = 0; u < KR; ++u) mac(s[u], Ai[u], x);
+      Ai += lda;
+      Xj += r;
+    }
+    Z v[KR];
+    if (!first) {
+#pragma unroll
+      for (int u = 0; u < KR; ++u) v[u] = R[max(j, min(i0 + u, r - 1)) * m + j];
+    } else {
+#pragma unroll
+      for (int u = 0; u < KR; ++u) v[u] = f.at(at0 + max(j, min(i0 + u, r - 1)), at0 + j);
+    }
+#pragma unroll
+    for (int u = 0; u < KR; ++u) {
+      const int i = i0 + u;
+      if (i < r && j <= i) R[i * m + j] = zadd(v[u], acc_get(s[u]));
+    }
+  }
+}
+
+// Y = X R (w x r, inner length n): one column and KR rows per thread, the rows nrb apart, X (row
+// stride ldx) broadcast from shared memory, R (row stride step) from shared or global memory (L1
+// and L2 hold it).  kGlobal: R is Rg, in global memory; else at Ro, and the rows of Y go to Yg (row
+// stride m) too.  kMap: R's rows and columns go through map (R in the parent's front).
+template <typename Z, int KR, bool kMap, bool kGlobal>
+__device__ __noinline__ void times(const Group gr, int w, int n, int r, int Xo, int ldx, int Yo,
+                                   int ldy, const Z* Rg, int Ro, int step, int mapo, Z* Yg, int m) {
+  using Acc = typename AccOf<Z>::type;
+  extern __shared__ __align__(16) unsigned char smem[];
+  const Z* X = reinterpret_cast<const Z*>(smem + Xo);
+  Z* Y = reinterpret_cast<Z*>(smem + Yo);
+  const Z* Rs = reinterpret_cast<const Z*>(smem + Ro);
+  const int16_t* map = reinterpret_cast<const int16_t*>(smem + mapo);
+  __builtin_assume(__isGlobal(Rg));
+  const int nrb = (w + KR - 1) / KR;
+  for (int e = gr.tid; e < nrb * r; e += gr.size) {
+    const int b = e / r, j = e - b * r;
+    Acc s[KR];
+    int Xi[KR];
+#pragma unroll
+    for (int u = 0; u < KR; ++u) {
+      s[u] = Acc{};
+      Xi[u] = min(b + u * nrb, w - 1) * ldx;
+    }
+    const int jj = kMap ? map[j] : j;
+    if constexpr (kGlobal) {  // two rows ahead
+      auto load = [&](int k) {
+        k = min(k, n - 1);
+        return Rg[(kMap ? map[k] : k) * step + jj];
+      };
+      Z g0 = load(0), g1 = load(1);
+#pragma unroll 1
+      for (int k = 0; k + 1 < n; k += 2) {
+        Z g = g0;
+        g0 = load(k + 2);
+#pragma unroll
+        for (int u = 0; u < KR; ++u) mac(s[u], X[Xi[u] + k], g);
+        g = g1;
+        g1 = load(k + 3);
+#pragma unroll
+        for (int u = 0; u < KR; ++u) mac(s[u], X[Xi[u] + k + 1], g);
+      }
+      if (n & 1) {
+#pragma unroll
+        for (int u = 0; u < KR; ++u) mac(s[u], X[Xi[u] + n - 1], g0);
+      }
+    } else {
+#pragma unroll 2
+      for (int k = 0; k < n; ++k) {
+        const Z g = Rs[k * step + jj];
+#pragma unroll
+        for (int u = 0; u < KR; ++u) mac(s[u], X[Xi[u] + k], g);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < KR; ++u) {
+      const int i = b + u * nrb;
+      if (i < w) {
+        const Z v = acc_get(s[u]);
+        Y[i * ldy + j] = v;
+        if (!kGlobal) Yg[i * m + j] = v;
+      }
+    }
+  }
+}
+
+// The row count that fits the outputs per thread: passes over the threads, each of KR products and
+// about a third of a product's overhead.
+template <typename Z, bool kMap, bool kGlobal>
+__device__ __forceinline__ void times_fit(const Group& gr, int w, int n, int r, int Xo, int ldx,
+                                          int Yo, int ldy, const Z* Rg, int Ro, int step, int mapo,
+                                          Z* Yg, int m) {
+  auto cost = [&](int kr) {
+    return ((w + kr - 1) / kr * r + gr.size - 1) / gr.size * (3 * kr + 1);
+  };
+  if (cost(2) <= cost(1) || kMap)
+    times<Z, 2, kMap, kGlobal>(gr, w, n, r, Xo, ldx, Yo, ldy, Rg, Ro, step, mapo, Yg, m);
+  else
+    times<Z, 1, kMap, kGlobal>(gr, w, n, r, Xo, ldx, Yo, ldy, Rg, Ro, step, mapo, Yg, m);
+}
+
+// One front, up: see the file comment.  -X is kept (in the front and here), as both later products
+// want it with that sign.  Shared memory: F12 and -X (w x r each), F11 (then -P), the inversion's
+// buffers, the leaf's blacks, the pivots' diagonal, index maps.
+template <typename Z>
+__device__ __forceinline__ void front_up(const Block<Z>& B, int node, const Group& gr, int at) {
   extern __shared__ __align__(16) unsigned char smem[];
   using Acc = typename AccOf<Z>::type;
-  constexpr int kEntries = (nested::kPanel * nested::kPanel + NT - 1) / NT;
-  const int mat = blockIdx.y, tid = threadIdx.x;
-  int n, sg;
-  const Lattice la = block_lattice(a.la, a.b0 + mat, n, sg);
-  double zr = la.mu, zi = (2.0 * n + 1.0) * kPi * la.T;
-  if (la.zshift) {
-    zr = la.zshift[2 * n];
-    zi = la.zshift[2 * n + 1];
-  }
-  const Node* nodes = tree_of(a, la.t, zi);
-  const Node nd = nodes[first + blockIdx.x];
-  const int p = nd.p, m = nd.p + nd.q;
-  Z* base = a.fronts + (size_t)mat * a.stride;
-  Z* F = base + nd.front;
-  Z* A = reinterpret_cast<Z*>(smem);
-  Z* X = A + nd.pw * m;
-  Z* bt = X + nd.pw * (m - nd.pw);
+  const int tid = gr.tid, NT = gr.size;
+  const Node nd = B.nodes[node];
+  const int p = nd.p, m = nd.p + nd.q, pw = nd.pw;
+  Z* F = B.fronts + nd.front;
+  Z* A = reinterpret_cast<Z*>(smem + at);
+  Z* X = A + pw * (m - pw + kRows);
+  Z* F11 = X + pw * (m - pw);
+  Z* rowb = F11 + pw * pw;        // [2][pw]: the pivot's row
+  Z* colb = rowb + 2 * pw;        // [2][pw + 1]: minus its column, then the reciprocal
+  Z* bt = colb + 2 * (pw + 1);
   Z* diag = bt + nd.blacks;
-  double* mag = reinterpret_cast<double*>(diag + p);
+  double* mag = reinterpret_cast<double*>(diag + p + 1);
   int16_t* site = reinterpret_cast<int16_t*>(mag + 32);
   int16_t* cm0 = site + m;
   int16_t* cm1 = cm0 + m;
   int16_t* adj = cm1 + m;
-  double ld = 0.0;  // warp 0
+  double mant = 1.0;  // first warp: the node's share of |det A|^2
+  int expo = 0;
   for (int i = tid; i < m; i += NT) {
-    site[i] = a.tab[nd.sites + i];
-    cm0[i] = nd.child[0] >= 0 ? a.tab[nd.cmap[0] + i] : (int16_t)-1;
-    cm1[i] = nd.child[1] >= 0 ? a.tab[nd.cmap[1] + i] : (int16_t)-1;
-    if (i < p) zset(diag[i], zr - site_energy(la, a.tab[nd.sites + i], sg), zi);
+    const int s = B.tab[nd.sites + i], x = s / B.la.L;
+    site[i] = (int16_t)((x << 8) | (s - x * B.la.L));
+    cm0[i] = nd.child[0] >= 0 ? B.tab[nd.cmap[0] + i] : (int16_t)-1;
+    cm1[i] = nd.child[1] >= 0 ? B.tab[nd.cmap[1] + i] : (int16_t)-1;
   }
+  for (int i = tid; i <= p; i += NT)
+    zset(diag[i], i < p ? B.zr - site_energy(B.la, B.tab[nd.sites + i], B.sg) : B.la.t,
+         i < p ? B.zi : 0.0);
   if (nd.blacks) {
-    for (int i = tid; i < 4 * m; i += NT) adj[i] = a.tab[nd.adj + i];
-    for (int b0 = 0; b0 < nd.blacks; b0 += 32)
-      if (tid < 32) {
-        double l = 0.0;
-        if (b0 + tid < nd.blacks) {
-          const double ar = zr - site_energy(la, a.tab[nd.bsite + b0 + tid], sg);
-          Z z, t2;
-          zset(z, ar, zi);
-          zset(t2, la.t * la.t, 0.0);
-          bt[b0 + tid] = zmul(t2, zinv(z));
-          const double m2 = ar * ar + zi * zi;
-          const bool ok = m2 > 0.0 && isfinite(m2);
-          if (!ok) atomicOr(a.flags, 1);
-          l = 0.5 * log(ok ? m2 : 1.0);
-        }
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) l += __shfl_xor_sync(0xffffffffu, l, off);
-        ld += l;
+    for (int i = tid; i < m; i += NT) adj[i] = B.tab[nd.adj + i];
+    if (tid < 32) {
+      double m2 = 1.0;
+      if (tid < nd.blacks) {
+        Z z, t2;
+        zset(z, B.zr - site_energy(B.la, B.tab[nd.bsite + tid], B.sg), B.zi);
+        zset(t2, B.la.t * B.la.t, 0.0);
+        bt[tid] = zneg(zmul(t2, zinv(z, &m2)));
       }
+      det_mul(m2, mant, expo, B.flags);
+    }
   }
   Front<Z> f;
-  f.L = la.L;
-  f.t = la.t;
+  f.L = B.la.L;
   for (int c = 0; c < 2; ++c) {
     f.c[c] = nullptr;
     f.cm[c] = 0;
     if (nd.child[c] >= 0) {
-      const Node k = nodes[nd.child[c]];
+      const Node k = B.nodes[nd.child[c]];
       const int mc = k.p + k.q;
-      f.c[c] = base + k.front + (size_t)k.p * mc + k.p;
+      f.c[c] = B.fronts + k.front + (size_t)k.p * mc + k.p;
       f.cm[c] = mc;
     }
   }
   f.p = p;
   f.leaf = nd.blacks > 0;
-  f.site = site;
-  f.cmap0 = cm0;
-  f.cmap1 = cm1;
-  f.adj = adj;
-  f.bt = bt;
-  f.diag = diag;
-  __syncthreads();
+  f.site = off(site);
+  f.cmap0 = off(cm0);
+  f.cmap1 = off(cm1);
+  f.adj = off(adj);
+  f.bt = off(bt);
+  f.diag = off(diag);
+  gr.sync();
   for (int pa = 0; pa < nd.npan; ++pa) {
-    const int o = pa * nd.pw, w = min(nd.pw, p - o), l = m - o, r = l - w;
-    // ---- the panel's rows
-    for (int e = tid; e < w * l; e += NT) {
-      const int i = e / l, j = e - i * l;
-      const int hi = max(i, j) + o, lo = min(i, j) + o;
-      A[i * l + j] = pa == 0 ? f.at(hi, lo) : F[(size_t)hi * m + lo];
-    }
-    __syncthreads();
-    // ---- P = F11^{-1} in place (Gauss-Jordan, diagonal pivots in order)
-    for (int c = 0; c < w; ++c) {
-      const Z d = A[c * l + c];
-      const Z dinv = zinv(d);
-      if (tid == 0) mag[c] = zre(d) * zre(d) + zim(d) * zim(d);
-      Z val[kEntries];
-#pragma unroll
-      for (int u = 0; u < kEntries; ++u) {
-        const int e = tid + u * NT;
-        if (e >= w * w) break;
-        const int i = e / w, j = e - i * w;
-        const Z row = A[c * l + j], col = A[i * l + c];
-        if (i == c) {
-          val[u] = j == c ? dinv : zmul(row, dinv);
-        } else if (j == c) {
-          val[u] = zneg(zmul(col, dinv));
-        } else {
-          Acc s;
-          acc_of(s, A[i * l + j]);
-          mac(s, zneg(col), zmul(row, dinv));
-          val[u] = acc_get(s);
-        }
-      }
-      __syncthreads();
-#pragma unroll
-      for (int u = 0; u < kEntries; ++u) {
-        const int e = tid + u * NT;
-        if (e >= w * w) break;
-        const int i = e / w, j = e - i * w;
-        A[i * l + j] = val[u];
-      }
-      __syncthreads();
-    }
-    if (tid < 32) {
-      const double m2 = tid < w ? mag[tid] : 1.0;
-      const bool ok = m2 > 0.0 && isfinite(m2);
-      if (!ok) atomicOr(a.flags, 1);
-      double v = 0.5 * log(ok ? m2 : 1.0);
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-      ld += v;
-    }
-    // ---- X = P F12, two rows per thread
-    const int hw = (w + 1) / 2;
-    for (int e = tid; e < hw * r; e += NT) {
-      const int i = e / r, j = e - i * r;
-      const int i1 = min(i + hw, w - 1);
-      Acc s0{}, s1{};
+    const int o = pa * pw, w = min(pw, p - o), l = m - o, r = l - w;
+    const int lda = r + kRows;  // row blocks read up to kRows - 1 entries past r
+    // ---- the panel to shared memory (F12 stays there), then to the registers
+    for (int i = tid >> 5; i < w; i += NT >> 5)
 #pragma unroll 2
-      for (int k = 0; k < w; ++k) {
-        const Z v = A[k * l + w + j];
-        mac(s0, A[i * l + k], v);
-        mac(s1, A[i1 * l + k], v);
+      for (int j = tid & 31; j < l; j += 32) {
+        const int hi = max(i, j) + o, lo = min(i, j) + o;
+        const Z v = pa == 0 ? f.at(hi, lo) : F[hi * m + lo];
+        if (j < w)
+          F11[i * w + j] = v;
+        else
+          A[i * lda + j - w] = v;
       }
-      X[i * r + j] = acc_get(s0);
-      if (i + hw < w) X[i1 * r + j] = acc_get(s1);
-    }
-    __syncthreads();
-    // ---- P and X to the front's panel rows
-    for (int e = tid; e < w * l; e += NT) {
-      const int i = e / l, j = e - i * l;
-      F[(size_t)(o + i) * m + o + j] = j < w ? A[i * l + j] : X[i * r + j - w];
-    }
-    // ---- F22 - F12^T X, lower triangle: each thread four entries, rows and columns h apart so
-    // that neighbouring lanes read neighbouring entries
-    const int h = (r + 1) / 2, tiles = h * (h + 1) / 2;
+    gr.sync();
+    Z* Fo = F + (size_t)o * (m + 1);
+    if (w <= NT / w)
+      invert<Z, 1>(gr, w, off(F11), off(rowb), off(colb), off(mag), Fo, m);
+    else
+      invert<Z, kSlots>(gr, w, off(F11), off(rowb), off(colb), off(mag), Fo, m);
+    gr.sync();
+    if (r > 0)
+      times_fit<Z, false, false>(gr, w, w, r, off(F11), w, off(X), r, (const Z*)F, off(A), lda, 0,
+                                 Fo + w, m);
+    gr.sync();
+    if (tid < 32) det_mul(tid < w ? mag[tid] : 1.0, mant, expo, B.flags);
+    // ---- the rest; fewer rows per thread where more would leave threads idle
     Z* R = F + (size_t)(o + w) * (m + 1);
-    for (int e = tid; e < tiles; e += NT) {
-      int ti = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);
-      while ((ti + 1) * (ti + 2) / 2 <= e) ++ti;
-      while (ti * (ti + 1) / 2 > e) --ti;
-      const int tj = e - ti * (ti + 1) / 2;
-      const bool in_i = ti + h < r, in_j = tj + h < r;
-      const int i1 = in_i ? ti + h : ti, j1 = in_j ? tj + h : tj;
-      Acc s00{}, s10{}, s01{}, s11{};
-#pragma unroll 2
-      for (int k = 0; k < w; ++k) {
-        const Z* Ak = A + k * l + w;
-        const Z a0 = zneg(Ak[ti]), a1 = zneg(Ak[i1]);
-        const Z x0 = X[k * r + tj], x1 = X[k * r + j1];
-        mac(s00, a0, x0);
-        mac(s10, a1, x0);
-        mac(s01, a0, x1);
-        mac(s11, a1, x1);
-      }
-      auto put = [&](int i, int j, const Acc& s) {
-        const Z v = pa == 0 ? f.at(o + w + i, o + w + j) : R[(size_t)i * m + j];
-        R[(size_t)i * m + j] = zadd(v, acc_get(s));
-      };
-      put(ti, tj, s00);
-      if (in_i) put(i1, tj, s10);
-      if (in_i && in_j) put(i1, j1, s11);
-      if (in_j && ti != tj) put(j1, ti, s01);
-    }
-    __syncthreads();
+    auto cost = [&](int kr) {
+      const int nb = (r + kr - 1) / kr;
+      return (kr * nb * (nb + 1) / 2 + NT - 1) / NT * (3 * kr + 1);
+    };
+    if (cost(2) <= cost(1))
+      update_rest<Z, 2>(gr, f, pa == 0, o + w, w, r, m, off(A), lda, off(X), R);
+    else
+      update_rest<Z, 1>(gr, f, pa == 0, o + w, w, r, m, off(A), lda, off(X), R);
+    gr.sync();
   }
-  double* ldp = a.ldp + (size_t)mat * a.nnodes;
-  if (tid == 0) ldp[first + blockIdx.x] = ld;
-  if (nd.parent < 0) {  // the root: ln|det A| over all nodes in a fixed order
-    __syncthreads();
-    __shared__ double part[NT];
-    double v = 0.0;
-    for (int k = tid; k < a.nnodes; k += NT) v += ldp[k];
-    part[tid] = v;
-    __syncthreads();
-    for (int s = NT / 2; s > 0; s >>= 1) {
-      if (tid < s) part[tid] += part[tid + s];
-      __syncthreads();
-    }
-    if (tid == 0) a.ld[a.b0 + mat] = part[0];
-  }
+  if (tid == 0) B.det[node] = {mant, expo, 0};
 }
 
-// One node of one block, down.  Panels in reverse; R is the part of the front after the panel,
-// already G.  Four rows of Y = X R per thread: R is read from global memory (L1 and L2 hold it),
-// X broadcast from shared memory.
-template <typename Z, int NT>
-__global__ void __launch_bounds__(NT) k_nest_down(NestArgs<Z> a, int first) {
+// One front, down.  Panels in reverse; R is the part of the front after the panel, already G.  A
+// node without children keeps nothing but its own rows: R is then read from the parent's front.
+template <typename Z>
+__device__ __forceinline__ void front_down(const Block<Z>& B, int node, const Group& gr, int at) {
   extern __shared__ __align__(16) unsigned char smem[];
   using Acc = typename AccOf<Z>::type;
-  const int mat = blockIdx.y, tid = threadIdx.x;
-  int n, sg;
-  const Lattice la = block_lattice(a.la, a.b0 + mat, n, sg);
-  double zr = la.mu, zi = (2.0 * n + 1.0) * kPi * la.T;
-  if (la.zshift) {
-    zr = la.zshift[2 * n];
-    zi = la.zshift[2 * n + 1];
-  }
-  const Node* nodes = tree_of(a, la.t, zi);
-  const Node nd = nodes[first + blockIdx.x];
+  const int tid = gr.tid, NT = gr.size;
+  const Node nd = B.nodes[node];
   const int p = nd.p, q = nd.q, m = nd.p + nd.q;
-  Z* base = a.fronts + (size_t)mat * a.stride;
-  Z* F = base + nd.front;
+  Z* F = B.fronts + nd.front;
   const int ldx = (m - nd.pw) | 1;  // odd: rows of 16-byte entries start in different banks
-  Z* X = reinterpret_cast<Z*>(smem);
+  Z* X = reinterpret_cast<Z*>(smem + at);
   Z* Y = X + nd.pw * ldx;
-  int16_t* map = reinterpret_cast<int16_t*>(Y + nd.pw * ldx);
-  double* gd = a.gd + (size_t)(a.b0 + mat) * la.N;
+  Z* P = Y + nd.pw * ldx;
+  int16_t* map = reinterpret_cast<int16_t*>(P + nd.pw * nd.pw);
+  const bool direct = nd.child[0] < 0 && nd.npan <= 1 && nd.parent >= 0;
+  const Z* G = nullptr;  // the parent's front
+  int mp = 0;
   if (nd.parent >= 0) {
-    const Node pr = nodes[nd.parent];
-    const int mp = pr.p + pr.q;
-    const Z* G = base + pr.front;
-    for (int i = tid; i < q; i += NT) map[i] = a.tab[nd.pmap + i];
-    __syncthreads();
-    for (int e = tid; e < q * q; e += NT) {
-      const int i = e / q, j = e - i * q;
-      F[(size_t)(p + i) * m + p + j] = G[(size_t)map[i] * mp + map[j]];
+    const Node pr = B.nodes[nd.parent];
+    mp = pr.p + pr.q;
+    G = B.fronts + pr.front;
+    for (int i = tid; i < q; i += NT) map[i] = B.tab[nd.pmap + i];
+    gr.sync();
+    if (!direct) {
+      // G_bb into the front, several entries in flight per thread
+      for (int i = tid >> 5; i < q; i += NT >> 5) {
+        const Z* Gi = G + map[i] * mp;
+        Z* Fi = F + (p + i) * m + p;
+        for (int j0 = tid & 31; j0 < q; j0 += 128) {
+          Z v[4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) v[u] = Gi[map[min(j0 + 32 * u, q - 1)]];
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+            if (j0 + 32 * u < q) Fi[j0 + 32 * u] = v[u];
+        }
+      }
+      gr.sync();
     }
-    __syncthreads();
   }
   for (int pa = nd.npan - 1; pa >= 0; --pa) {
     const int o = pa * nd.pw, w = min(nd.pw, p - o), r = m - o - w;
-    Z* R = F + (size_t)(o + w) * (m + 1);
-    for (int e = tid; e < w * r; e += NT) {
-      const int i = e / r, j = e - i * r;
-      X[i * ldx + j] = F[(size_t)(o + i) * m + o + w + j];
-    }
-    __syncthreads();
-    const int hw = (w + 3) / 4;
-    for (int e = tid; e < hw * r; e += NT) {
-      const int i = e / r, j = e - i * r;
-      const int i1 = min(i + hw, w - 1), i2 = min(i + 2 * hw, w - 1), i3 = min(i + 3 * hw, w - 1);
-      Acc s0{}, s1{}, s2{}, s3{};
+    const Z* R = F + (size_t)(o + w) * (m + 1);
+    for (int i = tid >> 5; i < w; i += NT >> 5)
+      for (int j = tid & 31; j < r; j += 32) X[i * ldx + j] = F[(o + i) * m + o + w + j];
+    gr.sync();
+    if (direct)
+      times_fit<Z, true, true>(gr, w, r, r, off(X), ldx, off(Y), ldx, G, 0, mp, off(map), (Z*)nullptr, 0);
+    else if (r > 0)
+      times_fit<Z, false, true>(gr, w, r, r, off(X), ldx, off(Y), ldx, R, 0, m, 0, (Z*)nullptr, 0);
+    gr.sync();
+    // ---- G_pp = P + Y (-X)^T, lower triangle; ks threads share an entry's sum (by the front's
+    // shape alone: the order of a sum must not depend on how many threads there are)
+    const int outs = w * (w + 1) / 2, ks = r >= 48 ? 4 : 2;
+    for (int e0 = 0; e0 < outs; e0 += NT / ks) {
+      const int e = min(e0 + tid / ks, outs - 1), k0 = tid % ks;
+      int i, j;
+      triangle(e, i, j);
+      Acc s{};
+      if (k0 == 0) acc_of(s, F[(size_t)(o + i) * m + o + j]);
 #pragma unroll 2
-      for (int k = 0; k < r; ++k) {
-        const Z g = R[(size_t)k * m + j];
-        mac(s0, X[i * ldx + k], g);
-        mac(s1, X[i1 * ldx + k], g);
-        mac(s2, X[i2 * ldx + k], g);
-        mac(s3, X[i3 * ldx + k], g);
+      for (int k = k0; k < r; k += ks) mac(s, Y[i * ldx + k], X[j * ldx + k]);
+      Z g = acc_get(s);
+      for (int off = 1; off < ks; off <<= 1) g = zadd(g, zshfl_xor(g, off));
+      if (k0 == 0 && e0 + tid / ks < outs) {
+        if (direct) {
+          P[i * w + j] = g;
+          P[j * w + i] = g;
+        } else {
+          F[(size_t)(o + i) * m + o + j] = g;
+          F[(size_t)(o + j) * m + o + i] = g;
+        }
+        if (i == j) B.gd[B.tab[nd.sites + o + i]] = B.la.zshift ? zim(g) : B.sg * zre(g);
       }
-      Y[i * ldx + j] = acc_get(s0);
-      if (i + hw < w) Y[i1 * ldx + j] = acc_get(s1);
-      if (i + 2 * hw < w) Y[i2 * ldx + j] = acc_get(s2);
-      if (i + 3 * hw < w) Y[i3 * ldx + j] = acc_get(s3);
     }
-    __syncthreads();
-    for (int e = tid; e < w * (w + 1) / 2; e += NT) {
-      int i = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);
-      while ((i + 1) * (i + 2) / 2 <= e) ++i;
-      while (i * (i + 1) / 2 > e) --i;
-      const int j = e - i * (i + 1) / 2;
-      Acc s;
-      acc_of(s, F[(size_t)(o + i) * m + o + j]);
-#pragma unroll 2
-      for (int k = 0; k < r; ++k) mac(s, Y[i * ldx + k], X[j * ldx + k]);
-      const Z g = acc_get(s);
-      F[(size_t)(o + i) * m + o + j] = g;
-      if (i != j) F[(size_t)(o + j) * m + o + i] = g;
-      if (i == j)
-        gd[a.tab[nd.sites + o + i]] = la.zshift ? zim(g) : sg * zre(g);
+    if (!direct) {
+      for (int i = tid >> 5; i < w; i += NT >> 5)
+        for (int j = tid & 31; j < r; j += 32) F[(o + i) * m + o + w + j] = Y[i * ldx + j];
+      for (int j = tid >> 4; j < r; j += NT >> 4)
+        for (int i = tid & 15; i < w; i += 16) F[(o + w + j) * m + o + i] = Y[i * ldx + j];
     }
-    for (int e = tid; e < w * r; e += NT) {
-      const int i = e / r, j = e - i * r;
-      F[(size_t)(o + i) * m + o + w + j] = zneg(Y[i * ldx + j]);
-    }
-    for (int e = tid; e < w * r; e += NT) {
-      const int j = e / w, i = e - j * w;
-      F[(size_t)(o + w + j) * m + o + i] = zneg(Y[i * ldx + j]);
-    }
-    __syncthreads();
+    gr.sync();
   }
-  // blacks: G_bb = 1/a + (t/a)^2 sum_{u,v} G_uv over the black's neighbours
+  // blacks: G_bb = 1/a + (t/a)^2 sum_{u,v} G_uv over the black's neighbours, four threads each
+  // (one neighbour u per thread); such leaves have one panel
   if (nd.blacks) {
-    for (int b = tid; b < nd.blacks; b += NT) {
-      const int s = a.tab[nd.bsite + b];
-      Z z, t2, sum;
-      zset(z, zr - site_energy(la, s, sg), zi);
-      zset(t2, la.t * la.t, 0.0);
+    for (int b0 = 0; b0 < nd.blacks; b0 += NT / 4) {
+      const int b = min(b0 + tid / 4, nd.blacks - 1), u = tid & 3;
+      const int s = B.tab[nd.bsite + b];
+      const int iu = B.tab[nd.bnbr + 4 * b + u];
+      Z sum;
       zset(sum, 0.0, 0.0);
-      for (int u = 0; u < 4; ++u) {
-        const int iu = a.tab[nd.bnbr + 4 * b + u];
-        for (int v = 0; v < 4; ++v) sum = zadd(sum, F[(size_t)iu * m + a.tab[nd.bnbr + 4 * b + v]]);
+#pragma unroll
+      for (int v = 0; v < 4; ++v) {
+        const int iv = B.tab[nd.bnbr + 4 * b + v], hi = max(iu, iv), lo = min(iu, iv);
+        sum = zadd(sum, hi < p    ? P[hi * p + lo]
+                        : lo < p  ? Y[lo * ldx + hi - p]
+                                  : G[(size_t)map[hi - p] * mp + map[lo - p]]);
       }
-      const Z ai = zinv(z);
-      const Z g = zadd(ai, zmul(zmul(zmul(ai, t2), ai), sum));
-      gd[s] = la.zshift ? zim(g) : sg * zre(g);
+      sum = zadd(sum, zshfl_xor(sum, 1));
+      sum = zadd(sum, zshfl_xor(sum, 2));
+      if (u == 0 && b0 + tid / 4 < nd.blacks) {
+        Z z, t2;
+        zset(z, B.zr - site_energy(B.la, s, B.sg), B.zi);
+        zset(t2, B.la.t * B.la.t, 0.0);
+        const Z ai = zinv(z);
+        const Z g = zadd(ai, zmul(zmul(zmul(ai, t2), ai), sum));
+        B.gd[s] = B.la.zshift ? zim(g) : B.sg * zre(g);
+      }
+    }
+    gr.sync();
+  }
+}
+
+// Barrier of the CTAs that share a block (global memory written before it is visible after it).
+template <bool kCluster>
+__device__ __forceinline__ void block_sync() {
+  if (kCluster)
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::
+                     : "memory");
+  else
+    __syncthreads();
+}
+
+// The elimination of one block by one CTA, or by a cluster of them: level after level, up and then
+// down, each level's fronts dealt out to the CTAs' thread groups.  A launch of a single level
+// (k1 = k0 + 1) needs no barrier and may spread a block over any number of CTAs.
+template <typename Z, int NT, bool kCluster>
+__global__ void __launch_bounds__(NT, NT == 256 ? 4 : 1) k_nested(NestArgs<Z> a) {
+  const int tid = threadIdx.x;
+  const int csize = a.csize, rank = blockIdx.x % csize;
+  const int mat = blockIdx.x / csize;
+  __shared__ Block<Z> B;  // read where needed: in registers it would be live everywhere
+  __shared__ int form;
+  if (tid == 0) {
+    int n;
+    B.la = block_lattice(a.la, a.b0 + mat, n, B.sg);
+    B.zr = B.la.mu;
+    B.zi = (2.0 * n + 1.0) * kPi * B.la.T;
+    if (B.la.zshift) {
+      B.zr = B.la.zshift[2 * n];
+      B.zi = B.la.zshift[2 * n + 1];
+    }
+    form = mat < a.ndense ? 1 : 0;
+    B.nodes = a.nodes + form * a.nnodes;
+    B.tab = a.tab;
+    B.fronts = a.fronts + (size_t)mat * a.stride;
+    B.det = a.det + (size_t)mat * a.nnodes;
+    B.gd = a.gd + (size_t)(a.b0 + mat) * B.la.N;
+    B.flags = a.flags;
+  }
+  __syncthreads();
+  for (int k = a.k0; k < a.k1; ++k) {
+    const bool up = k < a.nlevels;
+    const LevelPlan& lv = a.lv[form][up ? a.nlevels - 1 - k : k - a.nlevels];
+    const int group = tid / lv.group, groups = NT / lv.group;
+    const Group gr{lv.group, tid - group * lv.group, 1 + group};
+    const int at = group * lv.smem;
+    for (int f = rank + csize * group; f < lv.count; f += csize * groups) {
+      if (up)
+        front_up(B, lv.first + f, gr, at);
+      else
+        front_down(B, lv.first + f, gr, at);
+    }
+    if (k + 1 == a.k1 && k != a.nlevels - 1) break;
+    block_sync<kCluster>();
+    if (k == a.nlevels - 1 && rank == 0 && tid < 32) {  // ln|det A| over all nodes, fixed order
+      double v = 0.0;
+      int e = 0;
+      for (int i = tid; i < a.nnodes; i += 32) {
+        v += log(B.det[i].mant);
+        e += B.det[i].exp;
+      }
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) {
+        v += __shfl_xor_sync(0xffffffffu, v, off);
+        e += __shfl_xor_sync(0xffffffffu, e, off);
+      }
+      if (tid == 0) a.ld[a.b0 + mat] = 0.5 * (v + (double)e * 0.69314718055994530942);
     }
   }
 }
@@ -552,68 +863,86 @@ __global__ void __launch_bounds__(256) k_nest_trace(int N, int b0, const double*
   } while (0)
 
 size_t up_smem(const nested::Node& n) {
-  const size_t m = n.p + n.q;
-  return 16 * ((size_t)n.pw * (2 * m - n.pw) + n.blacks + n.p) + 32 * sizeof(double) +
-         sizeof(int16_t) * m * (n.blacks ? 7 : 3);
+  const size_t m = n.p + n.q, pw = n.pw;
+  return 16 * (pw * (2 * (m - pw) + kRows) + pw * pw + 2 * pw + 2 * (pw + 1) + n.blacks + n.p + 1) +
+         32 * sizeof(double) + sizeof(int16_t) * m * (n.blacks ? 4 : 3);
 }
 size_t down_smem(const nested::Node& n) {
   const size_t m = n.p + n.q;
-  return 32 * (size_t)n.pw * ((m - n.pw) | 1) + sizeof(int16_t) * n.q;
+  return 16 * (2 * (size_t)n.pw * ((m - n.pw) | 1) + (size_t)n.pw * n.pw) + sizeof(int16_t) * n.q;
 }
-
-struct LevelPlan {
-  int first, count, nt;
-  size_t smem_up, smem_down;
-};
 
 }  // namespace
 
-// Per-context state: the tree's tables on the device and the launch plan.
+// Per-context state: the tree's tables on the device and the shapes that the launch plans follow.
 struct Nested {
   Node* d_nodes = nullptr;
   int16_t* d_tab = nullptr;
-  std::vector<LevelPlan> levels;
+  struct Shape {
+    int first, count, group, smem;  // group: the fewest threads for a front
+  };
+  std::vector<Shape> levels[2];
   int nnodes = 0;
   long long stride = 0;   // entries per block
   int cap = 0;            // blocks per pass
+  int sms = 1;
 };
 
 namespace {
 
-template <typename Z, int NT>
-sca_status allow_smem() {
-  static ContextOnce once;
-  if (once.done()) return SCA_OK;
-  int dev = 0, optin = 0;
-  cudaError_t err = cudaGetDevice(&dev);
-  if (err == cudaSuccess) err = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  cudaFuncAttributes fa;
-  if (err == cudaSuccess) err = cudaFuncGetAttributes(&fa, k_nest_up<Z, NT>);
-  if (err == cudaSuccess)
-    err = cudaFuncSetAttribute(k_nest_up<Z, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               optin - (int)fa.sharedSizeBytes);
-  if (err == cudaSuccess) err = cudaFuncGetAttributes(&fa, k_nest_down<Z, NT>);
-  if (err == cudaSuccess)
-    err = cudaFuncSetAttribute(k_nest_down<Z, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               optin - (int)fa.sharedSizeBytes);
-  if (err != cudaSuccess) return cuda_fail(err, "nested elimination set-up");
-  once.mark();
-  return SCA_OK;
+// Plan of a whole elimination by CTAs of 512 threads, a.csize of them per block: a level's fronts
+// are dealt out over the CTAs' groups, whose size is the fewest threads for a front where there
+// are fronts enough and grows to the whole CTA where there are not, or where shared memory needs
+// fewer groups.  Returns the shared memory that a CTA needs.
+template <typename Z>
+size_t plan_levels(const Nested& ne, NestArgs<Z>& a) {
+  constexpr int nt = 512, room = 220 << 10;
+  static_assert(nt / 64 < 16, "a group above a warp needs one of the 15 barriers left");
+  size_t need = 0;
+  for (int form = 0; form < 2; ++form)
+    for (size_t k = 0; k < ne.levels[form].size(); ++k) {
+      const Nested::Shape& s = ne.levels[form][k];
+      int g = s.group;
+      while (2 * g <= nt && ((nt / (2 * g)) * a.csize >= s.count || nt / g * s.smem > room)) g *= 2;
+      a.lv[form][k] = {s.first, s.count, g, s.smem};
+      need = std::max(need, (size_t)(nt / g) * s.smem);
+    }
+  return need;
 }
 
-template <typename Z, int NT>
-sca_status launch_level(Engine& e, const NestArgs<Z>& a, const LevelPlan& lv, int cnt, bool up,
-                        cudaStream_t s) {
-  sca_status st = allow_smem<Z, NT>();
-  if (st != SCA_OK) return st;
-  const int kind = up ? kNestUp : kNestDown;
+template <typename Z, int NT, bool kCluster>
+sca_status launch(Engine& e, const NestArgs<Z>& a, int cnt, size_t smem, cudaStream_t s) {
+  static ContextOnce once;
+  cudaError_t err;
+  if (!once.done()) {
+    int dev = 0, optin = 0;
+    cudaFuncAttributes fa;
+    if ((err = cudaGetDevice(&dev)) != cudaSuccess ||
+        (err = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess ||
+        (err = cudaFuncGetAttributes(&fa, k_nested<Z, NT, kCluster>)) != cudaSuccess ||
+        (err = cudaFuncSetAttribute(k_nested<Z, NT, kCluster>,
+                                    cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    optin - (int)fa.sharedSizeBytes)) != cudaSuccess)
+      return cuda_fail(err, "nested elimination set-up");
+    once.mark();
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(cnt * a.csize));
+  cfg.blockDim = dim3(NT);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)a.csize;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = kCluster ? 1 : 0;
+  const int kind = a.k0 < a.nlevels ? kNestUp : kNestDown;
   prof_begin(e, kind, s);
-  if (up)
-    k_nest_up<Z, NT><<<dim3(lv.count, cnt), NT, lv.smem_up, s>>>(a, lv.first);
-  else
-    k_nest_down<Z, NT><<<dim3(lv.count, cnt), NT, lv.smem_down, s>>>(a, lv.first);
+  err = cudaLaunchKernelEx(&cfg, k_nested<Z, NT, kCluster>, a);
   prof_end(e, kind, s);
-  SCA_LAUNCH_CHECK(up ? "nested elimination" : "nested inverse diagonal");
+  g_launches.fetch_add(1, std::memory_order_relaxed);
+  if (err != cudaSuccess) return cuda_fail(err, "nested elimination");
   return SCA_OK;
 }
 
@@ -626,26 +955,67 @@ sca_status run_nested_t(Engine& e, const Lattice& la, bool up, bool down, cudaSt
   a.fronts = static_cast<Z*>(e.M);
   a.stride = ne.stride;
   a.nnodes = ne.nnodes;
+  a.nlevels = (int)ne.levels[0].size();
   a.la = la;
   a.ld = e.ld;
   a.gd = e.gd;
   a.flags = e.flags;
-  const int cap = std::min(ne.cap, 65535);
-  for (int b0 = 0; b0 < e.B; b0 += cap) {
-    const int cnt = std::min(cap, e.B - b0);
+  for (int b0 = 0; b0 < e.B; b0 += ne.cap) {
+    const int cnt = std::min(ne.cap, e.B - b0);
     a.b0 = b0;
-    a.ldp = reinterpret_cast<double*>(a.fronts + (size_t)cnt * ne.stride);
-    const int nl = (int)ne.levels.size();
-    for (int pass = 0; pass < 2; ++pass) {
-      if (!(pass == 0 ? up : down)) continue;
-      for (int k = 0; k < nl; ++k) {
-        const LevelPlan& lv = ne.levels[pass == 0 ? nl - 1 - k : k];
-        const sca_status st = lv.nt == 64    ? launch_level<Z, 64>(e, a, lv, cnt, pass == 0, s)
-                              : lv.nt == 128 ? launch_level<Z, 128>(e, a, lv, cnt, pass == 0, s)
-                                             : launch_level<Z, 256>(e, a, lv, cnt, pass == 0, s);
-        if (st != SCA_OK) return st;
+    a.det = reinterpret_cast<Det*>(a.fronts + (size_t)cnt * ne.stride);
+    const int nl = a.nlevels, p0 = up ? 0 : nl, p1 = down ? 2 * nl : nl;
+    sca_status st = SCA_OK;
+    const int dense = std::min(cnt, std::max(0, e.nest_dense - b0));
+    a.ndense = dense;
+    if (cnt > ne.sms) {
+      // the two forms side by side: the few blocks with dense leaves on the high-priority stream
+      const bool fork = dense > 0 && dense < cnt && e.side != nullptr;
+      cudaError_t err = cudaSuccess;
+      if (fork) {
+        err = cudaEventRecord(e.ev_fork, s);
+        if (err == cudaSuccess) err = cudaStreamWaitEvent(e.side, e.ev_fork, 0);
+        if (err != cudaSuccess) return cuda_fail(err, "fork");
       }
+      for (int form = 1; form >= 0; --form) {
+        const int n = form ? dense : cnt - dense;
+        if (n == 0) continue;
+        NestArgs<Z> f = a;  // the form's blocks alone
+        f.b0 = b0 + (form ? 0 : dense);
+        f.fronts = a.fronts + (size_t)(f.b0 - b0) * a.stride;
+        f.det = a.det + (size_t)(f.b0 - b0) * a.nnodes;
+        f.ndense = form ? n : 0;
+        for (int k = p0; k < p1; ++k) {
+          const int level = k < nl ? nl - 1 - k : k - nl;
+          f.k0 = k;
+          f.k1 = k + 1;
+          const Nested::Shape& sh = ne.levels[form][level];
+          int g = sh.group;  // the fewest threads while they fill the SMs; four CTAs per SM
+          while (2 * g <= 256 && ((long long)sh.count * n * g < 1024ll * ne.sms ||
+                                  256 / g * sh.smem > 55 << 10))
+            g *= 2;
+          f.lv[form][level] = {sh.first, sh.count, g, sh.smem};
+          f.csize = (sh.count + 256 / g - 1) / (256 / g);
+          st = launch<Z, 256, false>(e, f, n, (size_t)(256 / g) * sh.smem, form && fork ? e.side : s);
+          if (st != SCA_OK) return st;
+        }
+      }
+      if (fork) {
+        err = cudaEventRecord(e.ev_join, e.side);
+        if (err == cudaSuccess) err = cudaStreamWaitEvent(s, e.ev_join, 0);
+        if (err != cudaSuccess) return cuda_fail(err, "join");
+      }
+    } else {
+      // CTAs per block: as many as there are SMs for, up to the portable cluster size
+      a.k0 = p0;
+      a.k1 = p1;
+      a.csize = 1;
+      while (a.csize < 8 && 2 * a.csize * cnt <= ne.sms) a.csize *= 2;
+      const size_t smem = plan_levels(ne, a);
+      st = a.csize > 1 ? launch<Z, 512, true>(e, a, cnt, smem, s)
+                       : launch<Z, 512, false>(e, a, cnt, smem, s);
     }
+    if (st != SCA_OK) return st;
     if (down && la.zshift) {
       prof_begin(e, kRefine, s);
       k_nest_trace<<<cnt, 256, 0, s>>>(e.N, b0, e.gd, e.tr);
@@ -670,7 +1040,7 @@ sca_status nested_prepare(Engine& e) {
   const nested::Tree td = nested::Builder(e.L).build(true);
   const size_t S = e.fp64 ? 8 : 4;
   const long long stride = std::max(t.entries, td.entries);
-  const size_t per_block = 16 * (size_t)stride + sizeof(double) * t.nodes.size();
+  const size_t per_block = 16 * (size_t)stride + sizeof(Det) * t.nodes.size();
   const size_t room = e.block_room;
   const long long cap = (long long)(room / per_block);
   if (cap < e.chunk) return SCA_OK;
@@ -680,15 +1050,18 @@ sca_status nested_prepare(Engine& e) {
   ne->nnodes = (int)td.nodes.size();
   ne->stride = stride;
   ne->cap = (int)std::min<long long>(cap, e.B);
-  for (const nested::Level& lv : t.levels) {
-    LevelPlan p{lv.first, lv.count, lv.mmax >= 80 ? 256 : lv.mmax >= 40 ? 128 : 64, 0, 0};
-    for (int k = lv.first; k < lv.first + lv.count; ++k)
-      for (const nested::Tree* f : {(const nested::Tree*)&t, &td}) {
-        p.smem_up = std::max(p.smem_up, up_smem(f->nodes[k]));
-        p.smem_down = std::max(p.smem_down, down_smem(f->nodes[k]));
+  const nested::Tree* forms[2] = {&t, &td};
+  for (int form = 0; form < 2; ++form)
+    for (const nested::Level& lv : forms[form]->levels) {
+      Nested::Shape sh{lv.first, lv.count, 32, 0};
+      for (int k = lv.first; k < lv.first + lv.count; ++k) {
+        const nested::Node& n = forms[form]->nodes[k];
+        while (10 * sh.group < 9 * (n.p + n.q) || n.pw > kSlots * (sh.group / n.pw)) sh.group *= 2;
+        sh.smem = (int)std::max<size_t>(sh.smem, std::max(up_smem(n), down_smem(n)));
       }
-    ne->levels.push_back(p);
-  }
+      sh.smem = (sh.smem + 15) / 16 * 16;
+      ne->levels[form].push_back(sh);
+    }
   // both forms in one table: the second's offsets follow the first's entries
   const int toff = (int)t.table.size();
   t.table.insert(t.table.end(), td.table.begin(), td.table.end());
@@ -696,7 +1069,12 @@ sca_status nested_prepare(Engine& e) {
     for (int* o : {&n.sites, &n.cmap[0], &n.cmap[1], &n.pmap, &n.bsite, &n.bnbr, &n.adj}) *o += toff;
     t.nodes.push_back(n);
   }
-  cudaError_t err = cudaMalloc((void**)&ne->d_nodes, sizeof(Node) * t.nodes.size());
+  int dev = 0;
+  cudaError_t err = cudaGetDevice(&dev);
+  if (err == cudaSuccess)
+    err = cudaDeviceGetAttribute(&ne->sms, cudaDevAttrMultiProcessorCount, dev);
+  if (err != cudaSuccess) { nested_release(e); return cuda_fail(err, "nested elimination set-up"); }
+  err = cudaMalloc((void**)&ne->d_nodes, sizeof(Node) * t.nodes.size());
   if (err == cudaSuccess) err = cudaMalloc((void**)&ne->d_tab, sizeof(int16_t) * t.table.size());
   if (err != cudaSuccess) {
     nested_release(e);

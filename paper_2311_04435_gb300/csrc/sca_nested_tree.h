@@ -35,10 +35,16 @@ namespace nested {
 constexpr int kMinL = 8;        // smallest lattice the tree is built for
 // A leaf's region: a 4 x 4 leaf has 8 blacks and 8 pivots (or 16 pivots) under 16 boundary sites.
 constexpr int kLeafSites = 20;
-constexpr int kPanel = 20;      // widest panel
-// Panels of large fronts stay narrower: two panels of w x m entries of 16 bytes in shared memory
-// then leave room for two CTAs per SM (m <= 192 at L = 64).
-inline int panel_width(int m) { return m > 150 ? 16 : kPanel; }
+// Widest panel of a front of m variables: F12 and X of a panel, 2 w (m - w) entries of 16 bytes,
+// and two w x w blocks take at most 50 KB of shared memory.
+inline int panel_width(int m) {
+  int w = 20;
+  while (16 * (w * (2 * (m - w) + 2) + 2 * w * w) > 50 * 1024) --w;
+  return w;
+}
+constexpr int kRows = 2;        // rows of a thread's output tile at most
+constexpr int kSlots = 2;       // entries of a pivots' block that a thread can hold
+constexpr int kMaxLevels = 10;
 
 struct Node {
   int p, q;            // pivots, boundary sites
@@ -50,7 +56,7 @@ struct Node {
   int blacks;          // number of blacks (leaves only)
   int bsite;           // table offset: site of each black
   int bnbr;            // table offset: 4 local variables per black
-  int adj;             // table offset: 4 blacks next to each local variable, -1 padded
+  int adj;             // table offset: bit mask of the blacks next to each local variable
   int npan, pw;        // panels and the width of the first ones (the last may be narrower)
   long long front;     // offset of the m x m front in a block's storage (entries)
 };
@@ -114,20 +120,19 @@ class Builder {
           n.bsite = (int)t.table.size();
           for (int s : black) t.table.push_back((int16_t)s);
           n.bnbr = (int)t.table.size();
-          std::vector<std::vector<int>> adj(m);
+          std::vector<int> adj(m, 0);
           for (int b = 0; b < n.blacks; ++b) {
             int nb[4];
             neighbours(black[b], nb);
             for (int k = 0; k < 4; ++k) {
               t.table.push_back((int16_t)pos_[nb[k]]);
-              adj[pos_[nb[k]]].push_back(b);
+              adj[pos_[nb[k]]] |= 1 << b;
             }
           }
           n.adj = (int)t.table.size();
-          for (int i = 0; i < m; ++i)
-            for (int k = 0; k < 4; ++k)
-              t.table.push_back((int16_t)(k < (int)adj[i].size() ? adj[i][k] : -1));
+          for (int i = 0; i < m; ++i) t.table.push_back((int16_t)adj[i]);
         }
+        // (a leaf is one panel: its block as a whole is well conditioned, parts of it are not)
         const int pw = panel_width(m);
         n.npan = (n.p + pw - 1) / pw;
         n.pw = n.npan ? (n.p + n.npan - 1) / n.npan : 0;

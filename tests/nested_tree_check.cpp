@@ -39,9 +39,11 @@ static void structure(const Tree& t, int* mmax, int* wmax) {
     for (int b = 0; b < n.blacks; ++b) ++seen.at(t.table.at(n.bsite + b));
     for (int k = 0; k < 4 * n.blacks; ++k)
       need(t.table.at(n.bnbr + k) >= 0 && t.table[n.bnbr + k] < m, "black's neighbour");
-    for (int k = 0; n.blacks && k < 4 * m; ++k) need(t.table.at(n.adj + k) < n.blacks, "adjacent black");
-    need(n.blacks <= 32 && n.pw <= kPanel, "a warp's width");
-    need(n.p == 0 || (n.npan * n.pw >= n.p && (n.npan - 1) * n.pw < n.p), "panels");
+    for (int k = 0; n.blacks && k < m; ++k)
+      need((t.table.at(n.adj + k) >> n.blacks) == 0, "adjacent black");
+    need(n.blacks <= 15 && n.pw <= 32, "a warp's width");
+    need(n.p > 0 && n.npan * n.pw >= n.p && (n.npan - 1) * n.pw < n.p, "panels");
+    need((n.child[0] < 0) == (n.child[1] < 0), "one child");
     if (n.parent >= 0) {
       const Node& par = t.nodes.at(n.parent);
       int prev = -1;
@@ -53,7 +55,7 @@ static void structure(const Tree& t, int* mmax, int* wmax) {
       }
     }
   }
-  need(entries == t.entries, "entries");
+  need(entries == t.entries && t.levels.size() <= kMaxLevels, "entries");
   for (int s : seen) need(s == 1, "site not eliminated once");
 }
 
@@ -130,11 +132,8 @@ static void eliminate(const Tree& t, double* ld_err, double* g_err) {
           if (hi == lo) v += a[tab(n.sites + hi)];
           else if (adjacent(tab(n.sites + hi), tab(n.sites + lo))) v += tt;
         }
-        for (int x = 0; n.blacks && x < 4; ++x) {
-          const int b = tab(n.adj + 4 * hi + x);
-          for (int y = 0; b >= 0 && y < 4; ++y)
-            if (tab(n.adj + 4 * lo + y) == b) v -= bt.at(b);
-        }
+        for (int b = 0; b < n.blacks; ++b)
+          if (tab(n.adj + hi) >> b & tab(n.adj + lo) >> b & 1) v -= bt[b];
         return v;
       };
       for (int pa = 0; pa < n.npan; ++pa) {

@@ -90,7 +90,8 @@ def test_chunks_forward_backward_and_nan(L, prec, monkeypatch):
     assert om3 == om and np.array_equal(g3, g)
 
 
-def test_profile_counts_one_launch_per_level():
+def test_profile_counts_the_nested_launches():
+    """One launch eliminates and takes diag(G); a forward / backward pair takes two."""
     p = api.Params(20, 4, U=4.0, T=0.1, delta=0.4, prec="bf16x3")
     phi = inputs.seed_phi(1, p.N)
     with api.Context(p) as c:
@@ -98,7 +99,7 @@ def test_profile_counts_one_launch_per_level():
         c.profile(2)
         got = c.grad(phi)
         prof = c.profile_read()
-    assert prof["nest_up"][1] == prof["nest_down"][1] == 5 and prof["update"][1] == 0
+    assert prof["nest_up"][1] == 1 and prof["nest_down"][1] == 0 and prof["update"][1] == 0
     assert prof["nest_up"][0] > 0.0 and got[0] == ref[0] and np.array_equal(got[1], ref[1])
 
 
