@@ -2473,25 +2473,41 @@ __global__ void __launch_bounds__(256)
 // (all at the phi the gradient was taken at) [5] number of updates applied (accumulates).
 // slots (optional): the workspace slot of each of the B blocks, in block order.
 constexpr int RT = 1024;
-// g_i = 2 phi_i / U - 2T sum_b gd[slot(b), i], b ascending, one thread per site: the B-term
-// sums are float64 chains (a slow pipe on this GPU), so they are spread over N / 128 CTAs
-// instead of the single reduction CTA.  slots (optional): the workspace slot of each block.
+// g_i = 2 phi_i / U - 2T sum_b gd[slot(b), i]: 32 sites per CTA, lane = site, warp y the blocks
+// y, y + 16, ..., in four running sums each (64 partial sums, added in a fixed order).  One thread
+// per site adding all B terms in turn was a chain of B loads and float64 adds (a slow pipe on this
+// GPU); with that and the chain of log-dets in k_reduce the two launches took 105 us at 20x20 with
+// 512 blocks, now 28.  slots (optional): the workspace slot of each block.
+constexpr int kSumWarps = 16;
 __device__ __forceinline__ void grad_sites(int N, int B, const int* slots, const double* gd,
                                            const double* phi, double U, double T, double* g_out) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= N) return;
-  double acc = 0.0;
-  for (int b = 0; b < B; ++b) acc += gd[(size_t)(slots ? slots[b] : b) * N + i];
-  g_out[i] = 2.0 * phi[i] / U - 2.0 * T * acc;
+  __shared__ double part[kSumWarps][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int i = blockIdx.x * 32 + lane, ic = min(i, N - 1);
+  double acc[4] = {0.0, 0.0, 0.0, 0.0};
+  for (int b0 = warp; b0 < B; b0 += 4 * kSumWarps)
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int b = b0 + u * kSumWarps;
+      if (b < B) acc[u] += gd[(size_t)(slots ? slots[b] : b) * N + ic];
+    }
+  part[warp][lane] = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+  __syncthreads();
+  if (warp == 0 && i < N) {
+    double sum = 0.0;
+#pragma unroll
+    for (int y = 0; y < kSumWarps; ++y) sum += part[y][lane];
+    g_out[i] = 2.0 * phi[i] / U - 2.0 * T * sum;
+  }
 }
 
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(32 * kSumWarps)
     k_grad_sites(int N, int B, const double* gd, const double* phi, double U, double T,
                  double* g_out) {
   grad_sites(N, B, nullptr, gd, phi, U, T, g_out);
 }
 
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(32 * kSumWarps)
     k_grad_sites_batch(int N, const ReqDesc* rq, const double* gd) {
   const ReqDesc r = rq[blockIdx.y];
   grad_sites(N, r.nblocks, r.slots, gd, r.phi, r.U, r.T, r.g);
@@ -2502,12 +2518,15 @@ __device__ __forceinline__ void reduce_body(
     const double* phi, double* phi_out, double* m, double* v, double* g_out, double* omega_out,
     double* status, const int* flags, double U, double T, int want_grad, int do_adam,
     double step, double sbc2, double beta1, double beta2, double eps, double grad_tol) {
-  __shared__ double s_q[RT], s_gm[RT], s_st[RT], s_ab[RT];
+  __shared__ double s_q[RT], s_gm[RT], s_st[RT], s_ab[RT], s_ld[RT];
   __shared__ int s_bad;
   const int tid = threadIdx.x;
   if (tid == 0) s_bad = 0;
-  double q = 0.0, gm = 0.0, st = 0.0, ab = 0.0;
+  double q = 0.0, gm = 0.0, st = 0.0, ab = 0.0, sl = 0.0;
   bool bad = false;
+  // ln|det| of all blocks, in the same fixed-order tree as the rest (one thread adding them in
+  // turn waited for B loads one after another)
+  for (int b = tid; b < B; b += RT) sl += ld[slots ? slots[b] : b];
   for (int i = tid; i < N; i += RT) {
     const double ph = phi[i];
     const int x = i / L, y = i - x * L;
@@ -2520,24 +2539,23 @@ __device__ __forceinline__ void reduce_body(
       gm = fmax(gm, fabs(g));
     }
   }
-  s_q[tid] = q; s_gm[tid] = gm; s_st[tid] = st; s_ab[tid] = ab;
+  s_q[tid] = q; s_gm[tid] = gm; s_st[tid] = st; s_ab[tid] = ab; s_ld[tid] = sl;
   __syncthreads();
   if (bad) atomicOr(&s_bad, 1);
-  for (int h = RT / 2; h > 0; h >>= 1) {
+  int top = RT / 2;  // threads past the sites and blocks hold zeros
+  while (top > 1 && top >= N && top >= B) top >>= 1;
+  for (int h = top; h > 0; h >>= 1) {
     if (tid < h) {
       s_q[tid] += s_q[tid + h];
       s_gm[tid] = fmax(s_gm[tid], s_gm[tid + h]);
       s_st[tid] += s_st[tid + h];
       s_ab[tid] += s_ab[tid + h];
+      s_ld[tid] += s_ld[tid + h];
     }
     __syncthreads();
   }
   __shared__ double s_om;
-  if (tid == 0) {
-    double sld = 0.0;
-    for (int b = 0; b < B; ++b) sld += ld[slots ? slots[b] : b];
-    s_om = s_q[0] / U - 2.0 * T * sld;
-  }
+  if (tid == 0) s_om = s_q[0] / U - 2.0 * T * s_ld[0];
   __syncthreads();
   const double om = s_om;
   const bool nonfinite = s_bad || !isfinite(om) || (flags && *flags);
@@ -3259,7 +3277,7 @@ sca_status run_reduce(Engine& e, const double* d_phi, double* d_omega, double* d
   double* g = d_grad ? d_grad : e.d_g;
   prof_begin(e, kReduce, s);
   if (want_grad) {
-    k_grad_sites<<<(e.N + 127) / 128, 128, 0, s>>>(e.N, e.B, e.gd, d_phi, e.p.U, e.p.T, g);
+    k_grad_sites<<<(e.N + 31) / 32, 32 * kSumWarps, 0, s>>>(e.N, e.B, e.gd, d_phi, e.p.U, e.p.T, g);
     SCA_LAUNCH_CHECK("gradient sums");
   }
   k_reduce<<<1, RT, 0, s>>>(e.N, e.L, e.B, e.ld, e.gd, d_phi, adam ? e.d_phi : nullptr, e.d_m,
@@ -3275,7 +3293,7 @@ sca_status run_reduce(Engine& e, const double* d_phi, double* d_omega, double* d
 
 sca_status run_reduce_batch(Engine& e, const ReqDesc* rq, int nreq, cudaStream_t s) {
   prof_begin(e, kReduce, s);
-  k_grad_sites_batch<<<dim3((e.N + 127) / 128, nreq), 128, 0, s>>>(e.N, rq, e.gd);
+  k_grad_sites_batch<<<dim3((e.N + 31) / 32, nreq), 32 * kSumWarps, 0, s>>>(e.N, rq, e.gd);
   SCA_LAUNCH_CHECK("gradient sums");
   k_reduce_batch<<<nreq, RT, 0, s>>>(e.N, e.L, rq, e.ld, e.gd, e.flags);
   prof_end(e, kReduce, s);

@@ -51,21 +51,26 @@ __global__ void __launch_bounds__(MT)
                    double* __restrict__ phi, double* __restrict__ metro, const int* flags,
                    double U, double T, unsigned long long seed, long long step, int init,
                    double* trace) {
-  __shared__ double s_q[MT];
+  __shared__ double s_q[MT], s_ld[MT];
   __shared__ int s_acc;
   const int tid = threadIdx.x;
-  double q = 0.0;
+  double q = 0.0, sl = 0.0;
   for (int i = tid; i < N; i += MT) q += prop[i] * prop[i];
+  for (int b = tid; b < B; b += MT) sl += ld[b];
   s_q[tid] = q;
+  s_ld[tid] = sl;
   __syncthreads();
-  for (int h = MT / 2; h > 0; h >>= 1) {
-    if (tid < h) s_q[tid] += s_q[tid + h];
+  int top = MT / 2;  // threads past the sites and blocks hold zeros
+  while (top > 1 && top >= N && top >= B) top >>= 1;
+  for (int h = top; h > 0; h >>= 1) {
+    if (tid < h) {
+      s_q[tid] += s_q[tid + h];
+      s_ld[tid] += s_ld[tid + h];
+    }
     __syncthreads();
   }
   if (tid == 0) {
-    double sld = 0.0;
-    for (int b = 0; b < B; ++b) sld += ld[b];
-    const double om2 = s_q[0] / U - 2.0 * T * sld;
+    const double om2 = s_q[0] / U - 2.0 * T * s_ld[0];
     const bool finite = isfinite(om2) && !(flags && *flags);
     int acc;
     if (init) {
