@@ -35,7 +35,7 @@
  *  - A context is not thread-safe; use one per thread.  A server is safe for
  *    concurrent sca_submit / sca_poll from several threads.
  *  - Elimination.  Every evaluation eliminates all 2 n_omega blocks A_{n,sigma} exactly.  From
- *    L = 8 up, and while pi T >= 0.03 |t| (for a density of states: eta >= 0.03 |t|), it goes
+ *    L = 6 up, and while pi T >= 0.03 |t| (for a density of states: eta >= 0.03 |t|), it goes
  *    through the lattice's sparsity: nested dissection of the torus, then the entries of
  *    A^{-1} inside the fronts, in float64 (SCA_PREC_FP64) or double-float (48 bits, the other
  *    three).  Below that line, for smaller lattices, and where the caller asks for it

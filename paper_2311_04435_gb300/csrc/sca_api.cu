@@ -226,7 +226,7 @@ sca_status allocate(Engine& e) {
 #define SCA_ALLOC(ptr, bytes, what) \
   if ((st = dev_alloc(&(ptr), (bytes), e, what)) != SCA_OK) return st;
   // Blocks, F and W in one allocation.  The nested elimination's fronts take the blocks' place;
-  // at 8 x 8 sites they need more than the float32 blocks and run into F and W, which hold no
+  // up to 8 x 8 sites they need more than the float32 blocks and run into F and W, which hold no
   // zero padding there (one elimination step: the whole block is its pivot block).
   const size_t mbytes = round_up((size_t)e.chunk * e.mat_stride * S, 1024);
   const size_t fbytes = round_up((size_t)e.chunk * e.fw_mat * S, 1024);

@@ -88,6 +88,30 @@ __device__ __forceinline__ dsf ds_of(double v) {
   return {h, (float)(v - (double)h)};
 }
 
+// 1 / m for finite m > 0: a float32 reciprocal and two Newton steps, 4 float64 instructions where
+// a division takes some 15 and conversions two more of the slow pipe (the conversions are shifts
+// of the bits here; outside float32's normal range: the division).
+__device__ __forceinline__ double recip(double m) {
+  const int hi = __double2hiint(m), lo = __double2loint(m), ex = (hi >> 20) - 1023;
+  if (ex < -120 || ex > 120) return 1.0 / m;
+  const float q = __frcp_rn(__int_as_float(((ex + 127) << 23) | ((hi & 0xfffff) << 3) |
+                                           ((unsigned)lo >> 29)));
+  const int qb = __float_as_int(q);
+  double d = __hiloint2double((((qb >> 23) + 896) << 20) | ((qb >> 3) & 0xfffff), qb << 29);
+  d = fma(d, fma(-m, d, 1.0), d);
+  return fma(d, fma(-m, d, 1.0), d);
+}
+
+// m into [1, 2), its exponent added to e (m > 0, finite).
+__device__ __forceinline__ void det_norm(double& m, int& e) {
+  if (m < 0x1p-1000) {  // subnormal range
+    m *= 0x1p200;
+    e -= 200;
+  }
+  const int hi = __double2hiint(m);
+  e += ((hi >> 20) & 0x7ff) - 1023;
+  m = __hiloint2double((hi & 0x800fffff) | 0x3ff00000, __double2loint(m));
+}
 
 // sum_k 0.5 ln(mag2[k]) over k < n: logs in parallel, then a pairwise reduction in a fixed
 // order (deterministic); every thread gets the sum.  Flags non-positive / non-finite moduli.

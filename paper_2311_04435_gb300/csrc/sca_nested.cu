@@ -156,15 +156,7 @@ __device__ __forceinline__ Z zmul(Z a, Z b) {
 // 1 / z, and |z|^2 in float64.
 __device__ __forceinline__ Zd zinv(Zd z, double* mag2 = nullptr) {
   const double m = z.re * z.re + z.im * z.im;
-  const float mf = (float)m;
-  double d;
-  if (mf > 1e-37f && mf < 1e37f) {  // float32 reciprocal and two Newton steps: 6 float64
-    d = (double)__frcp_rn(mf);      // instructions where a division takes some 15
-    d = fma(d, fma(-m, d, 1.0), d);
-    d = fma(d, fma(-m, d, 1.0), d);
-  } else {
-    d = 1.0 / m;
-  }
+  const double d = recip(m);
   if (mag2) *mag2 = m;
   return {z.re * d, -z.im * d};
 }
@@ -192,15 +184,6 @@ struct alignas(16) Det {
   double mant;
   int exp, pad;
 };
-__device__ __forceinline__ void det_norm(double& m, int& e) {
-  if (m < 0x1p-1000) {  // subnormal range
-    m *= 0x1p200;
-    e -= 200;
-  }
-  const int hi = __double2hiint(m);
-  e += ((hi >> 20) & 0x7ff) - 1023;
-  m = __hiloint2double((hi & 0x800fffff) | 0x3ff00000, __double2loint(m));
-}
 // Product over the warp's lanes of m2 (1.0 where a lane has none), in a fixed order, times
 // (mant, exp); flags non-positive or non-finite moduli.
 __device__ __forceinline__ void det_mul(double m2, double& mant, int& exp, int* flags) {

@@ -32,7 +32,7 @@
 namespace sca {
 namespace nested {
 
-constexpr int kMinL = 8;        // smallest lattice the tree is built for
+constexpr int kMinL = 6;        // smallest lattice the tree is built for
 // A leaf's region: a 4 x 4 leaf has 8 blacks and 8 pivots (or 16 pivots) under 16 boundary sites.
 constexpr int kLeafSites = 20;
 // Widest panel of a front of m variables: F12 and X of a panel, 2 w (m - w) entries of 16 bytes,

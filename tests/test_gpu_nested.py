@@ -1,4 +1,4 @@
-"""The nested elimination (the path of a new context from 8 x 8 sites up) against the dense pivoted
+"""The nested elimination (the path of a new context from 6 x 6 sites up) against the dense pivoted
 elimination of the same context and the FP64 oracle.
 
 Tolerances: float64 1e-11 (the oracle's dense LU and both GPU paths are good to a few hundred
@@ -22,7 +22,7 @@ def _oparams(p):
 # trees of every depth up to eight levels; fronts of one and several panels; leaves of 1 to 20
 # sites, odd and even sides, in both forms (omega_0 and omega_1 below 4t, the others above)
 @pytest.mark.parametrize("prec", ["fp64", "fp32", "bf16x3"])
-@pytest.mark.parametrize("L", [8, 10, 12, 14, 16, 18, 22, 24, 34])
+@pytest.mark.parametrize("L", [6, 8, 10, 12, 14, 16, 18, 22, 24, 34])
 def test_blocks_match_dense_elimination_and_oracle(L, prec):
     p = api.Params(L, 4, U=4.0, T=0.3, delta=0.9, mu=0.2, t=0.8, prec=prec, ionic="half")
     phi = inputs.random_phi(200 + L, p.N, 1.0)
