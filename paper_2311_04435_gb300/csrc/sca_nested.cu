@@ -19,9 +19,11 @@
 // callers with Im z below kNestedMinImag |t| take the pivoted dense elimination (nested_rule).
 //
 // Arithmetic: float64, or on the reduced-precision paths double-float (an unevaluated sum of two
-// float32, 48 bits): products exact by FMA, sums by two-sums, 12 float32 instructions per real
-// multiply-add.  This GPU does 64 float32 FMAs in the time of one float64 FMA, so double-float is
-// 5 times as fast as float64 and keeps 24 bits more than the float32 blocks of the dense paths.
+// float32, 48 bits): products exact by FMA, sums by two-sums, 12 float32 operations per real
+// multiply-add, two of them per instruction (real and imaginary part side by side: 20x20 with 512
+// blocks 1150 to 1080 us per gradient, 40x40 with 256 3794 to 3490, 64x64 with 128 8281 to 7360).
+// This GPU does 64 float32 FMAs in the time of one float64 FMA, so double-float is 5 times as
+// fast as float64 and keeps 24 bits more than the float32 blocks of the dense paths.
 //
 // Work split: a group of threads per front (a warp for the smallest, 256 or 512 threads for the
 // largest), fronts in global memory (a block's take 3.2 MB at N = 1600), the current panel of at
@@ -31,7 +33,7 @@
 // dense leaves run beside the others on a second stream.  Microseconds per gradient, one launch
 // against one per level: 16x16 with 64 blocks 176 / 254, 24x24 with 128 578 / 687, 32x32 with 128
 // 1100 / 1217, 64x64 with 128 7850 / 8281; 20x20 with 512 blocks 1313 / 1150, float64 2892 / 2429,
-// 40x40 with 256 5766 / 3570.  An entry's arithmetic is the same in every split: results do not
+// 40x40 with 256 5766 / 3570 (all before the packed instructions, which took 4 to 11 % off).  An entry's arithmetic is the same in every split: results do not
 // depend on it.
 //
 // What bounds it: float64, the float64 pipe (80 % active at 20x20: 2.1 times the instructions that
@@ -59,32 +61,69 @@ using nested::Node;
 struct alignas(16) Zd {
   double re, im;
 };
-struct alignas(16) Zf {  // re = rh + rl, im = ih + il
-  float rh, rl, ih, il;
+struct alignas(16) Zf {  // re = rh + rl, im = ih + il: two pairs for the packed instructions
+  float rh, ih, rl, il;
 };
 
-// Running sums: float64, or a float32 sum with the sum of its rounding errors.
+// Running sums of products a b: float64, or float32 sums s with the sums c of their rounding
+// errors, two to a register pair.  Af holds (re, im); Aw holds (a.re, a.im) b.re in (s1, c1) and
+// (a.re, a.im) b.im in (s2, c2), so that a is used as it is loaded and only b, which the rows of a
+// thread share, is spread over pairs: for the long sums, as its result takes more to put together.
 struct Ad {
   double re, im;
 };
+using f2 = unsigned long long;  // two float32 in a register pair
 struct Af {
-  float rs, rc, is, ic;
+  f2 s, c;
 };
+struct Aw {
+  f2 s1, c1, s2, c2;
+};
+__device__ __forceinline__ f2 f2_of(float lo, float hi) {
+  f2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void f2_get(f2 a, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(a));
+}
+__device__ __forceinline__ f2 f2_mul(f2 a, f2 b) {
+  f2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f2 f2_add(f2 a, f2 b) {
+  f2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f2 f2_sub(f2 a, f2 b) {
+  f2 r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f2 f2_fma(f2 a, f2 b, f2 c) {
+  f2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
 template <typename Z>
 struct AccOf;
 template <>
 struct AccOf<Zd> {
   using type = Ad;
+  using wide = Ad;
 };
 template <>
 struct AccOf<Zf> {
   using type = Af;
+  using wide = Aw;
 };
 
 __device__ __forceinline__ void zset(Zd& z, double re, double im) { z = {re, im}; }
 __device__ __forceinline__ void zset(Zf& z, double re, double im) {
   const dsf a = ds_of(re), b = ds_of(im);
-  z = {a.h, a.l, b.h, b.l};
+  z = {a.h, b.h, a.l, b.l};
 }
 __device__ __forceinline__ void zset0(Zd& z) { z = {0.0, 0.0}; }
 __device__ __forceinline__ void zset0(Zf& z) { z = {0.f, 0.f, 0.f, 0.f}; }
@@ -93,33 +132,50 @@ __device__ __forceinline__ double zim(Zd z) { return z.im; }
 __device__ __forceinline__ double zre(Zf z) { return (double)z.rh + (double)z.rl; }
 __device__ __forceinline__ double zim(Zf z) { return (double)z.ih + (double)z.il; }
 __device__ __forceinline__ Zd zneg(Zd z) { return {-z.re, -z.im}; }
-__device__ __forceinline__ Zf zneg(Zf z) { return {-z.rh, -z.rl, -z.ih, -z.il}; }
+__device__ __forceinline__ Zf zneg(Zf z) { return {-z.rh, -z.ih, -z.rl, -z.il}; }
 __device__ __forceinline__ Zd zadd(Zd a, Zd b) { return {a.re + b.re, a.im + b.im}; }
 __device__ __forceinline__ Zf zadd(Zf a, Zf b) {
   const dsf r = ds_add({a.rh, a.rl}, {b.rh, b.rl}), i = ds_add({a.ih, a.il}, {b.ih, b.il});
-  return {r.h, r.l, i.h, i.l};
+  return {r.h, i.h, r.l, i.l};
 }
 
 __device__ __forceinline__ Zd zsel(bool c, Zd a, Zd b) {
   return {c ? a.re : b.re, c ? a.im : b.im};
 }
 __device__ __forceinline__ Zf zsel(bool c, Zf a, Zf b) {
-  return {c ? a.rh : b.rh, c ? a.rl : b.rl, c ? a.ih : b.ih, c ? a.il : b.il};
+  return {c ? a.rh : b.rh, c ? a.ih : b.ih, c ? a.rl : b.rl, c ? a.il : b.il};
 }
 __device__ __forceinline__ Zd zshfl_xor(Zd z, int off) {
   return {__shfl_xor_sync(0xffffffffu, z.re, off), __shfl_xor_sync(0xffffffffu, z.im, off)};
 }
 __device__ __forceinline__ Zf zshfl_xor(Zf z, int off) {
-  return {__shfl_xor_sync(0xffffffffu, z.rh, off), __shfl_xor_sync(0xffffffffu, z.rl, off),
-          __shfl_xor_sync(0xffffffffu, z.ih, off), __shfl_xor_sync(0xffffffffu, z.il, off)};
+  return {__shfl_xor_sync(0xffffffffu, z.rh, off), __shfl_xor_sync(0xffffffffu, z.ih, off),
+          __shfl_xor_sync(0xffffffffu, z.rl, off), __shfl_xor_sync(0xffffffffu, z.il, off)};
 }
 
 __device__ __forceinline__ void acc_of(Ad& a, Zd z) { a = {z.re, z.im}; }
-__device__ __forceinline__ void acc_of(Af& a, Zf z) { a = {z.rh, z.rl, z.ih, z.il}; }
+__device__ __forceinline__ void acc_of(Af& a, Zf z) {
+  a = {f2_of(z.rh, z.ih), f2_of(z.rl, z.il)};
+}
 __device__ __forceinline__ Zd acc_get(Ad a) { return {a.re, a.im}; }
 __device__ __forceinline__ Zf acc_get(Af a) {
-  const dsf r = two_sum(a.rs, a.rc), i = two_sum(a.is, a.ic);
-  return {r.h, r.l, i.h, i.l};
+  float rs, rc, is, ic;
+  f2_get(a.s, rs, is);
+  f2_get(a.c, rc, ic);
+  const dsf r = two_sum(rs, rc), i = two_sum(is, ic);
+  return {r.h, i.h, r.l, i.l};
+}
+
+__device__ __forceinline__ Zf acc_get(Aw a) {
+  float p, q, pc, qc, u, v, uc, vc;
+  f2_get(a.s1, p, q);
+  f2_get(a.c1, pc, qc);
+  f2_get(a.s2, u, v);
+  f2_get(a.c2, uc, vc);
+  dsf r = two_sum(p, -v), i = two_sum(q, u);
+  r = two_sum(r.h, r.l + (pc - vc));
+  i = two_sum(i.h, i.l + (qc + uc));
+  return {r.h, i.h, r.l, i.l};
 }
 
 __device__ __forceinline__ void mac(Ad& s, Zd a, Zd b) {
@@ -141,11 +197,38 @@ __device__ __forceinline__ void mac1(float& s, float& c, float ah, float al, flo
   s = t;
   c = __fadd_rn(c, __fadd_rn(r, e));
 }
+// The same for both halves of a pair, in half the instructions.  A pair cannot be negated in
+// place: -p is taken apart and put together again, or, in the second form, minus b comes in.
+__device__ __forceinline__ void mac2(f2& s, f2& c, f2 ah, f2 al, f2 bh, f2 bl) {
+  const f2 p = f2_mul(ah, bh);
+  float p0, p1;
+  f2_get(p, p0, p1);
+  f2 e = f2_fma(ah, bh, f2_of(-p0, -p1));
+  e = f2_fma(ah, bl, e);
+  e = f2_fma(al, bh, e);
+  const f2 t = f2_add(s, p), z = f2_sub(t, s);
+  const f2 r = f2_add(f2_sub(s, f2_sub(t, z)), f2_sub(p, z));
+  s = t;
+  c = f2_add(c, f2_add(r, e));
+}
 __device__ __forceinline__ void mac(Af& s, Zf a, Zf b) {
-  mac1(s.rs, s.rc, a.rh, a.rl, b.rh, b.rl);
-  mac1(s.is, s.ic, a.rh, a.rl, b.ih, b.il);
-  mac1(s.rs, s.rc, -a.ih, -a.il, b.ih, b.il);
-  mac1(s.is, s.ic, a.ih, a.il, b.rh, b.rl);
+  mac2(s.s, s.c, f2_of(a.rh, a.rh), f2_of(a.rl, a.rl), f2_of(b.rh, b.ih), f2_of(b.rl, b.il));
+  mac2(s.s, s.c, f2_of(a.ih, a.ih), f2_of(a.il, a.il), f2_of(-b.ih, b.rh), f2_of(-b.il, b.rl));
+}
+__device__ __forceinline__ void mac2(f2& s, f2& c, f2 ah, f2 al, f2 bh, f2 nbh, f2 nbl) {
+  const f2 p = f2_mul(ah, bh);
+  f2 e = f2_fma(ah, nbh, p);  // minus the rest of the product
+  e = f2_fma(ah, nbl, e);
+  e = f2_fma(al, nbh, e);
+  const f2 t = f2_add(s, p), z = f2_sub(t, s);
+  const f2 r = f2_add(f2_sub(s, f2_sub(t, z)), f2_sub(p, z));
+  s = t;
+  c = f2_add(c, f2_sub(r, e));
+}
+__device__ __forceinline__ void mac(Aw& s, Zf a, Zf b) {
+  const f2 ah = f2_of(a.rh, a.ih), al = f2_of(a.rl, a.il);
+  mac2(s.s1, s.c1, ah, al, f2_of(b.rh, b.rh), f2_of(-b.rh, -b.rh), f2_of(-b.rl, -b.rl));
+  mac2(s.s2, s.c2, ah, al, f2_of(b.ih, b.ih), f2_of(-b.ih, -b.ih), f2_of(-b.il, -b.il));
 }
 template <typename Z>
 __device__ __forceinline__ Z zmul(Z a, Z b) {
@@ -174,7 +257,7 @@ __device__ __forceinline__ Zf zinv(Zf z, double* mag2 = nullptr) {
   mac1(rs, rc, z.rh, z.rl, q, ql);
   mac1(is, ic, -z.ih, -z.il, q, ql);
   const dsf r = two_sum(rs, rc), i = two_sum(is, ic);
-  return {r.h, r.l, i.h, i.l};
+  return {r.h, i.h, r.l, i.l};
 }
 
 // A product of moduli squared as mantissa in [1, 2) and exponent: a node's share of |det A|^2.
@@ -451,12 +534,16 @@ __device__ __noinline__ void update_rest(const Group gr, const Front<Z>& f, bool
 
 // Y = X R (w x r, inner length n): one column and KR rows per thread, the rows nrb apart, X (row
 // stride ldx) broadcast from shared memory, R (row stride step) from shared or global memory (L1
-// and L2 hold it).  kGlobal: R is Rg, in global memory; else at Ro, and the rows of Y go to Yg (row
-// stride m) too.  kMap: R's rows and columns go through map (R in the parent's front).
-template <typename Z, int KR, bool kMap, bool kGlobal>
+// and L2 hold it).  kAhead > 0: R is Rg, in global memory, read kAhead rows ahead; else at Ro, and
+// the rows of Y go to Yg (row stride m) too.  Four rows ahead where a CTA of 512 threads has the SM
+// to itself (64x64: 7.6 ms with two, 7.3 with four, 7.2 with six, which costs 12x12 and densities
+// of states 1.5 %), two where four CTAs of 256 share it (64 registers).  kMap: R's rows and columns
+// go through map (R in the parent's front).
+template <typename Z, int KR, bool kMap, int kAhead>
 __device__ __noinline__ void times(const Group gr, int w, int n, int r, int Xo, int ldx, int Yo,
                                    int ldy, const Z* Rg, int Ro, int step, int mapo, Z* Yg, int m) {
-  using Acc = typename AccOf<Z>::type;
+  constexpr bool kGlobal = kAhead > 0;
+  using Acc = std::conditional_t<(kAhead > 0), typename AccOf<Z>::wide, typename AccOf<Z>::type>;
   extern __shared__ __align__(16) unsigned char smem[];
   const Z* X = reinterpret_cast<const Z*>(smem + Xo);
   Z* Y = reinterpret_cast<Z*>(smem + Yo);
@@ -474,27 +561,31 @@ __device__ __noinline__ void times(const Group gr, int w, int n, int r, int Xo, 
       Xi[u] = min(b + u * nrb, w - 1) * ldx;
     }
     const int jj = kMap ? map[j] : j;
-    if constexpr (kGlobal) {  // two rows ahead
+    if constexpr (kGlobal) {
       auto load = [&](int k) {
         k = min(k, n - 1);
         return Rg[(kMap ? map[k] : k) * step + jj];
       };
-      Z g0 = load(0), g1 = load(1);
+      Z g[kAhead];
+#pragma unroll
+      for (int d = 0; d < kAhead; ++d) g[d] = load(d);
+      int k = 0;
 #pragma unroll 1
-      for (int k = 0; k + 1 < n; k += 2) {
-        Z g = g0;
-        g0 = load(k + 2);
+      for (; k + kAhead <= n; k += kAhead) {
 #pragma unroll
-        for (int u = 0; u < KR; ++u) mac(s[u], X[Xi[u] + k], g);
-        g = g1;
-        g1 = load(k + 3);
+        for (int d = 0; d < kAhead; ++d) {
+          const Z x = g[d];
+          g[d] = load(k + kAhead + d);
 #pragma unroll
-        for (int u = 0; u < KR; ++u) mac(s[u], X[Xi[u] + k + 1], g);
+          for (int u = 0; u < KR; ++u) mac(s[u], X[Xi[u] + k + d], x);
+        }
       }
-      if (n & 1) {
 #pragma unroll
-        for (int u = 0; u < KR; ++u) mac(s[u], X[Xi[u] + n - 1], g0);
-      }
+      for (int d = 0; d + 1 < kAhead; ++d)
+        if (k + d < n) {
+#pragma unroll
+          for (int u = 0; u < KR; ++u) mac(s[u], X[Xi[u] + k + d], g[d]);
+        }
     } else {
 #pragma unroll 2
       for (int k = 0; k < n; ++k) {
@@ -517,7 +608,7 @@ __device__ __noinline__ void times(const Group gr, int w, int n, int r, int Xo, 
 
 // The row count that fits the outputs per thread: passes over the threads, each of KR products and
 // about a third of a product's overhead.
-template <typename Z, bool kMap, bool kGlobal>
+template <typename Z, bool kMap, int kAhead>
 __device__ __forceinline__ void times_fit(const Group& gr, int w, int n, int r, int Xo, int ldx,
                                           int Yo, int ldy, const Z* Rg, int Ro, int step, int mapo,
                                           Z* Yg, int m) {
@@ -525,9 +616,9 @@ __device__ __forceinline__ void times_fit(const Group& gr, int w, int n, int r, 
     return ((w + kr - 1) / kr * r + gr.size - 1) / gr.size * (3 * kr + 1);
   };
   if (cost(2) <= cost(1) || kMap)
-    times<Z, 2, kMap, kGlobal>(gr, w, n, r, Xo, ldx, Yo, ldy, Rg, Ro, step, mapo, Yg, m);
+    times<Z, 2, kMap, kAhead>(gr, w, n, r, Xo, ldx, Yo, ldy, Rg, Ro, step, mapo, Yg, m);
   else
-    times<Z, 1, kMap, kGlobal>(gr, w, n, r, Xo, ldx, Yo, ldy, Rg, Ro, step, mapo, Yg, m);
+    times<Z, 1, kMap, kAhead>(gr, w, n, r, Xo, ldx, Yo, ldy, Rg, Ro, step, mapo, Yg, m);
 }
 
 // One front, up: see the file comment.  -X is kept (in the front and here), as both later products
@@ -537,7 +628,7 @@ template <typename Z>
 __device__ __forceinline__ void front_up(const Block<Z>& B, int node, const Group& gr, int at) {
   extern __shared__ __align__(16) unsigned char smem[];
   using Acc = typename AccOf<Z>::type;
-  const int tid = gr.tid, NT = gr.size;
+  const int tid = gr.tid, size = gr.size;
   const Node nd = B.nodes[node];
   const int p = nd.p, m = nd.p + nd.q, pw = nd.pw;
   Z* F = B.fronts + nd.front;
@@ -555,17 +646,17 @@ __device__ __forceinline__ void front_up(const Block<Z>& B, int node, const Grou
   int16_t* adj = cm1 + m;
   double mant = 1.0;  // first warp: the node's share of |det A|^2
   int expo = 0;
-  for (int i = tid; i < m; i += NT) {
+  for (int i = tid; i < m; i += size) {
     const int s = B.tab[nd.sites + i], x = s / B.la.L;
     site[i] = (int16_t)((x << 8) | (s - x * B.la.L));
     cm0[i] = nd.child[0] >= 0 ? B.tab[nd.cmap[0] + i] : (int16_t)-1;
     cm1[i] = nd.child[1] >= 0 ? B.tab[nd.cmap[1] + i] : (int16_t)-1;
   }
-  for (int i = tid; i <= p; i += NT)
+  for (int i = tid; i <= p; i += size)
     zset(diag[i], i < p ? B.zr - site_energy(B.la, B.tab[nd.sites + i], B.sg) : B.la.t,
          i < p ? B.zi : 0.0);
   if (nd.blacks) {
-    for (int i = tid; i < m; i += NT) adj[i] = B.tab[nd.adj + i];
+    for (int i = tid; i < m; i += size) adj[i] = B.tab[nd.adj + i];
     if (tid < 32) {
       double m2 = 1.0;
       if (tid < nd.blacks) {
@@ -602,7 +693,7 @@ __device__ __forceinline__ void front_up(const Block<Z>& B, int node, const Grou
     const int o = pa * pw, w = min(pw, p - o), l = m - o, r = l - w;
     const int lda = r + kRows;  // row blocks read up to kRows - 1 entries past r
     // ---- the panel to shared memory (F12 stays there), then to the registers
-    for (int i = tid >> 5; i < w; i += NT >> 5)
+    for (int i = tid >> 5; i < w; i += size >> 5)
 #pragma unroll 2
       for (int j = tid & 31; j < l; j += 32) {
         const int hi = max(i, j) + o, lo = min(i, j) + o;
@@ -614,13 +705,13 @@ __device__ __forceinline__ void front_up(const Block<Z>& B, int node, const Grou
       }
     gr.sync();
     Z* Fo = F + (size_t)o * (m + 1);
-    if (w <= NT / w)
+    if (w <= size / w)
       invert<Z, 1>(gr, w, off(F11), off(rowb), off(colb), off(mag), Fo, m);
     else
       invert<Z, kSlots>(gr, w, off(F11), off(rowb), off(colb), off(mag), Fo, m);
     gr.sync();
     if (r > 0)
-      times_fit<Z, false, false>(gr, w, w, r, off(F11), w, off(X), r, (const Z*)F, off(A), lda, 0,
+      times_fit<Z, false, 0>(gr, w, w, r, off(F11), w, off(X), r, (const Z*)F, off(A), lda, 0,
                                  Fo + w, m);
     gr.sync();
     if (tid < 32) det_mul(tid < w ? mag[tid] : 1.0, mant, expo, B.flags);
@@ -628,7 +719,7 @@ __device__ __forceinline__ void front_up(const Block<Z>& B, int node, const Grou
     Z* R = F + (size_t)(o + w) * (m + 1);
     auto cost = [&](int kr) {
       const int nb = (r + kr - 1) / kr;
-      return (kr * nb * (nb + 1) / 2 + NT - 1) / NT * (3 * kr + 1);
+      return (kr * nb * (nb + 1) / 2 + size - 1) / size * (3 * kr + 1);
     };
     if (cost(2) <= cost(1))
       update_rest<Z, 2>(gr, f, pa == 0, o + w, w, r, m, off(A), lda, off(X), R);
@@ -641,11 +732,11 @@ __device__ __forceinline__ void front_up(const Block<Z>& B, int node, const Grou
 
 // One front, down.  Panels in reverse; R is the part of the front after the panel, already G.  A
 // node without children keeps nothing but its own rows: R is then read from the parent's front.
-template <typename Z>
+template <typename Z, int NT>
 __device__ __forceinline__ void front_down(const Block<Z>& B, int node, const Group& gr, int at) {
   extern __shared__ __align__(16) unsigned char smem[];
   using Acc = typename AccOf<Z>::type;
-  const int tid = gr.tid, NT = gr.size;
+  const int tid = gr.tid, size = gr.size;
   const Node nd = B.nodes[node];
   const int p = nd.p, q = nd.q, m = nd.p + nd.q;
   Z* F = B.fronts + nd.front;
@@ -661,11 +752,11 @@ __device__ __forceinline__ void front_down(const Block<Z>& B, int node, const Gr
     const Node pr = B.nodes[nd.parent];
     mp = pr.p + pr.q;
     G = B.fronts + pr.front;
-    for (int i = tid; i < q; i += NT) map[i] = B.tab[nd.pmap + i];
+    for (int i = tid; i < q; i += size) map[i] = B.tab[nd.pmap + i];
     gr.sync();
     if (!direct) {
       // G_bb into the front, several entries in flight per thread
-      for (int i = tid >> 5; i < q; i += NT >> 5) {
+      for (int i = tid >> 5; i < q; i += size >> 5) {
         const Z* Gi = G + map[i] * mp;
         Z* Fi = F + (p + i) * m + p;
         for (int j0 = tid & 31; j0 < q; j0 += 128) {
@@ -683,18 +774,18 @@ __device__ __forceinline__ void front_down(const Block<Z>& B, int node, const Gr
   for (int pa = nd.npan - 1; pa >= 0; --pa) {
     const int o = pa * nd.pw, w = min(nd.pw, p - o), r = m - o - w;
     const Z* R = F + (size_t)(o + w) * (m + 1);
-    for (int i = tid >> 5; i < w; i += NT >> 5)
+    for (int i = tid >> 5; i < w; i += size >> 5)
       for (int j = tid & 31; j < r; j += 32) X[i * ldx + j] = F[(o + i) * m + o + w + j];
     gr.sync();
     if (direct)
-      times_fit<Z, true, true>(gr, w, r, r, off(X), ldx, off(Y), ldx, G, 0, mp, off(map), (Z*)nullptr, 0);
+      times_fit<Z, true, NT == 512 ? 4 : 2>(gr, w, r, r, off(X), ldx, off(Y), ldx, G, 0, mp, off(map), (Z*)nullptr, 0);
     else if (r > 0)
-      times_fit<Z, false, true>(gr, w, r, r, off(X), ldx, off(Y), ldx, R, 0, m, 0, (Z*)nullptr, 0);
+      times_fit<Z, false, NT == 512 ? 4 : 2>(gr, w, r, r, off(X), ldx, off(Y), ldx, R, 0, m, 0, (Z*)nullptr, 0);
     gr.sync();
     // ---- G_pp = P + Y (-X)^T, lower triangle; ks threads share an entry's sum (by the front's
     // shape alone: the order of a sum must not depend on how many threads there are)
     const int outs = w * (w + 1) / 2, ks = r >= 48 ? 4 : 2;
-    for (int e0 = 0; e0 < outs; e0 += NT / ks) {
+    for (int e0 = 0; e0 < outs; e0 += size / ks) {
       const int e = min(e0 + tid / ks, outs - 1), k0 = tid % ks;
       int i, j;
       triangle(e, i, j);
@@ -716,9 +807,9 @@ __device__ __forceinline__ void front_down(const Block<Z>& B, int node, const Gr
       }
     }
     if (!direct) {
-      for (int i = tid >> 5; i < w; i += NT >> 5)
+      for (int i = tid >> 5; i < w; i += size >> 5)
         for (int j = tid & 31; j < r; j += 32) F[(o + i) * m + o + w + j] = Y[i * ldx + j];
-      for (int j = tid >> 4; j < r; j += NT >> 4)
+      for (int j = tid >> 4; j < r; j += size >> 4)
         for (int i = tid & 15; i < w; i += 16) F[(o + w + j) * m + o + i] = Y[i * ldx + j];
     }
     gr.sync();
@@ -726,7 +817,7 @@ __device__ __forceinline__ void front_down(const Block<Z>& B, int node, const Gr
   // blacks: G_bb = 1/a + (t/a)^2 sum_{u,v} G_uv over the black's neighbours, four threads each
   // (one neighbour u per thread); such leaves have one panel
   if (nd.blacks) {
-    for (int b0 = 0; b0 < nd.blacks; b0 += NT / 4) {
+    for (int b0 = 0; b0 < nd.blacks; b0 += size / 4) {
       const int b = min(b0 + tid / 4, nd.blacks - 1), u = tid & 3;
       const int s = B.tab[nd.bsite + b];
       const int iu = B.tab[nd.bnbr + 4 * b + u];
@@ -802,7 +893,7 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : 1) k_nested(NestArgs<Z> a)
       if (up)
         front_up(B, lv.first + f, gr, at);
       else
-        front_down(B, lv.first + f, gr, at);
+        front_down<Z, NT>(B, lv.first + f, gr, at);
     }
     if (k + 1 == a.k1 && k != a.nlevels - 1) break;
     block_sync<kCluster>();
