@@ -33,13 +33,15 @@
 // dense leaves run beside the others on a second stream.  Microseconds per gradient, one launch
 // against one per level: 16x16 with 64 blocks 176 / 254, 24x24 with 128 578 / 687, 32x32 with 128
 // 1100 / 1217, 64x64 with 128 7850 / 8281; 20x20 with 512 blocks 1313 / 1150, float64 2892 / 2429,
-// 40x40 with 256 5766 / 3570 (all before the packed instructions, which took 4 to 11 % off).  An entry's arithmetic is the same in every split: results do not
-// depend on it.
+// 40x40 with 256 5766 / 3570 (all before the packed instructions, which took 4 to 11 % off).  An
+// entry's arithmetic is the same in every split: results do not depend on it.
 //
 // What bounds it: float64, the float64 pipe (80 % active at 20x20: 2.1 times the instructions that
-// the products alone need, for lanes that idle at the edges of small fronts); double-float, issue
-// (IPC 2.1 of 4 with 16 warps per SM) and the dependent chain of a panel's pivots, some 1800
-// cycles per pivot, which other fronts' products overlap only in part.
+// the products alone need, for lanes that idle at the edges of small fronts); double-float, the
+// float32 pipe, busy half of the time (1.9 instructions issued per cycle, most of them packed, which
+// hold the pipe for two), the latency of reads of the parents' fronts (30 % of the downward
+// products at 64x64), and the dependent chain of a panel's pivots, some 1800 cycles per pivot,
+// which other fronts' products overlap only in part.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -537,8 +539,8 @@ __device__ __noinline__ void update_rest(const Group gr, const Front<Z>& f, bool
 // and L2 hold it).  kAhead > 0: R is Rg, in global memory, read kAhead rows ahead; else at Ro, and
 // the rows of Y go to Yg (row stride m) too.  Four rows ahead where a CTA of 512 threads has the SM
 // to itself (64x64: 7.6 ms with two, 7.3 with four, 7.2 with six, which costs 12x12 and densities
-// of states 1.5 %), two where four CTAs of 256 share it (64 registers).  kMap: R's rows and columns
-// go through map (R in the parent's front).
+// of states 1.5 %), two where four CTAs of 256 share it (64 registers; three cost 2 %).  kMap: R's
+// rows and columns go through map (R in the parent's front).
 template <typename Z, int KR, bool kMap, int kAhead>
 __device__ __noinline__ void times(const Group gr, int w, int n, int r, int Xo, int ldx, int Yo,
                                    int ldy, const Z* Rg, int Ro, int step, int mapo, Z* Yg, int m) {

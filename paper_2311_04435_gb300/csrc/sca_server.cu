@@ -38,8 +38,8 @@ namespace {
 constexpr int32_t kRoundSteps = 8;     // Adam iterations enqueued per request per round
 constexpr int kBucketSlots = 256;      // block slots of a size bucket's workspace
 // How long the workspace of a bucket that has lost its last request waits for another of its
-// size.  Allocating and freeing one takes milliseconds (L = 32: 1.9 and 4.6 ms for 128 slots,
-// against 4.5 ms for the nine evaluations of two requests); in a served mix of 12 requests of
+// size.  Allocating and freeing one takes milliseconds (L = 32, 256 slots: 1.7 and 4.5 ms,
+// against 6.3 ms for all nine evaluations of two requests); in a served mix of 12 requests of
 // six sizes that was 12 of 28 ms.
 constexpr double kIdleSeconds = 10.0;
 
