@@ -29,12 +29,14 @@
 // largest), fronts in global memory (a block's take 3.2 MB at N = 1600), the current panel of at
 // most 20 pivot rows and its X in shared memory.  Up to one block per SM the whole elimination is
 // one launch, a CTA of 512 threads per block or a cluster of them, with a barrier per tree level;
-// more blocks take one launch per level and direction, spread over the chip, and the blocks with
-// dense leaves run beside the others on a second stream.  Microseconds per gradient, one launch
+// more blocks take one launch per level and direction, spread over the chip, in parts side by side:
+// the blocks with dense leaves, and two halves of the others.  Microseconds per gradient, one launch
 // against one per level: 16x16 with 64 blocks 176 / 254, 24x24 with 128 578 / 687, 32x32 with 128
 // 1100 / 1217, 64x64 with 128 7850 / 8281; 20x20 with 512 blocks 1313 / 1150, float64 2892 / 2429,
-// 40x40 with 256 5766 / 3570 (all before the packed instructions, which took 4 to 11 % off).  An
-// entry's arithmetic is the same in every split: results do not depend on it.
+// 40x40 with 256 5766 / 3570 (all before the packed instructions, which took 4 to 11 % off, and
+// the halves; with both, dealing 128 blocks out by level still loses: 64x64 7333 / 7595, 32x32
+// 1086 / 1108, 20x20 density of states 461 / 521).  An entry's arithmetic is the same in every
+// split: results do not depend on it.
 //
 // What bounds it: float64, the float64 pipe (80 % active at 20x20: 2.1 times the instructions that
 // the products alone need, for lanes that idle at the edges of small fronts); double-float, the
@@ -291,6 +293,12 @@ __device__ __forceinline__ void det_mul(double m2, double& mant, int& exp, int* 
 // ------------------------------------------------------------------ kernels
 constexpr int kRows = nested::kRows;    // rows of a thread's output tile at most
 constexpr int kSlots = nested::kSlots;  // entries of a pivots' block that a thread holds at most
+
+// Blocks from which a launch per level takes them in two halves on two streams (20x20 with 500
+// such blocks 1072 / 1000 us per gradient in one part / in halves, float64 2413 / 2249, 40x40 with
+// 244 3478 / 3185, its potential 1628 / 1555).  A pass with a launch per level has more blocks
+// than SMs, so the line only keeps a small rest beside blocks with dense leaves in one piece.
+constexpr int kHalves = 64;
 
 // How one level's fronts are worked on: `group` threads per front, each group with `smem` bytes.
 struct LevelPlan {
@@ -962,6 +970,8 @@ struct Nested {
   long long stride = 0;   // entries per block
   int cap = 0;            // blocks per pass
   int sms = 1;
+  cudaStream_t half = nullptr;  // the second half of a pass that takes a launch per level
+  cudaEvent_t ev_half = nullptr;
 };
 
 namespace {
@@ -1045,42 +1055,58 @@ sca_status run_nested_t(Engine& e, const Lattice& la, bool up, bool down, cudaSt
     const int dense = std::min(cnt, std::max(0, e.nest_dense - b0));
     a.ndense = dense;
     if (cnt > ne.sms) {
-      // the two forms side by side: the few blocks with dense leaves on the high-priority stream
-      const bool fork = dense > 0 && dense < cnt && e.side != nullptr;
-      cudaError_t err = cudaSuccess;
-      if (fork) {
-        err = cudaEventRecord(e.ev_fork, s);
-        if (err == cudaSuccess) err = cudaStreamWaitEvent(e.side, e.ev_fork, 0);
-        if (err != cudaSuccess) return cuda_fail(err, "fork");
-      }
+      // side by side: the few blocks with dense leaves on the high-priority stream, and the others
+      // in two halves, so that one half's fronts fill the SMs that the last wave of the other's
+      // level leaves idle
+      struct Part {
+        int form, first, n, all;  // all: blocks of the form, which the group sizes follow
+        cudaStream_t s;
+        cudaEvent_t join;
+      } parts[3];
+      int nparts = 0;
+      const bool two = dense > 0 && dense < cnt && e.side != nullptr;
       for (int form = 1; form >= 0; --form) {
-        const int n = form ? dense : cnt - dense;
+        const int n = form ? dense : cnt - dense, first = form ? 0 : dense;
+        const int h = ne.half && n >= kHalves && !(form && two) ? n / 2 : 0;
         if (n == 0) continue;
-        NestArgs<Z> f = a;  // the form's blocks alone
-        f.b0 = b0 + (form ? 0 : dense);
-        f.fronts = a.fronts + (size_t)(f.b0 - b0) * a.stride;
-        f.det = a.det + (size_t)(f.b0 - b0) * a.nnodes;
-        f.ndense = form ? n : 0;
-        for (int k = p0; k < p1; ++k) {
+        if (form && two)
+          parts[nparts++] = {form, first, n, n, e.side, e.ev_join};
+        else
+          parts[nparts++] = {form, first, n - h, n, s, nullptr};
+        if (h) parts[nparts++] = {form, first + n - h, h, n, ne.half, ne.ev_half};
+      }
+      cudaError_t err = cudaSuccess;
+      if (nparts > 1) err = cudaEventRecord(e.ev_fork, s);
+      for (int i = 0; i < nparts && err == cudaSuccess; ++i)
+        if (parts[i].join) err = cudaStreamWaitEvent(parts[i].s, e.ev_fork, 0);
+      if (err != cudaSuccess) return cuda_fail(err, "fork");
+      for (int k = p0; k < p1; ++k)
+        for (int i = 0; i < nparts; ++i) {
+          const Part& pt = parts[i];
+          NestArgs<Z> f = a;  // the part's blocks alone
+          f.b0 = b0 + pt.first;
+          f.fronts = a.fronts + (size_t)pt.first * a.stride;
+          f.det = a.det + (size_t)pt.first * a.nnodes;
+          f.ndense = pt.form ? pt.n : 0;
           const int level = k < nl ? nl - 1 - k : k - nl;
           f.k0 = k;
           f.k1 = k + 1;
-          const Nested::Shape& sh = ne.levels[form][level];
+          const Nested::Shape& sh = ne.levels[pt.form][level];
           int g = sh.group;  // the fewest threads while they fill the SMs; four CTAs per SM
-          while (2 * g <= 256 && ((long long)sh.count * n * g < 1024ll * ne.sms ||
+          while (2 * g <= 256 && ((long long)sh.count * pt.all * g < 1024ll * ne.sms ||
                                   256 / g * sh.smem > 55 << 10))
             g *= 2;
-          f.lv[form][level] = {sh.first, sh.count, g, sh.smem};
+          f.lv[pt.form][level] = {sh.first, sh.count, g, sh.smem};
           f.csize = (sh.count + 256 / g - 1) / (256 / g);
-          st = launch<Z, 256, false>(e, f, n, (size_t)(256 / g) * sh.smem, form && fork ? e.side : s);
+          st = launch<Z, 256, false>(e, f, pt.n, (size_t)(256 / g) * sh.smem, pt.s);
           if (st != SCA_OK) return st;
         }
-      }
-      if (fork) {
-        err = cudaEventRecord(e.ev_join, e.side);
-        if (err == cudaSuccess) err = cudaStreamWaitEvent(s, e.ev_join, 0);
-        if (err != cudaSuccess) return cuda_fail(err, "join");
-      }
+      for (int i = 0; i < nparts && err == cudaSuccess; ++i)
+        if (parts[i].join) {
+          err = cudaEventRecord(parts[i].join, parts[i].s);
+          if (err == cudaSuccess) err = cudaStreamWaitEvent(s, parts[i].join, 0);
+        }
+      if (err != cudaSuccess) return cuda_fail(err, "join");
     } else {
       // CTAs per block: as many as there are SMs for, up to the portable cluster size
       a.k0 = p0;
@@ -1150,6 +1176,11 @@ sca_status nested_prepare(Engine& e) {
   if (err == cudaSuccess)
     err = cudaDeviceGetAttribute(&ne->sms, cudaDevAttrMultiProcessorCount, dev);
   if (err != cudaSuccess) { nested_release(e); return cuda_fail(err, "nested elimination set-up"); }
+  if (e.B > ne->sms) {
+    err = cudaStreamCreateWithFlags(&ne->half, cudaStreamNonBlocking);
+    if (err == cudaSuccess) err = cudaEventCreateWithFlags(&ne->ev_half, cudaEventDisableTiming);
+    if (err != cudaSuccess) { nested_release(e); return cuda_fail(err, "nested elimination set-up"); }
+  }
   err = cudaMalloc((void**)&ne->d_nodes, sizeof(Node) * t.nodes.size());
   if (err == cudaSuccess) err = cudaMalloc((void**)&ne->d_tab, sizeof(int16_t) * t.table.size());
   if (err != cudaSuccess) {
@@ -1167,6 +1198,11 @@ sca_status nested_prepare(Engine& e) {
 
 void nested_release(Engine& e) {
   if (!e.nest) return;
+  if (e.nest->half) {
+    cudaStreamSynchronize(e.nest->half);
+    cudaStreamDestroy(e.nest->half);
+  }
+  if (e.nest->ev_half) cudaEventDestroy(e.nest->ev_half);
   if (e.nest->d_nodes) cudaFree(e.nest->d_nodes);
   if (e.nest->d_tab) cudaFree(e.nest->d_tab);
   delete e.nest;

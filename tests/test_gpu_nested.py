@@ -118,3 +118,29 @@ def test_served_requests_on_both_sides_of_the_line():
         mixed = [srv.poll(rid, 256) for rid in ids]
     for x, y in zip(alone, mixed):
         assert x.steps == y.steps and x.omega == y.omega and np.array_equal(x.phi, y.phi)
+
+
+@pytest.mark.parametrize("L,prec,n_omega,t", [(6, "fp32", 77, 1.0), (8, "bf16x3", 110, 1.0),
+                                              (8, "fp64", 80, 8.0), (20, "bf16x3", 100, 1.0)])
+def test_more_blocks_than_sms(L, prec, n_omega, t):
+    """A launch per level, the blocks in parts side by side (with t = 8 fewer than 64 of them have
+    closed-form leaves): every block as the oracle has it, and to the bit what a pass of few
+    blocks gives; the same for a density of states, where every block has dense leaves."""
+    p = api.Params(L, n_omega, U=4.0, T=0.1, delta=0.9, t=t, prec=prec)
+    phi = inputs.random_phi(400 + L, p.N, 1.0)
+    w = np.linspace(-4.0, 4.0, 90)
+    with api.Context(p) as c:
+        ld, gd = c.blocks(phi)
+        om = c.potential(phi)
+        g = c.grad(phi)
+        rho = c.dos(phi, w, 0.3)
+    with api.Context(api.Params(L, 10, U=4.0, T=0.1, delta=0.9, t=t, prec=prec)) as c:
+        few = c.blocks(phi)
+        rho_few = np.concatenate([c.dos(phi, w[k:k + 10], 0.3) for k in range(0, 90, 10)], axis=1)
+    assert np.array_equal(ld[:20], few[0]) and np.array_equal(gd[:20], few[1])
+    assert np.array_equal(rho, rho_few) and om == g[0]
+    o_om, o_g, o_ld, o_gd = oracle.omega_grad(_oparams(p), phi, per_block=True)
+    tol = 1e-11 if prec == "fp64" else 1e-10
+    assert np.max(np.abs(gd - o_gd)) <= tol
+    assert np.max(np.abs(ld - o_ld) / np.abs(o_ld)) <= tol
+    assert om == pytest.approx(o_om, rel=tol) and np.max(np.abs(g[1] - o_g)) <= 10 * tol
