@@ -770,7 +770,7 @@ def serve_sweep(args):
         "value": round(len(ids) / wall, 4), "unit": "solves/s", "n_gpus": world,
         "steps": len(ids), "warmup": 0, "ms_per_step": round(1e3 * wall / len(ids), 2),
         "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
-        "dtype": f"f32 storage, {prec} contractions (f32 below 128 x 128), f64 refinement"
+        "dtype": "double-float (unevaluated sums of two f32)"
         if prec != "fp64" else "f64",
         "data": "synthetic (seeded Poisson trace, SplitMix64 start fields)",
         "config": {"workload": f"{len(ids)} requests, L in {{8..32}}, Poisson {args.serve_rate}/s, "

@@ -224,8 +224,8 @@ sca_status sca_solve(const sca_params* params, const sca_adam* adam, const doubl
  * fused kernel's size (N > 144; FP64: N > 64) are batched by size bucket: those
  * with the same L and precision share one workspace of up to 256 block slots
  * (counted against the budget while the bucket has requests; then kept up to 10 s,
- * within the budget, for the next one of its size) and one launch sequence per step.  A request's result is the same bit for bit as with
- * sca_solve.  Errors: SCA_EINVAL, SCA_ENOMEM, SCA_ECUDA. */
+ * within the budget, for the next one of its size) and one launch sequence per
+ * step.  A request's result is the same bit for bit as with sca_solve.  Errors: SCA_EINVAL, SCA_ENOMEM, SCA_ECUDA. */
 sca_status sca_server_create(uint64_t hbm_budget_bytes, int32_t max_slots, sca_server** out);
 
 /* Queues a solve request (parameters and Adam settings are copied; phi0 is
@@ -345,8 +345,8 @@ sca_status sca_metropolis_step(sca_ctx* ctx, int32_t n_steps, double* omega_trac
  *     dominance is not guaranteed (omega_n <= 4|t|); the remaining blocks provably keep their
  *     diagonal pivots and skip the search.
  *   SCA_PIVOT_NONE: every block is eliminated without interchanges: nested where it applies,
- *     elsewhere as a dense complex-symmetric (LDL^T-type) elimination that updates one triangle on the tensor-core path.  The paper
- *     has no such variant.  -i A_{n,sigma} has Hermitian part omega_n I > 0, so every leading
+ *     elsewhere as a dense complex-symmetric (LDL^T-type) elimination that updates one
+ *     triangle on the tensor-core path.  The paper has no such variant.  -i A_{n,sigma} has Hermitian part omega_n I > 0, so every leading
  *     principal minor is nonzero and the elimination exists; its growth has no a-priori bound
  *     and rises as omega_n falls (the largest growth met in tests is below 10, down to
  *     T = 0.02).  The fused small-block path (N <= 144) always pivots.

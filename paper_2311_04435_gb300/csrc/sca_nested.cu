@@ -1062,7 +1062,7 @@ sca_status run_nested_t(Engine& e, const Lattice& la, bool up, bool down, cudaSt
         int form, first, n, all;  // all: blocks of the form, which the group sizes follow
         cudaStream_t s;
         cudaEvent_t join;
-      } parts[3];
+      } parts[4];
       int nparts = 0;
       const bool two = dense > 0 && dense < cnt && e.side != nullptr;
       for (int form = 1; form >= 0; --form) {

@@ -214,13 +214,13 @@ def test_replayed_trace_bookkeeping_is_bit_exact():
         assert alone.steps == o[2] and np.array_equal(alone.phi, o[5]) and alone.omega == o[3]
 
 
-@pytest.mark.parametrize("budget", [8 << 30, 150 << 20])
+@pytest.mark.parametrize("budget", [8 << 30, 340 << 20])
 def test_idle_workspaces_are_reused_and_given_back(budget):
     """Waves of requests on one server: a size bucket that lost its last request serves the
     next wave (large budget), or is freed for another size (a budget that does not hold two)."""
     reqs = [(api.Params(L, 6, U=4.0, T=0.2, delta=d, prec="bf16x3"),
              api.AdamConfig(lr=0.02, grad_tol=1e-6, max_steps=20, seed=s))
-            for s, (L, d) in enumerate([(8, 0.5), (12, 1.0), (12, 0.0), (10, 0.5)])]
+            for s, (L, d) in enumerate([(14, 0.5), (16, 1.0), (16, 0.0), (18, 0.5)])]
     alone = [api.solve(p, a) for p, a in reqs]
     with api.Server(hbm_budget_bytes=budget, max_slots=4) as srv:
         for _ in range(3):
