@@ -240,9 +240,10 @@ __device__ __forceinline__ Z zmul(Z a, Z b) {
   mac(s, a, b);
   return acc_get(s);
 }
-// 1 / z, and |z|^2 in float64.
+// 1 / z, and |z|^2 in float64.  (Which of the two products goes into the FMA is written out: left
+// to the compiler it differed between the kernels, and a result's last bit with the split.)
 __device__ __forceinline__ Zd zinv(Zd z, double* mag2 = nullptr) {
-  const double m = z.re * z.re + z.im * z.im;
+  const double m = fma(z.im, z.im, __dmul_rn(z.re, z.re));
   const double d = recip(m);
   if (mag2) *mag2 = m;
   return {z.re * d, -z.im * d};
