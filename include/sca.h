@@ -38,7 +38,8 @@
  *    L = 6 up, and while pi T >= 0.03 |t| (for a density of states: eta >= 0.03 |t|), it goes
  *    through the lattice's sparsity: nested dissection of the torus, then the entries of
  *    A^{-1} inside the fronts, in float64 (SCA_PREC_FP64) or double-float (48 bits, the other
- *    three).  Below that line, for smaller lattices, and where the caller asks for it
+ *    three); blocks of small omega_n, and float64 densities of states of small eta, in sums of
+ *    three float32 (72 bits), as rounding grows there on weak fields.  Below that line, for smaller lattices, and where the caller asks for it
  *    (sca_set_pivoting, sca_set_panel_precision, sca_profile_enable(ctx, 1), or one of the
  *    dense elimination's environment switches set when the context is created), every block is
  *    eliminated as a dense matrix in the context's precision ("the dense elimination" below).

@@ -192,6 +192,7 @@ sca_status plan(const sca_params& p, Engine& e) {
   if (const char* v = std::getenv("SCA_PAIR"))
     if (std::atoi(v) == 0) e.pair = false;
   e.nest_rule = nested_rule(p.t, M_PI * p.T, (2.0 * p.n_omega - 1.0) * M_PI * p.T);
+  e.nest_wide = nested_wide_blocks(e.fp64, p.L, p.t, p.T, p.n_omega);
   e.dense_only = dense_switch_set();
   size_t bytes = 0;
   bytes += (size_t)e.chunk * e.mat_stride * S;           // blocks
@@ -659,7 +660,11 @@ sca_status sca_dos(sca_ctx* c, const double* phi_host, const double* w_host, int
   e.dos_mode = true;
   e.dos_eta = eta;
   const int dense_saved = e.nest_dense;
+  const int wide_saved = e.nest_wide;
   e.nest_dense = eta > thr ? 0 : e.B;
+  // (the reduced precisions promise a density of states from float32 inverses without refinement,
+  // which double-float exceeds at every eta)
+  e.nest_wide = e.fp64 && nested_wide(true, e.L, e.p.t, eta) ? e.B : 0;
   for (int32_t k0 = 0; k0 < n_w && st == SCA_OK; k0 += half) {
     const int cnt = std::min<int>(half, n_w - k0);
     for (int n = 0; n < half; ++n) {  // a short last batch repeats its last frequency
@@ -689,6 +694,7 @@ sca_status sca_dos(sca_ctx* c, const double* phi_host, const double* w_host, int
   }
   e.dos_mode = false;
   e.nest_dense = dense_saved;
+  e.nest_wide = wide_saved;
   e.piv_blocks = saved;
   return st;
 }

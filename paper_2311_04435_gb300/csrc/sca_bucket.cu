@@ -1,7 +1,7 @@
 // Size buckets: the factorisations of several solve requests with the same lattice size and
 // precision share one workspace and one launch sequence.  Each pass stacks the blocks of a set
-// of requests (the pivoted blocks of all of them first, then the dominant ones, each request's
-// in block order), with a per-slot table of the request's field, t, Delta_eff, mu, T, n and
+// of requests (the pivoted blocks of all of them first, those in wider arithmetic before the others,
+// then the dominant ones, each request's in block order), with a per-slot table of the request's field, t, Delta_eff, mu, T, n and
 // sigma; one reduction CTA per request then forms its Omega, gradient and Adam update from its
 // own blocks.  Every block goes through the same kernels as in a pass of its own request, and
 // the sums run over the request's blocks in block order, so a request's result does not depend
@@ -131,6 +131,7 @@ sca_status bucket_req_init(Bucket* b, BucketReq* r, const sca_params& p, const s
   r->nb = 2 * p.n_omega;
   r->npiv = pivoted_count(p);
   r->nested = nested_rule(p.t, M_PI * p.T, (2.0 * p.n_omega - 1.0) * M_PI * p.T);
+  r->wide = nested_wide_blocks(p.prec == SCA_PREC_FP64, p.L, p.t, p.T, p.n_omega);
   r->delta_eff = (p.ionic == SCA_IONIC_HALF) ? 0.5 * p.delta : p.delta;
   cudaError_t err = cudaMalloc((void**)&r->d, sizeof(double) * (4 * (size_t)N + 8));
   if (err != cudaSuccess) { r->d = nullptr; return cuda_fail(err, "request state"); }
@@ -179,18 +180,19 @@ sca_status bucket_run(Bucket* b, BucketReq* const* requests, int n, int nsteps, 
   const int P = (int)first.size();
   sca_status st = ensure_tables(b, P, nsteps);
   if (st != SCA_OK) return st;
-  std::vector<int> npiv(P), ntot(P);
+  std::vector<int> wide(P), npiv(P), ntot(P);
   for (int p = 0; p < P; ++p) {
     BlockDesc* bd = b->h_bd + (size_t)p * b->cap;
     int* slots = b->h_slots + (size_t)p * b->cap;
-    // slot of each request's blocks: pivoted blocks of every request first, then the rest
+    // slot of each request's blocks: in wider arithmetic, the other pivoted ones, the rest
     int next = 0, off = 0;
     std::vector<int> base(count[p]);
     for (int k = 0; k < count[p]; ++k) { base[k] = off; off += reqs[first[p] + k]->nb; }
-    for (int pass_piv = 1; pass_piv >= 0; --pass_piv)
+    for (int range = 0; range < 3; ++range) {
       for (int k = 0; k < count[p]; ++k) {
         const BucketReq* r = reqs[first[p] + k];
-        const int lo = pass_piv ? 0 : r->npiv, hi = pass_piv ? r->npiv : r->nb;
+        const int ends[4] = {0, r->nested ? std::min(r->wide, r->npiv) : 0, r->npiv, r->nb};
+        const int lo = ends[range], hi = ends[range + 1];
         for (int blk = lo; blk < hi; ++blk) {
           BlockDesc d;
           d.phi = r->d;
@@ -205,8 +207,10 @@ sca_status bucket_run(Bucket* b, BucketReq* const* requests, int n, int nsteps, 
           slots[base[k] + blk] = next;
           ++next;
         }
-        if (pass_piv && k == count[p] - 1) npiv[p] = next;
       }
+      if (range == 0) wide[p] = next;
+      if (range == 1) npiv[p] = next;
+    }
     ntot[p] = next;
     for (int sidx = 0; sidx < nsteps; ++sidx) {
       ReqDesc* rq = b->h_req + ((size_t)p * b->steps + sidx) * b->rmax;
@@ -238,11 +242,13 @@ sca_status bucket_run(Bucket* b, BucketReq* const* requests, int n, int nsteps, 
                         cudaMemcpyHostToDevice, s);
   if (err != cudaSuccess) return cuda_fail(err, "bucket tables upload");
   const int B0 = e.B, piv0 = e.piv_blocks, dense0 = e.nest_dense;
+  const int wide0 = e.nest_wide;
   for (int sidx = 0; sidx < nsteps && st == SCA_OK; ++sidx)
     for (int p = 0; p < P && st == SCA_OK; ++p) {
       e.B = ntot[p];
       e.piv_blocks = npiv[p];
       e.nest_dense = npiv[p];
+      e.nest_wide = wide[p];
       e.nest_rule = reqs[first[p]]->nested;
       e.bd = b->d_bd + (size_t)p * b->cap;
       st = run_blocks(e, reqs[first[p]]->d, true, s);
@@ -252,6 +258,7 @@ sca_status bucket_run(Bucket* b, BucketReq* const* requests, int n, int nsteps, 
   e.B = B0;
   e.piv_blocks = piv0;
   e.nest_dense = dense0;
+  e.nest_wide = wide0;
   e.bd = nullptr;
   if (st != SCA_OK) return st;
   if (adam)

@@ -137,6 +137,7 @@ struct Engine {
   Nested* nest = nullptr;
   bool nest_rule = false;
   int nest_dense = 0;       // leading blocks without column dominance (dense leaves)
+  int nest_wide = 0;        // ... and those in wider arithmetic
   bool dense_only = false;
   bool fronts_kept = false;
   double dos_eta = 0.0;
@@ -237,15 +238,33 @@ sca_status run_refine_resident(Engine& e, const double* d_phi, cudaStream_t s);
 sca_status run_reduce(Engine& e, const double* d_phi, double* d_omega, double* d_grad,
                       const AdamStep* adam, cudaStream_t s);
 
-// Nested elimination (sca_nested.cu).  Its rounding errors can grow by powers of |t| / Im z, so
-// contexts whose smallest omega_n, and densities of states whose eta, lie below
-// kNestedMinImag |t| take the pivoted dense elimination.  Where the line lies: in float64 on
-// 100..400 sites with disorder, gradients are as close to the exact ones as the dense path's down
-// to T = 0.01 (omega_0 = 0.031), densities of states down to eta = 0.02 (8.2e-14 against 7.9e-14);
-// at eta = 0.01 the nested error is 1.7 times the dense one (1.8e-13 against 1.1e-13).  The other
-// limits keep double-float squares inside float32's range.
+// Nested elimination (sca_nested.cu).  Its rounding errors grow by powers of |t| / Im z where the
+// field is weak: a part of the lattice cut out by separators has levels at the energy itself
+// (bipartite pieces at half filling have zero modes), and its Schur complement is as large as
+// t^2 / Im z.  So the arithmetic of a block follows its Im z (omega_n; eta for a density of
+// states), such that results are as close to the exact ones as the pivoted dense elimination's,
+// field by field.  Largest error of G_ii relative to the largest |G_ii| over clean, staggered and
+// random fields of amplitude 0 to 1, t = 1, float64 dense / nested and float32 dense with its
+// refinement / double-float nested:
+//              6x6 to 10x10 sites                   12x12 to 20x20
+//   Im z 0.03  2e-15 / 4e-11   2e-11 / 1e-9         3e-15 / 1e-11   2e-11 / 3e-10
+//        0.05  2e-15 / 5e-12   8e-12 / 2e-10        2e-15 / 1e-12   7e-12 / 3e-11
+//        0.08  2e-15 / 9e-13   3e-12 / 2e-11        3e-15 / 2e-13   9e-12 / 5e-12
+//        0.11  1e-15 / 2e-13   2e-12 / 6e-12        3e-15 / 5e-14   7e-12 / 2e-12
+//        0.16  1e-15 / 6e-14   1e-12 / 2e-12        2e-15 / 1e-14   2e-11 / 4e-13
+//        0.31  1e-15 / 6e-15   1e-12 / 2e-13        5e-15 / 3e-15   1e-10 / 1e-13
+//        0.5   2e-15 / 2e-15   6e-13 / 4e-14        3e-15 / 2e-15   2e-12 / 4e-14
+// Below the lines a block is eliminated in sums of three float32 (72 bits; 3e-11 of float64's 53
+// are 1e-15 there, 2^-70 per operation), in float64 contexts in double-double where an entry leaves
+// float32's range.  Below kNestedMinImag |t| contexts take the dense elimination.  The limits on
+// the absolute values keep double-float squares inside float32's range.
 constexpr double kNestedMinImag = 0.03;
 bool nested_rule(double t, double imag_min, double imag_max);
+constexpr double kFloat64Enough = 0.5;  // in units of |t|
+constexpr double kFloat2EnoughSmall = 0.3, kFloat2Enough = 0.15;  // up to 10x10 sites, above
+enum class NestedArith { kFloat2, kFloat64, kWide32, kWide64 };  // the last: of a float64 context
+bool nested_wide(bool fp64, int L, double t, double imag);
+int nested_wide_blocks(bool fp64, int L, double t, double T, int n_omega);  // leading blocks
 sca_status nested_prepare(Engine& e);  // tables (leaves e.nest null where it does not apply)
 void nested_release(Engine& e);
 bool nested_now(const Engine& e);      // whether the next evaluation takes it
@@ -306,6 +325,7 @@ struct BucketReq {
   int32_t step = 0;
   int nb = 0, npiv = 0;
   bool nested = false;  // its frequencies admit the nested elimination
+  int wide = 0;         // its blocks in wider arithmetic there
   double delta_eff = 0.0;
   double* d = nullptr;
 };

@@ -15,15 +15,22 @@
 //
 // No pivot is searched for: -i A has the Hermitian part (Im z) I with Im z = w_n > 0 (eta for a
 // density of states), and so has every Schur complement and every leading block of one; each
-// pivot is at least Im z in modulus.  Rounding errors grow by powers of |t| / Im z, which is why
-// callers with Im z below kNestedMinImag |t| take the pivoted dense elimination (nested_rule).
+// pivot is at least Im z in modulus.  Rounding errors grow by powers of |t| / Im z on weak fields,
+// which is why blocks of small Im z take wider arithmetic (nested_wide) and callers with Im z below
+// kNestedMinImag |t| the pivoted dense elimination (nested_rule).
 //
 // Arithmetic: float64, or on the reduced-precision paths double-float (an unevaluated sum of two
 // float32, 48 bits): products exact by FMA, sums by two-sums, 12 float32 operations per real
 // multiply-add, two of them per instruction (real and imaginary part side by side: 20x20 with 512
 // blocks 1150 to 1080 us per gradient, 40x40 with 256 3794 to 3490, 64x64 with 128 8281 to 7360).
 // This GPU does 64 float32 FMAs in the time of one float64 FMA, so double-float is 5 times as
-// fast as float64 and keeps 24 bits more than the float32 blocks of the dense paths.
+// fast as float64 and keeps 24 bits more than the float32 blocks of the dense paths.  The few
+// blocks of small Im z: sums of three float32 (72 bits, 46 operations per real multiply-add, which
+// takes no longer than one of float64 does here: a 20x20 float64 density of states 1013 us in float64,
+// 1004 in these, 11324 in double-double).  They go beside the others, on a stream of their own, in
+// clusters of up to eight CTAs per block: a 20x20 gradient, T = 0.05, 124 blocks in float64 and 4 in
+// these, 1009 us, 1004 with all 128 in float64; 512 blocks, T = 0.1, 2 of them in these, 2291 / 2251.
+// On small lattices their dependent chain shows: 8x8 densities of states 287 us, 151 in float64.
 //
 // Work split: a group of threads per front (a warp for the smallest, 256 or 512 threads for the
 // largest), fronts in global memory (a block's take 3.2 MB at N = 1600), the current panel of at
@@ -68,6 +75,12 @@ struct alignas(16) Zd {
 struct alignas(16) Zf {  // re = rh + rl, im = ih + il: two pairs for the packed instructions
   float rh, ih, rl, il;
 };
+struct Zt {  // sums of three float32 each, 72 bits, as pairs (re, im)
+  unsigned long long h, m, l;
+};
+struct alignas(16) Zw {  // as Zf, of two float64 each: 106 bits
+  double rh, ih, rl, il;
+};
 
 // Running sums of products a b: float64, or float32 sums s with the sums c of their rounding
 // errors, two to a register pair.  Af holds (re, im); Aw holds (a.re, a.im) b.re in (s1, c1) and
@@ -82,6 +95,12 @@ struct Af {
 };
 struct Aw {
   f2 s1, c1, s2, c2;
+};
+struct At {  // sums, their rounding errors', and those sums' own
+  f2 s, c, d;
+};
+struct Aq {  // sums and the sums of their rounding errors, float64
+  double rs, rc, is, ic;
 };
 __device__ __forceinline__ f2 f2_of(float lo, float hi) {
   f2 r;
@@ -123,18 +142,58 @@ struct AccOf<Zf> {
   using type = Af;
   using wide = Aw;
 };
+template <>
+struct AccOf<Zt> {
+  using type = At;
+  using wide = At;
+};
+template <>
+struct AccOf<Zw> {
+  using type = Aq;
+  using wide = Aq;
+};
 
 __device__ __forceinline__ void zset(Zd& z, double re, double im) { z = {re, im}; }
 __device__ __forceinline__ void zset(Zf& z, double re, double im) {
   const dsf a = ds_of(re), b = ds_of(im);
   z = {a.h, b.h, a.l, b.l};
 }
+__device__ __forceinline__ void zset(Zt& z, double re, double im) {
+  const dsf a = ds_of(re), b = ds_of(im);
+  z.h = f2_of(a.h, b.h);
+  z.m = f2_of(a.l, b.l);
+  z.l = f2_of((float)((re - a.h) - a.l), (float)((im - b.h) - b.l));
+}
+__device__ __forceinline__ void zset0(Zt& z) { z = {0, 0, 0}; }
+__device__ __forceinline__ double zre(Zt z) {
+  float h, m, l, u;
+  f2_get(z.h, h, u);
+  f2_get(z.m, m, u);
+  f2_get(z.l, l, u);
+  return ((double)h + (double)m) + (double)l;
+}
+__device__ __forceinline__ double zim(Zt z) {
+  float h, m, l, u;
+  f2_get(z.h, u, h);
+  f2_get(z.m, u, m);
+  f2_get(z.l, u, l);
+  return ((double)h + (double)m) + (double)l;
+}
+__device__ __forceinline__ Zt zneg(Zt z) {
+  constexpr unsigned long long sign = 0x8000000080000000ull;
+  return {z.h ^ sign, z.m ^ sign, z.l ^ sign};
+}
+__device__ __forceinline__ void zset(Zw& z, double re, double im) { z = {re, im, 0.0, 0.0}; }
+__device__ __forceinline__ void zset0(Zw& z) { z = {0.0, 0.0, 0.0, 0.0}; }
 __device__ __forceinline__ void zset0(Zd& z) { z = {0.0, 0.0}; }
 __device__ __forceinline__ void zset0(Zf& z) { z = {0.f, 0.f, 0.f, 0.f}; }
 __device__ __forceinline__ double zre(Zd z) { return z.re; }
 __device__ __forceinline__ double zim(Zd z) { return z.im; }
 __device__ __forceinline__ double zre(Zf z) { return (double)z.rh + (double)z.rl; }
 __device__ __forceinline__ double zim(Zf z) { return (double)z.ih + (double)z.il; }
+__device__ __forceinline__ double zre(Zw z) { return z.rh + z.rl; }
+__device__ __forceinline__ double zim(Zw z) { return z.ih + z.il; }
+__device__ __forceinline__ Zw zneg(Zw z) { return {-z.rh, -z.ih, -z.rl, -z.il}; }
 __device__ __forceinline__ Zd zneg(Zd z) { return {-z.re, -z.im}; }
 __device__ __forceinline__ Zf zneg(Zf z) { return {-z.rh, -z.ih, -z.rl, -z.il}; }
 __device__ __forceinline__ Zd zadd(Zd a, Zd b) { return {a.re + b.re, a.im + b.im}; }
@@ -142,12 +201,67 @@ __device__ __forceinline__ Zf zadd(Zf a, Zf b) {
   const dsf r = ds_add({a.rh, a.rl}, {b.rh, b.rl}), i = ds_add({a.ih, a.il}, {b.ih, b.il});
   return {r.h, i.h, r.l, i.l};
 }
+// Sum s and rounding error r of a + b, of a - b.
+__device__ __forceinline__ void two_sum_f2(f2 a, f2 b, f2& s, f2& r) {
+  const f2 t = f2_add(a, b), z = f2_sub(t, a);
+  r = f2_add(f2_sub(a, f2_sub(t, z)), f2_sub(b, z));
+  s = t;
+}
+__device__ __forceinline__ void two_diff_f2(f2 a, f2 b, f2& s, f2& r) {
+  const f2 t = f2_sub(a, b), z = f2_sub(t, a);
+  r = f2_sub(f2_sub(a, f2_sub(t, z)), f2_add(b, z));
+  s = t;
+}
+// A number of three parts from sums of falling size.
+__device__ __forceinline__ Zt three(f2 s, f2 c, f2 d) {
+  two_sum_f2(c, d, c, d);
+  two_sum_f2(s, c, s, c);
+  two_sum_f2(c, d, c, d);
+  return {s, c, d};
+}
+__device__ __forceinline__ Zt zadd(Zt a, Zt b) {
+  f2 s, c, e, u;
+  two_sum_f2(a.h, b.h, s, e);
+  two_sum_f2(a.m, b.m, c, u);
+  f2 d = f2_add(f2_add(a.l, b.l), u);
+  two_sum_f2(c, e, c, u);
+  return three(s, c, f2_add(d, u));
+}
+// The same in float64 (the intrinsics keep the compiler from contracting).
+__device__ __forceinline__ void two_sum_d(double a, double b, double& s, double& r) {
+  s = __dadd_rn(a, b);
+  const double z = __dadd_rn(s, -a);
+  r = __dadd_rn(__dadd_rn(a, -__dadd_rn(s, -z)), __dadd_rn(b, -z));
+}
+__device__ __forceinline__ Zw zadd(Zw a, Zw b) {
+  double rs, rr, is, ir;
+  two_sum_d(a.rh, b.rh, rs, rr);
+  two_sum_d(a.ih, b.ih, is, ir);
+  Zw z;
+  two_sum_d(rs, rr + (a.rl + b.rl), z.rh, z.rl);
+  two_sum_d(is, ir + (a.il + b.il), z.ih, z.il);
+  return z;
+}
 
 __device__ __forceinline__ Zd zsel(bool c, Zd a, Zd b) {
   return {c ? a.re : b.re, c ? a.im : b.im};
 }
 __device__ __forceinline__ Zf zsel(bool c, Zf a, Zf b) {
   return {c ? a.rh : b.rh, c ? a.ih : b.ih, c ? a.rl : b.rl, c ? a.il : b.il};
+}
+__device__ __forceinline__ Zt zsel(bool c, Zt a, Zt b) {
+  return {c ? a.h : b.h, c ? a.m : b.m, c ? a.l : b.l};
+}
+__device__ __forceinline__ Zt zshfl_xor(Zt z, int off) {
+  return {__shfl_xor_sync(0xffffffffu, z.h, off), __shfl_xor_sync(0xffffffffu, z.m, off),
+          __shfl_xor_sync(0xffffffffu, z.l, off)};
+}
+__device__ __forceinline__ Zw zsel(bool c, Zw a, Zw b) {
+  return {c ? a.rh : b.rh, c ? a.ih : b.ih, c ? a.rl : b.rl, c ? a.il : b.il};
+}
+__device__ __forceinline__ Zw zshfl_xor(Zw z, int off) {
+  return {__shfl_xor_sync(0xffffffffu, z.rh, off), __shfl_xor_sync(0xffffffffu, z.ih, off),
+          __shfl_xor_sync(0xffffffffu, z.rl, off), __shfl_xor_sync(0xffffffffu, z.il, off)};
 }
 __device__ __forceinline__ Zd zshfl_xor(Zd z, int off) {
   return {__shfl_xor_sync(0xffffffffu, z.re, off), __shfl_xor_sync(0xffffffffu, z.im, off)};
@@ -160,6 +274,15 @@ __device__ __forceinline__ Zf zshfl_xor(Zf z, int off) {
 __device__ __forceinline__ void acc_of(Ad& a, Zd z) { a = {z.re, z.im}; }
 __device__ __forceinline__ void acc_of(Af& a, Zf z) {
   a = {f2_of(z.rh, z.ih), f2_of(z.rl, z.il)};
+}
+__device__ __forceinline__ void acc_of(At& a, Zt z) { a = {z.h, z.m, z.l}; }
+__device__ __forceinline__ Zt acc_get(At a) { return three(a.s, a.c, a.d); }
+__device__ __forceinline__ void acc_of(Aq& a, Zw z) { a = {z.rh, z.rl, z.ih, z.il}; }
+__device__ __forceinline__ Zw acc_get(Aq a) {
+  Zw z;
+  two_sum_d(a.rs, a.rc, z.rh, z.rl);
+  two_sum_d(a.is, a.ic, z.ih, z.il);
+  return z;
 }
 __device__ __forceinline__ Zd acc_get(Ad a) { return {a.re, a.im}; }
 __device__ __forceinline__ Zf acc_get(Af a) {
@@ -201,6 +324,23 @@ __device__ __forceinline__ void mac1(float& s, float& c, float ah, float al, flo
   s = t;
   c = __fadd_rn(c, __fadd_rn(r, e));
 }
+__device__ __forceinline__ void mac1(double& s, double& c, double ah, double al, double bh,
+                                     double bl) {
+  const double p = __dmul_rn(ah, bh);
+  double e = fma(ah, bh, -p);
+  e = fma(ah, bl, e);
+  e = fma(al, bh, e);
+  double t, r;
+  two_sum_d(s, p, t, r);
+  s = t;
+  c = __dadd_rn(c, __dadd_rn(r, e));
+}
+__device__ __forceinline__ void mac(Aq& s, Zw a, Zw b) {
+  mac1(s.rs, s.rc, a.rh, a.rl, b.rh, b.rl);
+  mac1(s.is, s.ic, a.rh, a.rl, b.ih, b.il);
+  mac1(s.rs, s.rc, -a.ih, -a.il, b.ih, b.il);
+  mac1(s.is, s.ic, a.ih, a.il, b.rh, b.rl);
+}
 // The same for both halves of a pair, in half the instructions.  A pair cannot be negated in
 // place: -p is taken apart and put together again, or, in the second form, minus b comes in.
 __device__ __forceinline__ void mac2(f2& s, f2& c, f2 ah, f2 al, f2 bh, f2 bl) {
@@ -234,6 +374,34 @@ __device__ __forceinline__ void mac(Aw& s, Zf a, Zf b) {
   mac2(s.s1, s.c1, ah, al, f2_of(b.rh, b.rh), f2_of(-b.rh, -b.rh), f2_of(-b.rl, -b.rl));
   mac2(s.s2, s.c2, ah, al, f2_of(b.ih, b.ih), f2_of(-b.ih, -b.ih), f2_of(-b.il, -b.il));
 }
+// (s, c, d) += (a0 + a1 + a2)(b0 + b1 + b2), n = -b: the leading product with its error exactly, the
+// two of the next order likewise, the three of the order after (and the errors of the second) to
+// float32 accuracy; what is added to c keeps its errors in d.
+__device__ __forceinline__ void mac3(At& s, f2 a0, f2 a1, f2 a2, f2 b0, f2 b1, f2 b2, f2 n0, f2 n1) {
+  const f2 p = f2_mul(a0, b0), p1 = f2_mul(a0, b1), p2 = f2_mul(a1, b0);
+  const f2 e = f2_fma(a0, n0, p), e1 = f2_fma(a0, n1, p1), e2 = f2_fma(a1, n0, p2);  // minus them
+  const f2 q = f2_fma(a0, b2, f2_fma(a1, b1, f2_mul(a2, b0)));
+  f2 r, u, ue, v, ve, we, r1;
+  two_sum_f2(s.s, p, s.s, r);
+  two_sum_f2(p1, p2, u, ue);
+  two_diff_f2(r, e, v, ve);
+  two_sum_f2(u, v, u, we);
+  two_sum_f2(s.c, u, s.c, r1);
+  s.d = f2_add(s.d, f2_add(f2_add(f2_add(ue, ve), f2_add(we, r1)), f2_sub(q, f2_add(e1, e2))));
+}
+__device__ __forceinline__ void mac(At& s, Zt a, Zt b) {
+  float ar, ai, mr, mi, lr, li, br[3], bi[3];
+  f2_get(a.h, ar, ai);
+  f2_get(a.m, mr, mi);
+  f2_get(a.l, lr, li);
+  f2_get(b.h, br[0], bi[0]);
+  f2_get(b.m, br[1], bi[1]);
+  f2_get(b.l, br[2], bi[2]);
+  mac3(s, f2_of(ar, ar), f2_of(mr, mr), f2_of(lr, lr), b.h, b.m, b.l, f2_of(-br[0], -bi[0]),
+       f2_of(-br[1], -bi[1]));
+  mac3(s, f2_of(ai, ai), f2_of(mi, mi), f2_of(li, li), f2_of(-bi[0], br[0]), f2_of(-bi[1], br[1]),
+       f2_of(-bi[2], br[2]), f2_of(bi[0], -br[0]), f2_of(bi[1], -br[1]));
+}
 template <typename Z>
 __device__ __forceinline__ Z zmul(Z a, Z b) {
   typename AccOf<Z>::type s{};
@@ -263,6 +431,60 @@ __device__ __forceinline__ Zf zinv(Zf z, double* mag2 = nullptr) {
   mac1(is, ic, -z.ih, -z.il, q, ql);
   const dsf r = two_sum(rs, rc), i = two_sum(is, ic);
   return {r.h, i.h, r.l, i.l};
+}
+__device__ __forceinline__ Zt zinv(Zt z, double* mag2 = nullptr) {
+  At s{};
+  const Zt n = zneg(z);
+  mac3(s, z.h, z.m, z.l, z.h, z.m, z.l, n.h, n.m);  // re^2, im^2
+  const Zt sq = acc_get(s);
+  float h0, h1, m0, m1, l0, l1;
+  f2_get(sq.h, h0, h1);
+  f2_get(sq.m, m0, m1);
+  f2_get(sq.l, l0, l1);
+  dsf h = two_sum(h0, h1), m = two_sum(m0, m1);
+  float l = __fadd_rn(__fadd_rn(l0, l1), m.l);
+  m = two_sum(m.h, h.l);  // |z|^2 = h.h + m.h + l
+  l = __fadd_rn(l, m.l);
+  const dsf d = two_sum(h.h, m.h);
+  const dsf d2 = two_sum(d.l, l);
+  if (mag2) *mag2 = ((double)d.h + (double)d2.h) + (double)d2.l;
+  // 1 / |z|^2 = q (1 + e + e^2) to e^3 < 2^-69, e = 1 - q |z|^2 to 48 bits
+  const float q = __frcp_rn(d.h);
+  const float e0 = fmaf(-q, d.h, 1.0f), p = __fmul_rn(q, d2.h), pe = fmaf(q, d2.h, -p);
+  dsf e = two_sum(e0, -p);
+  e.l = __fadd_rn(e.l, -fmaf(q, d2.l, pe));
+  e = two_sum(e.h, fmaf(e.h, e.h, e.l));
+  const float f = __fmul_rn(q, e.h), fe = fmaf(q, e.l, fmaf(q, e.h, -f));
+  const dsf i0 = two_sum(q, f);
+  const dsf i1 = two_sum(i0.l, fe);
+  const f2 qh = f2_of(i0.h, i0.h), qm = f2_of(i1.h, i1.h), ql = f2_of(i1.l, i1.l);
+  float zr[3], zi[3];
+  f2_get(z.h, zr[0], zi[0]);
+  f2_get(z.m, zr[1], zi[1]);
+  f2_get(z.l, zr[2], zi[2]);
+  At r{};
+  mac3(r, qh, qm, ql, f2_of(zr[0], -zi[0]), f2_of(zr[1], -zi[1]), f2_of(zr[2], -zi[2]),
+       f2_of(-zr[0], zi[0]), f2_of(-zr[1], zi[1]));
+  return acc_get(r);
+}
+__device__ __forceinline__ Zw zinv(Zw z, double* mag2 = nullptr) {
+  double s = 0.0, c = 0.0;
+  mac1(s, c, z.rh, z.rl, z.rh, z.rl);
+  mac1(s, c, z.ih, z.il, z.ih, z.il);
+  double d, dl;
+  two_sum_d(s, c, d, dl);
+  if (mag2) *mag2 = d;
+  const double q = recip(d);  // then one Newton step: q + q (1 - d q)
+  double e = fma(-q, d, 1.0);
+  e = fma(-q, dl, e);
+  const double ql = __dmul_rn(q, e);
+  double rs = 0.0, rc = 0.0, is = 0.0, ic = 0.0;
+  mac1(rs, rc, z.rh, z.rl, q, ql);
+  mac1(is, ic, -z.ih, -z.il, q, ql);
+  Zw r;
+  two_sum_d(rs, rc, r.rh, r.rl);
+  two_sum_d(is, ic, r.ih, r.il);
+  return r;
 }
 
 // A product of moduli squared as mantissa in [1, 2) and exponent: a node's share of |det A|^2.
@@ -317,6 +539,7 @@ struct NestArgs {
   int b0;                // block of the pass's first slot
   int csize;             // CTAs per block
   int ndense;            // leading slots of the pass that take the dense leaves
+  int range;             // 1: not blocks whose entries leave float32's range; 2: those alone
   int k0, k1;            // phases: [0, nlevels) up from the leaves, [nlevels, 2 nlevels) down
   Lattice la;
   double* ld;            // ln|det A_b|
@@ -894,6 +1117,12 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : 1) k_nested(NestArgs<Z> a)
     B.flags = a.flags;
   }
   __syncthreads();
+  if (a.range) {
+    int big = 0;
+    for (int i = tid; i < B.la.N; i += NT)
+      if (!(fabs(B.zr - site_energy(B.la, i, B.sg)) < 0x1p60)) big = 1;
+    if (__syncthreads_or(big) != (a.range == 2)) return;  // (alike in all CTAs of a block)
+  }
   for (int k = a.k0; k < a.k1; ++k) {
     const bool up = k < a.nlevels;
     const LevelPlan& lv = a.lv[form][up ? a.nlevels - 1 - k : k - a.nlevels];
@@ -947,14 +1176,15 @@ __global__ void __launch_bounds__(256) k_nest_trace(int N, int b0, const double*
     if (err__ != cudaSuccess) return cuda_fail(err__, where);     \
   } while (0)
 
-size_t up_smem(const nested::Node& n) {
+// z: bytes of an entry
+size_t up_smem(const nested::Node& n, size_t z) {
   const size_t m = n.p + n.q, pw = n.pw;
-  return 16 * (pw * (2 * (m - pw) + kRows) + pw * pw + 2 * pw + 2 * (pw + 1) + n.blacks + n.p + 1) +
+  return z * (pw * (2 * (m - pw) + kRows) + pw * pw + 2 * pw + 2 * (pw + 1) + n.blacks + n.p + 1) +
          32 * sizeof(double) + sizeof(int16_t) * m * (n.blacks ? 4 : 3);
 }
-size_t down_smem(const nested::Node& n) {
+size_t down_smem(const nested::Node& n, size_t z) {
   const size_t m = n.p + n.q;
-  return 16 * (2 * (size_t)n.pw * ((m - n.pw) | 1) + (size_t)n.pw * n.pw) + sizeof(int16_t) * n.q;
+  return z * (2 * (size_t)n.pw * ((m - n.pw) | 1) + (size_t)n.pw * n.pw) + sizeof(int16_t) * n.q;
 }
 
 }  // namespace
@@ -964,15 +1194,29 @@ struct Nested {
   Node* d_nodes = nullptr;
   int16_t* d_tab = nullptr;
   struct Shape {
-    int first, count, group, smem;  // group: the fewest threads for a front
+    int first, count, group;  // group: the fewest threads for a front
+    int bytes[3];             // shared memory of a front with entries of 16, 24 and 32 bytes
+    template <typename Z>
+    int smem() const { return bytes[sizeof(Z) / 8 - 2]; }
   };
   std::vector<Shape> levels[2];
   int nnodes = 0;
   long long stride = 0;   // entries per block
-  int cap = 0;            // blocks per pass
+  char* fronts = nullptr; // where they are kept: the context's blocks, or `own`
+  size_t room = 0;
+  void* own = nullptr;    // their own memory where the blocks' is too small
   int sms = 1;
-  cudaStream_t half = nullptr;  // the second half of a pass that takes a launch per level
-  cudaEvent_t ev_half = nullptr;
+  // more blocks than SMs: the second half of a pass that takes a launch per level, and the blocks
+  // in wider arithmetic (which otherwise take the side stream)
+  cudaStream_t half = nullptr, wide = nullptr;
+  cudaEvent_t ev_half = nullptr, ev_wide = nullptr;
+
+  // A block's fronts, and with its shares of |det A|^2.  (A float64 context's wider blocks have
+  // room for double-double, at the same place for both arithmetics that they may take.)
+  size_t front_bytes(NestedArith a) const {
+    return (a == NestedArith::kWide64 ? 32 : a == NestedArith::kWide32 ? 24 : 16) * (size_t)stride;
+  }
+  size_t block_bytes(NestedArith a) const { return front_bytes(a) + sizeof(Det) * nnodes; }
 };
 
 namespace {
@@ -989,10 +1233,11 @@ size_t plan_levels(const Nested& ne, NestArgs<Z>& a) {
   for (int form = 0; form < 2; ++form)
     for (size_t k = 0; k < ne.levels[form].size(); ++k) {
       const Nested::Shape& s = ne.levels[form][k];
+      const int smem = s.smem<Z>();
       int g = s.group;
-      while (2 * g <= nt && ((nt / (2 * g)) * a.csize >= s.count || nt / g * s.smem > room)) g *= 2;
-      a.lv[form][k] = {s.first, s.count, g, s.smem};
-      need = std::max(need, (size_t)(nt / g) * s.smem);
+      while (2 * g <= nt && ((nt / (2 * g)) * a.csize >= s.count || nt / g * smem > room)) g *= 2;
+      a.lv[form][k] = {s.first, s.count, g, smem};
+      need = std::max(need, (size_t)(nt / g) * smem);
     }
   return need;
 }
@@ -1033,100 +1278,119 @@ sca_status launch(Engine& e, const NestArgs<Z>& a, int cnt, size_t smem, cudaStr
   return SCA_OK;
 }
 
+// Blocks [b0, b0 + cnt) in arithmetic Z, their fronts at `mem`, `bytes` for each, on `s`; `free_sms`
+// SMs are for them.
 template <typename Z>
-sca_status run_nested_t(Engine& e, const Lattice& la, bool up, bool down, cudaStream_t s) {
+sca_status run_blocks_of(Engine& e, const Lattice& la, int b0, int cnt, char* mem, size_t bytes,
+                         int free_sms, bool up, bool down, cudaStream_t s, int range = 0) {
   const Nested& ne = *e.nest;
   NestArgs<Z> a;
   a.nodes = ne.d_nodes;
   a.tab = ne.d_tab;
-  a.fronts = static_cast<Z*>(e.M);
-  a.stride = ne.stride;
+  a.fronts = reinterpret_cast<Z*>(mem);
+  a.stride = (long long)(bytes / sizeof(Z));
   a.nnodes = ne.nnodes;
   a.nlevels = (int)ne.levels[0].size();
   a.la = la;
   a.ld = e.ld;
   a.gd = e.gd;
   a.flags = e.flags;
-  for (int b0 = 0; b0 < e.B; b0 += ne.cap) {
-    const int cnt = std::min(ne.cap, e.B - b0);
-    a.b0 = b0;
-    a.det = reinterpret_cast<Det*>(a.fronts + (size_t)cnt * ne.stride);
-    const int nl = a.nlevels, p0 = up ? 0 : nl, p1 = down ? 2 * nl : nl;
-    sca_status st = SCA_OK;
-    const int dense = std::min(cnt, std::max(0, e.nest_dense - b0));
-    a.ndense = dense;
-    if (cnt > ne.sms) {
-      // side by side: the few blocks with dense leaves on the high-priority stream, and the others
-      // in two halves, so that one half's fronts fill the SMs that the last wave of the other's
-      // level leaves idle
-      struct Part {
-        int form, first, n, all;  // all: blocks of the form, which the group sizes follow
-        cudaStream_t s;
-        cudaEvent_t join;
-      } parts[4];
-      int nparts = 0;
-      const bool two = dense > 0 && dense < cnt && e.side != nullptr;
-      for (int form = 1; form >= 0; --form) {
-        const int n = form ? dense : cnt - dense, first = form ? 0 : dense;
-        const int h = ne.half && n >= kHalves && !(form && two) ? n / 2 : 0;
-        if (n == 0) continue;
-        if (form && two)
-          parts[nparts++] = {form, first, n, n, e.side, e.ev_join};
-        else
-          parts[nparts++] = {form, first, n - h, n, s, nullptr};
-        if (h) parts[nparts++] = {form, first + n - h, h, n, ne.half, ne.ev_half};
+  a.b0 = b0;
+  a.det = reinterpret_cast<Det*>(mem + (size_t)cnt * bytes);
+  const int nl = a.nlevels, p0 = up ? 0 : nl, p1 = down ? 2 * nl : nl;
+  sca_status st = SCA_OK;
+  const int dense = std::min(cnt, std::max(0, e.nest_dense - b0));
+  a.ndense = dense;
+  a.range = range;
+  if (cnt > ne.sms && sizeof(Z) == 16) {
+    // side by side: the few blocks with dense leaves on the high-priority stream, and the others
+    // in two halves, so that one half's fronts fill the SMs that the last wave of the other's
+    // level leaves idle
+    struct Part {
+      int form, first, n, all;  // all: blocks of the form, which the group sizes follow
+      cudaStream_t s;
+      cudaEvent_t join;
+    } parts[4];
+    int nparts = 0;
+    const bool two = dense > 0 && dense < cnt && e.side != nullptr;
+    for (int form = 1; form >= 0; --form) {
+      const int n = form ? dense : cnt - dense, first = form ? 0 : dense;
+      const int h = ne.half && n >= kHalves && !(form && two) ? n / 2 : 0;
+      if (n == 0) continue;
+      if (form && two)
+        parts[nparts++] = {form, first, n, n, e.side, e.ev_join};
+      else
+        parts[nparts++] = {form, first, n - h, n, s, nullptr};
+      if (h) parts[nparts++] = {form, first + n - h, h, n, ne.half, ne.ev_half};
+    }
+    cudaError_t err = cudaSuccess;
+    if (nparts > 1) err = cudaEventRecord(e.ev_fork, s);
+    for (int i = 0; i < nparts && err == cudaSuccess; ++i)
+      if (parts[i].join) err = cudaStreamWaitEvent(parts[i].s, e.ev_fork, 0);
+    if (err != cudaSuccess) return cuda_fail(err, "fork");
+    for (int k = p0; k < p1; ++k)
+      for (int i = 0; i < nparts; ++i) {
+        const Part& pt = parts[i];
+        NestArgs<Z> f = a;  // the part's blocks alone
+        f.b0 = b0 + pt.first;
+        f.fronts = a.fronts + (size_t)pt.first * a.stride;
+        f.det = a.det + (size_t)pt.first * a.nnodes;
+        f.ndense = pt.form ? pt.n : 0;
+        const int level = k < nl ? nl - 1 - k : k - nl;
+        f.k0 = k;
+        f.k1 = k + 1;
+        const Nested::Shape& sh = ne.levels[pt.form][level];
+        const int smem = sh.smem<Z>();
+        int g = sh.group;  // the fewest threads while they fill the SMs; four CTAs per SM
+        while (2 * g <= 256 && ((long long)sh.count * pt.all * g < 1024ll * ne.sms ||
+                                256 / g * smem > 55 << 10))
+          g *= 2;
+        f.lv[pt.form][level] = {sh.first, sh.count, g, smem};
+        f.csize = (sh.count + 256 / g - 1) / (256 / g);
+        if constexpr (sizeof(Z) == 16)
+          st = launch<Z, 256, false>(e, f, pt.n, (size_t)(256 / g) * smem, pt.s);
+        if (st != SCA_OK) return st;
       }
-      cudaError_t err = cudaSuccess;
-      if (nparts > 1) err = cudaEventRecord(e.ev_fork, s);
-      for (int i = 0; i < nparts && err == cudaSuccess; ++i)
-        if (parts[i].join) err = cudaStreamWaitEvent(parts[i].s, e.ev_fork, 0);
-      if (err != cudaSuccess) return cuda_fail(err, "fork");
-      for (int k = p0; k < p1; ++k)
-        for (int i = 0; i < nparts; ++i) {
-          const Part& pt = parts[i];
-          NestArgs<Z> f = a;  // the part's blocks alone
-          f.b0 = b0 + pt.first;
-          f.fronts = a.fronts + (size_t)pt.first * a.stride;
-          f.det = a.det + (size_t)pt.first * a.nnodes;
-          f.ndense = pt.form ? pt.n : 0;
-          const int level = k < nl ? nl - 1 - k : k - nl;
-          f.k0 = k;
-          f.k1 = k + 1;
-          const Nested::Shape& sh = ne.levels[pt.form][level];
-          int g = sh.group;  // the fewest threads while they fill the SMs; four CTAs per SM
-          while (2 * g <= 256 && ((long long)sh.count * pt.all * g < 1024ll * ne.sms ||
-                                  256 / g * sh.smem > 55 << 10))
-            g *= 2;
-          f.lv[pt.form][level] = {sh.first, sh.count, g, sh.smem};
-          f.csize = (sh.count + 256 / g - 1) / (256 / g);
-          st = launch<Z, 256, false>(e, f, pt.n, (size_t)(256 / g) * sh.smem, pt.s);
-          if (st != SCA_OK) return st;
-        }
-      for (int i = 0; i < nparts && err == cudaSuccess; ++i)
-        if (parts[i].join) {
-          err = cudaEventRecord(parts[i].join, parts[i].s);
-          if (err == cudaSuccess) err = cudaStreamWaitEvent(s, parts[i].join, 0);
-        }
-      if (err != cudaSuccess) return cuda_fail(err, "join");
-    } else {
-      // CTAs per block: as many as there are SMs for, up to the portable cluster size
-      a.k0 = p0;
-      a.k1 = p1;
-      a.csize = 1;
-      while (a.csize < 8 && 2 * a.csize * cnt <= ne.sms) a.csize *= 2;
-      const size_t smem = plan_levels(ne, a);
-      st = a.csize > 1 ? launch<Z, 512, true>(e, a, cnt, smem, s)
-                       : launch<Z, 512, false>(e, a, cnt, smem, s);
-    }
-    if (st != SCA_OK) return st;
-    if (down && la.zshift) {
-      prof_begin(e, kRefine, s);
-      k_nest_trace<<<cnt, 256, 0, s>>>(e.N, b0, e.gd, e.tr);
-      prof_end(e, kRefine, s);
-      SCA_LAUNCH_CHECK("nested trace");
-    }
+    for (int i = 0; i < nparts && err == cudaSuccess; ++i)
+      if (parts[i].join) {
+        err = cudaEventRecord(parts[i].join, parts[i].s);
+        if (err == cudaSuccess) err = cudaStreamWaitEvent(s, parts[i].join, 0);
+      }
+    if (err != cudaSuccess) return cuda_fail(err, "join");
+  } else {
+    // CTAs per block: as many as there are SMs for, up to the portable cluster size
+    a.k0 = p0;
+    a.k1 = p1;
+    a.csize = 1;
+    while (a.csize < 8 && 2 * a.csize * cnt <= free_sms) a.csize *= 2;
+    const size_t smem = plan_levels(ne, a);
+    st = a.csize > 1 ? launch<Z, 512, true>(e, a, cnt, smem, s)
+                     : launch<Z, 512, false>(e, a, cnt, smem, s);
+  }
+  if (st != SCA_OK) return st;
+  if (down && la.zshift && range != 1) {
+    prof_begin(e, kRefine, s);
+    k_nest_trace<<<cnt, 256, 0, s>>>(e.N, b0, e.gd, e.tr);
+    prof_end(e, kRefine, s);
+    SCA_LAUNCH_CHECK("nested trace");
   }
   return SCA_OK;
+}
+
+sca_status run_blocks_in(NestedArith ar, Engine& e, const Lattice& la, int b0, int cnt, char* mem,
+                         int free_sms, bool up, bool down, cudaStream_t s) {
+  const size_t by = e.nest->front_bytes(ar);
+  if (ar == NestedArith::kFloat2)
+    return run_blocks_of<Zf>(e, la, b0, cnt, mem, by, free_sms, up, down, s);
+  if (ar == NestedArith::kFloat64)
+    return run_blocks_of<Zd>(e, la, b0, cnt, mem, by, free_sms, up, down, s);
+  if (ar == NestedArith::kWide32)
+    return run_blocks_of<Zt>(e, la, b0, cnt, mem, by, free_sms, up, down, s);
+  // a float64 context: entries beyond float32's range take double-double (a launch that ends at
+  // once where there are none)
+  sca_status st = run_blocks_of<Zt>(e, la, b0, cnt, mem, by, free_sms, up, down, s, 1);
+  if (st == SCA_OK) st = run_blocks_of<Zw>(e, la, b0, cnt, mem, by, free_sms, up, down, s, 2);
+  return st;
 }
 
 }  // namespace
@@ -1136,33 +1400,39 @@ bool nested_rule(double t, double imag_min, double imag_max) {
          std::fabs(t) <= 1e9;
 }
 
+bool nested_wide(bool fp64, int L, double t, double imag) {
+  const double enough = fp64 ? kFloat64Enough : L <= 10 ? kFloat2EnoughSmall : kFloat2Enough;
+  return imag < enough * std::fabs(t);
+}
+
+int nested_wide_blocks(bool fp64, int L, double t, double T, int n_omega) {
+  int n = 0;
+  while (n < n_omega && nested_wide(fp64, L, t, (2.0 * n + 1.0) * M_PI * T)) ++n;
+  return 2 * n;
+}
+
 sca_status nested_prepare(Engine& e) {
   e.nest = nullptr;
   if (e.L < nested::kMinL) return SCA_OK;
   nested::Tree t = nested::Builder(e.L).build(false);
   const nested::Tree td = nested::Builder(e.L).build(true);
-  const size_t S = e.fp64 ? 8 : 4;
-  const long long stride = std::max(t.entries, td.entries);
-  const size_t per_block = 16 * (size_t)stride + sizeof(Det) * t.nodes.size();
-  const size_t room = e.block_room;
-  const long long cap = (long long)(room / per_block);
-  if (cap < e.chunk) return SCA_OK;
   Nested* ne = new (std::nothrow) Nested();
   if (!ne) { set_error("host allocation failed"); return SCA_ENOMEM; }
   e.nest = ne;
   ne->nnodes = (int)td.nodes.size();
-  ne->stride = stride;
-  ne->cap = (int)std::min<long long>(cap, e.B);
+  ne->stride = (std::max(t.entries, td.entries) + 5) / 6 * 6;  // whole entries of 16, 24, 32 bytes
   const nested::Tree* forms[2] = {&t, &td};
   for (int form = 0; form < 2; ++form)
     for (const nested::Level& lv : forms[form]->levels) {
-      Nested::Shape sh{lv.first, lv.count, 32, 0};
+      Nested::Shape sh{lv.first, lv.count, 32, {0, 0, 0}};
       for (int k = lv.first; k < lv.first + lv.count; ++k) {
         const nested::Node& n = forms[form]->nodes[k];
         while (10 * sh.group < 9 * (n.p + n.q) || n.pw > kSlots * (sh.group / n.pw)) sh.group *= 2;
-        sh.smem = (int)std::max<size_t>(sh.smem, std::max(up_smem(n), down_smem(n)));
+        for (int z = 16; z <= 32; z += 8) {
+          int& by = sh.bytes[z / 8 - 2];
+          by = std::max(by, ((int)std::max(up_smem(n, z), down_smem(n, z)) + 15) / 16 * 16);
+        }
       }
-      sh.smem = (sh.smem + 15) / 16 * 16;
       ne->levels[form].push_back(sh);
     }
   // both forms in one table: the second's offsets follow the first's entries
@@ -1177,17 +1447,37 @@ sca_status nested_prepare(Engine& e) {
   if (err == cudaSuccess)
     err = cudaDeviceGetAttribute(&ne->sms, cudaDevAttrMultiProcessorCount, dev);
   if (err != cudaSuccess) { nested_release(e); return cuda_fail(err, "nested elimination set-up"); }
-  if (e.B > ne->sms) {
-    err = cudaStreamCreateWithFlags(&ne->half, cudaStreamNonBlocking);
+  err = cudaEventCreateWithFlags(&ne->ev_wide, cudaEventDisableTiming);
+  if (err == cudaSuccess && e.B > ne->sms) {
+    int least = 0, greatest = 0;
+    err = cudaDeviceGetStreamPriorityRange(&least, &greatest);
+    if (err == cudaSuccess)
+      err = cudaStreamCreateWithPriority(&ne->wide, cudaStreamNonBlocking, greatest);
+    if (err == cudaSuccess) err = cudaStreamCreateWithFlags(&ne->half, cudaStreamNonBlocking);
     if (err == cudaSuccess) err = cudaEventCreateWithFlags(&ne->ev_half, cudaEventDisableTiming);
-    if (err != cudaSuccess) { nested_release(e); return cuda_fail(err, "nested elimination set-up"); }
   }
-  err = cudaMalloc((void**)&ne->d_nodes, sizeof(Node) * t.nodes.size());
+  if (err != cudaSuccess) { nested_release(e); return cuda_fail(err, "nested elimination set-up"); }
+  // Room for all blocks in their arithmetic where all are to be resident, and for one block of the
+  // wider one in any case.  From 10 x 10 sites up the dense blocks take more than either.
+  const NestedArith base = e.fp64 ? NestedArith::kFloat64 : NestedArith::kFloat2;
+  const NestedArith wide = e.fp64 ? NestedArith::kWide64 : NestedArith::kWide32;
+  size_t need = ne->block_bytes(wide);
+  if (e.chunk == e.B)
+    need = std::max(need, e.nest_wide * ne->block_bytes(wide) +
+                              (e.B - e.nest_wide) * ne->block_bytes(base) + 256);
+  ne->fronts = static_cast<char*>(e.M);
+  ne->room = e.block_room;
+  if (need > ne->room) {
+    err = cudaMalloc(&ne->own, need);
+    ne->fronts = static_cast<char*>(ne->own);
+    ne->room = need;
+  }
+  if (err == cudaSuccess) err = cudaMalloc((void**)&ne->d_nodes, sizeof(Node) * t.nodes.size());
   if (err == cudaSuccess) err = cudaMalloc((void**)&ne->d_tab, sizeof(int16_t) * t.table.size());
   if (err != cudaSuccess) {
     nested_release(e);
     (void)cudaGetLastError();
-    set_error("cudaMalloc failed for the elimination tree");
+    set_error("cudaMalloc failed for the elimination tree or its fronts");
     return SCA_ENOMEM;
   }
   err = cudaMemcpy(ne->d_nodes, t.nodes.data(), sizeof(Node) * t.nodes.size(), cudaMemcpyHostToDevice);
@@ -1203,7 +1493,13 @@ void nested_release(Engine& e) {
     cudaStreamSynchronize(e.nest->half);
     cudaStreamDestroy(e.nest->half);
   }
+  if (e.nest->wide) {
+    cudaStreamSynchronize(e.nest->wide);
+    cudaStreamDestroy(e.nest->wide);
+  }
   if (e.nest->ev_half) cudaEventDestroy(e.nest->ev_half);
+  if (e.nest->ev_wide) cudaEventDestroy(e.nest->ev_wide);
+  if (e.nest->own) cudaFree(e.nest->own);
   if (e.nest->d_nodes) cudaFree(e.nest->d_nodes);
   if (e.nest->d_tab) cudaFree(e.nest->d_tab);
   delete e.nest;
@@ -1211,11 +1507,67 @@ void nested_release(Engine& e) {
 }
 
 sca_status run_nested(Engine& e, const Lattice& la, bool up, bool down, cudaStream_t s) {
+  const Nested& ne = *e.nest;
+  cudaError_t err = cudaSuccess;
   if (up) {
-    const cudaError_t err = cudaMemsetAsync(e.flags, 0, sizeof(int), s);
+    err = cudaMemsetAsync(e.flags, 0, sizeof(int), s);
     if (err != cudaSuccess) return cuda_fail(err, "flags reset");
   }
-  return e.fp64 ? run_nested_t<Zd>(e, la, up, down, s) : run_nested_t<Zf>(e, la, up, down, s);
+  // the blocks in wider arithmetic first, then the others
+  struct Group {
+    NestedArith ar;
+    int first, n;
+    size_t bytes;
+  } groups[2];
+  int ng = 0;
+  const int nw = std::min(e.B, e.nest_wide);
+  const int ends[3] = {0, nw, e.B};
+  const NestedArith kinds[2] = {e.fp64 ? NestedArith::kWide64 : NestedArith::kWide32,
+                                e.fp64 ? NestedArith::kFloat64 : NestedArith::kFloat2};
+  size_t total = 0;
+  for (int k = 0; k < 2; ++k)
+    if (const int n = ends[k + 1] - ends[k]) {
+      groups[ng] = {kinds[k], ends[k], n, (n * ne.block_bytes(kinds[k]) + 255) / 256 * 256};
+      total += k == 0 && nw < e.B ? groups[ng].bytes : n * ne.block_bytes(kinds[k]);
+      ++ng;
+    }
+  if (total > ne.room) {  // one after another, in passes that fit
+    if (!up) {
+      set_error("the eliminated fronts are not all resident");
+      return SCA_ENOSTATE;
+    }
+    for (int g = 0; g < ng; ++g) {
+      const int cap = (int)std::min<size_t>(ne.room / ne.block_bytes(groups[g].ar), groups[g].n);
+      for (int b = 0; b < groups[g].n; b += cap) {
+        const sca_status st = run_blocks_in(groups[g].ar, e, la, groups[g].first + b,
+                                            std::min(cap, groups[g].n - b), ne.fronts, ne.sms, up,
+                                            down, s);
+        if (st != SCA_OK) return st;
+      }
+    }
+    return SCA_OK;
+  }
+  if (ng < 2)
+    return run_blocks_in(groups[0].ar, e, la, groups[0].first, groups[0].n, ne.fronts, ne.sms, up,
+                         down, s);
+  // Side by side: the few in wider arithmetic on a stream of their own, with the SMs that the
+  // others leave at one block per SM (all, where those take a launch per level).
+  const cudaStream_t ws = ne.wide ? ne.wide : e.side;
+  err = cudaEventRecord(ne.ev_wide, s);
+  if (err == cudaSuccess) err = cudaStreamWaitEvent(ws, ne.ev_wide, 0);
+  if (err != cudaSuccess) return cuda_fail(err, "fork");
+  const int others = e.B - nw, free_sms = ne.sms - (others <= ne.sms ? others : 0);
+  int c = 1;
+  while (c < 8 && 2 * c * nw <= free_sms) c *= 2;
+  sca_status st = run_blocks_in(groups[0].ar, e, la, 0, nw, ne.fronts, free_sms, up, down, ws);
+  if (st == SCA_OK)
+    st = run_blocks_in(groups[1].ar, e, la, nw, others, ne.fronts + groups[0].bytes,
+                       std::max(1, ne.sms - c * nw), up, down, s);
+  if (st != SCA_OK) return st;
+  err = cudaEventRecord(ne.ev_wide, ws);
+  if (err == cudaSuccess) err = cudaStreamWaitEvent(s, ne.ev_wide, 0);
+  if (err != cudaSuccess) return cuda_fail(err, "join");
+  return SCA_OK;
 }
 
 }  // namespace sca

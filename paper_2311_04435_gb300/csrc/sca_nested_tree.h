@@ -11,8 +11,9 @@
 // checkerboard colour couple only to the other colour and to the boundary: those ("blacks") can be
 // eliminated in closed form, which leaves the other colour as the node's pivots.
 //
-// A black is a pivot of modulus |A_bb|, which can be as small as w_n, while the leaf's block as a
-// whole is far better conditioned.  The tree therefore has two forms with the same nodes, which
+// A black is a pivot of modulus |A_bb|, which can be as small as w_n, while on disordered fields the
+// leaf's block as a whole is far better conditioned (on weak ones it has levels near zero too: see
+// the arithmetics in sca_internal.h).  The tree therefore has two forms with the same nodes, which
 // differ in the leaves only: `dense_leaves` (every site of a leaf is a pivot of its front), for
 // blocks without column dominance (w_n <= 4|t|), and the closed form for the others.  In float64
 // on random site energies in [-1, 1] (t = 1, L = 14 and 18) the largest error of G_ii is, dense
@@ -132,7 +133,7 @@ class Builder {
           n.adj = (int)t.table.size();
           for (int i = 0; i < m; ++i) t.table.push_back((int16_t)adj[i]);
         }
-        // (a leaf is one panel: its block as a whole is well conditioned, parts of it are not)
+        // (a leaf is one panel)
         const int pw = panel_width(m);
         n.npan = (n.p + pw - 1) / pw;
         n.pw = n.npan ? (n.p + n.npan - 1) / n.npan : 0;
