@@ -339,28 +339,29 @@ sca_status sca_metropolis_init(sca_ctx* ctx, const double* phi0_host, double del
 sca_status sca_metropolis_step(sca_ctx* ctx, int32_t n_steps, double* omega_trace,
                                uint8_t* accepted, double* omega, int64_t* accepted_total);
 
-/* Pivoting of the elimination of the A_{n,sigma} (Sec. II, Eq. 2).  A new context takes the nested
- * elimination where it applies (no interchanges: -i A and all its Schur complements have the
- * Hermitian part omega_n I > 0) and SCA_PIVOT_PARTIAL elsewhere.
- *   SCA_PIVOT_PARTIAL: the dense elimination, with partial pivoting for the blocks whose column diagonal
- *     dominance is not guaranteed (omega_n <= 4|t|); the remaining blocks provably keep their
- *     diagonal pivots and skip the search.
+/* Pivoting of the elimination of the A_{n,sigma} (Sec. II, Eq. 2).
+ *   SCA_PIVOT_AUTO (a new context's): the nested elimination where it applies (no interchanges:
+ *     -i A and all its Schur complements have the Hermitian part omega_n I > 0), elsewhere the
+ *     dense elimination with partial pivoting.
+ *   SCA_PIVOT_PARTIAL: always the dense elimination, with partial pivoting for the blocks whose
+ *     column diagonal dominance is not guaranteed (omega_n <= 4|t|); the remaining blocks provably
+ *     keep their diagonal pivots and skip the search.
  *   SCA_PIVOT_NONE: every block is eliminated without interchanges: nested where it applies,
  *     elsewhere as a dense complex-symmetric (LDL^T-type) elimination that updates one
- *     triangle on the tensor-core path.  The paper has no such variant.  -i A_{n,sigma} has Hermitian part omega_n I > 0, so every leading
- *     principal minor is nonzero and the elimination exists; its growth has no a-priori bound
- *     and rises as omega_n falls (the largest growth met in tests is below 10, down to
+ *     triangle on the tensor-core path.  The paper has no such variant.  -i A_{n,sigma} has
+ *     Hermitian part omega_n I > 0, so every leading principal minor is nonzero and the
+ *     elimination exists; its growth has no a-priori bound and rises as omega_n falls (the largest growth met in tests is below 10, down to
  *     T = 0.02).  The fused small-block path (N <= 144) always pivots.
  * Applies from the next call on the context; any other mode is SCA_EINVAL. */
-typedef enum { SCA_PIVOT_PARTIAL = 0, SCA_PIVOT_NONE = 1 } sca_pivot;
+typedef enum { SCA_PIVOT_PARTIAL = 0, SCA_PIVOT_NONE = 1, SCA_PIVOT_AUTO = 2 } sca_pivot;
 sca_status sca_set_pivoting(sca_ctx* ctx, int32_t mode);
 
 /* Arithmetic of the pivoted blocks' panel factorisation (the sub-panel LU with its pivot search,
  * the interchanges with U12 and the rest-of-panel update) on the reduced-precision paths:
  * SCA_PREC_FP32 (default: the blocks' compute type) or SCA_PREC_FP64 (float64 arithmetic on
  * the float32 blocks; the doubled shared-memory panel narrows the sub-panels, e.g. to 4
- * columns at N = 1600) takes the dense elimination.  The pivot-block inverses and the
- * contractions are unchanged.  Float64 contexts accept only SCA_PREC_FP64.  Applies from the
+ * columns at N = 1600).  While SCA_PREC_FP64 is set on them, the context takes the dense
+ * elimination.  The pivot-block inverses and the contractions are unchanged.  Float64 contexts accept only SCA_PREC_FP64.  Applies from the
  * next call; SCA_EINVAL otherwise. */
 sca_status sca_set_panel_precision(sca_ctx* ctx, int32_t prec);
 

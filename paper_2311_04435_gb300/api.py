@@ -251,10 +251,11 @@ class Context:
         check(_lib.lib().sca_set_wait_limit(self._h, int(cycles)))
 
     def set_pivoting(self, mode: str = "partial"):
-        """'partial': dense elimination, partial pivoting where diagonal dominance is not
-        guaranteed; 'none': no interchanges (nested elimination where it applies, as in a new
-        context; else a dense complex-symmetric elimination)."""
-        modes = {"partial": 0, "none": 1}
+        """'auto' (a new context's): nested elimination where it applies, else dense with partial
+        pivoting; 'partial': dense elimination, partial pivoting where diagonal dominance is not
+        guaranteed; 'none': no interchanges (nested elimination where it applies, else a dense
+        complex-symmetric elimination)."""
+        modes = {"partial": 0, "none": 1, "auto": 2}
         if mode not in modes:
             raise ValueError(f"pivoting mode must be one of {sorted(modes)}")
         check(_lib.lib().sca_set_pivoting(self._h, modes[mode]))

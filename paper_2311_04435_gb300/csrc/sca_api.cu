@@ -123,7 +123,9 @@ static bool dense_switch_set() {
 }
 
 bool nested_now(const Engine& e) {
-  if (!e.nest || e.dense_only || (e.prof && e.prof->on && e.prof->dense)) return false;
+  if (!e.nest || e.dense_switch || e.dense_pivoting || e.panel_fp64 ||
+      (e.prof && e.prof->on && e.prof->dense))
+    return false;
   return e.dos_mode ? nested_rule(e.p.t, e.dos_eta, e.dos_eta) : e.nest_rule;
 }
 
@@ -193,7 +195,7 @@ sca_status plan(const sca_params& p, Engine& e) {
     if (std::atoi(v) == 0) e.pair = false;
   e.nest_rule = nested_rule(p.t, M_PI * p.T, (2.0 * p.n_omega - 1.0) * M_PI * p.T);
   e.nest_wide = nested_wide_blocks(e.fp64, p.L, p.t, p.T, p.n_omega);
-  e.dense_only = dense_switch_set();
+  e.dense_switch = dense_switch_set();
   size_t bytes = 0;
   bytes += (size_t)e.chunk * e.mat_stride * S;           // blocks
   bytes += 2 * (size_t)e.chunk * e.fw_mat * S;            // F, W
@@ -936,13 +938,13 @@ sca_status sca_set_wait_limit(sca_ctx* c, int64_t cycles) {
 }
 
 sca_status sca_set_pivoting(sca_ctx* c, int32_t mode) {
-  if (!c || (mode != SCA_PIVOT_PARTIAL && mode != SCA_PIVOT_NONE)) {
+  if (!c || (mode != SCA_PIVOT_PARTIAL && mode != SCA_PIVOT_NONE && mode != SCA_PIVOT_AUTO)) {
     set_error("bad context or pivoting mode");
     return SCA_EINVAL;
   }
   c->e.piv_blocks = (mode == SCA_PIVOT_NONE) ? 0 : c->e.piv_planned;
   c->e.nopiv = (mode == SCA_PIVOT_NONE);
-  c->e.dense_only = mode == SCA_PIVOT_PARTIAL || dense_switch_set();
+  c->e.dense_pivoting = mode == SCA_PIVOT_PARTIAL;
   return SCA_OK;
 }
 
@@ -954,7 +956,6 @@ sca_status sca_set_panel_precision(sca_ctx* c, int32_t prec) {
     return SCA_EINVAL;
   }
   c->e.panel_fp64 = !c->e.fp64 && prec == SCA_PREC_FP64;
-  if (c->e.panel_fp64) c->e.dense_only = true;
   return SCA_OK;
 }
 

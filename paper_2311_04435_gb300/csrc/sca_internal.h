@@ -132,13 +132,14 @@ struct Engine {
   double* d_omega = nullptr;    // 1 double scratch
   double* h_status = nullptr;   // pinned 8 doubles
   // nested elimination (sca_nested.cu): its fronts use M.  nest_rule: the smallest omega_n
-  // admits it; dense_only: the caller or an environment switch chose the dense elimination's
-  // options; fronts_kept: the last pass left fronts (not dense inverses) in M.
+  // admits it; dense_switch: the context was created under one of the dense elimination's
+  // environment switches; dense_pivoting: SCA_PIVOT_PARTIAL was asked for; fronts_kept: the last pass left fronts (not dense inverses) in M.
   Nested* nest = nullptr;
   bool nest_rule = false;
   int nest_dense = 0;       // leading blocks without column dominance (dense leaves)
   int nest_wide = 0;        // ... and those in wider arithmetic
-  bool dense_only = false;
+  bool dense_switch = false;
+  bool dense_pivoting = false;
   bool fronts_kept = false;
   double dos_eta = 0.0;
   void* tmap = nullptr;         // host-side tensor-map storage (tc path)
