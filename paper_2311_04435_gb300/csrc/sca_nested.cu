@@ -487,6 +487,33 @@ __device__ __forceinline__ Zw zinv(Zw z, double* mag2 = nullptr) {
   return r;
 }
 
+// 1 / z for any z.  The float32 forms above square z within float32's range (no pivot is too
+// small: each is at least Im z >= 1e-9 in modulus); a larger one, which a site term makes, goes
+// through float64 (53 bits are enough there: what it couples with is 2^-60 of it or less).
+template <typename Z>
+constexpr bool kNarrow = std::is_same<Z, Zf>::value || std::is_same<Z, Zt>::value;
+__device__ __forceinline__ bool beyond(double x) {  // |x| >= 2^60, without the slow pipe
+  return (__double2hiint(x) & 0x7fffffff) >= 0x43b00000;
+}
+__device__ __forceinline__ bool beyond(Zf z) { return fmaxf(fabsf(z.rh), fabsf(z.ih)) >= 0x1p60f; }
+__device__ __forceinline__ bool beyond(Zt z) {
+  float r, i;
+  f2_get(z.h, r, i);
+  return fmaxf(fabsf(r), fabsf(i)) >= 0x1p60f;
+}
+__device__ __forceinline__ bool beyond(Zd) { return false; }
+__device__ __forceinline__ bool beyond(Zw) { return false; }
+template <typename Z>
+__device__ __forceinline__ Z zinv_any(Z z, double* mag2 = nullptr) {
+  if (!beyond(z)) return zinv(z, mag2);
+  const double re = zre(z), im = zim(z);
+  const double m = fma(im, im, __dmul_rn(re, re)), d = 1.0 / m;
+  if (mag2) *mag2 = m;
+  Z r;
+  zset(r, re * d, -im * d);
+  return r;
+}
+
 // A product of moduli squared as mantissa in [1, 2) and exponent: a node's share of |det A|^2.
 // One logarithm per node at the root instead of one per pivot (a float64 logarithm costs about
 // 40 instructions of the slowest pipe of this GPU).
@@ -621,6 +648,18 @@ struct Group {
     else
       asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(size) : "memory");
   }
+  // The same, and whether q holds in any of the threads.
+  __device__ __forceinline__ bool sync_any(bool q) const {
+    if (size == 32) return __any_sync(0xffffffffu, q);
+    int r;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\tsetp.ne.s32 p, %3, 0;\n\tbar.red.or.pred q, %1, %2, p;\n\t"
+        "selp.s32 %0, 1, 0, q;\n\t}"
+        : "=r"(r)
+        : "r"(bar), "r"(size), "r"((int)q)
+        : "memory");
+    return r != 0;
+  }
 };
 
 // Offset of a pointer into the CTA's dynamic shared memory.
@@ -652,8 +691,9 @@ struct Block {
 // (g, j), (g + G, j), ... of the w x w block, S of them, G = size / w.  A step needs the pivot's
 // row, its column and its reciprocal; their owners write them to shared memory as soon as they
 // have them (two buffers, one barrier per step).  The result replaces F11, negated, and goes to
-// the front.
-template <typename Z, int S>
+// the front.  kAny: a pivot may be beyond 2^60 (a check inside the chain of pivots costs 2 to 4 %,
+// so fronts without such a site term take the form without).
+template <typename Z, int S, bool kAny>
 __device__ __noinline__ void invert(const Group gr, int w, int F11o, int rowo, int colo,
                                     int mago, Z* Fo, int m) {
   using Acc = typename AccOf<Z>::type;
@@ -677,7 +717,7 @@ __device__ __noinline__ void invert(const Group gr, int w, int F11o, int rowo, i
 #pragma unroll
       for (int s = 0; s < S; ++s) colb[row[s]] = zneg(reg[s]);
     }
-    if (gr.tid == 0) colb[w] = zinv(reg[0], mag);
+    if (gr.tid == 0) colb[w] = kAny ? zinv_any(reg[0], mag) : zinv(reg[0], mag);
   }
 #pragma unroll 1
   for (int c = 0; c < w; ++c) {
@@ -704,7 +744,7 @@ __device__ __noinline__ void invert(const Group gr, int w, int F11o, int rowo, i
 #pragma unroll
         for (int s = 1; s < S; ++s) nr = zsel(row[s] == c + 1, reg[s], nr);
         rn[j] = nr;
-        if (j == c + 1) cn[w] = zinv(nr, mag + j);
+        if (j == c + 1) cn[w] = kAny ? zinv_any(nr, mag + j) : zinv(nr, mag + j);
       }
       if (j == c + 1) {
 #pragma unroll
@@ -886,9 +926,12 @@ __device__ __forceinline__ void front_up(const Block<Z>& B, int node, const Grou
     cm0[i] = nd.child[0] >= 0 ? B.tab[nd.cmap[0] + i] : (int16_t)-1;
     cm1[i] = nd.child[1] >= 0 ? B.tab[nd.cmap[1] + i] : (int16_t)-1;
   }
-  for (int i = tid; i <= p; i += size)
-    zset(diag[i], i < p ? B.zr - site_energy(B.la, B.tab[nd.sites + i], B.sg) : B.la.t,
-         i < p ? B.zi : 0.0);
+  bool big = false;
+  for (int i = tid; i <= p; i += size) {
+    const double re = i < p ? B.zr - site_energy(B.la, B.tab[nd.sites + i], B.sg) : B.la.t;
+    zset(diag[i], re, i < p ? B.zi : 0.0);
+    big |= beyond(re);
+  }
   if (nd.blacks) {
     for (int i = tid; i < m; i += size) adj[i] = B.tab[nd.adj + i];
     if (tid < 32) {
@@ -897,7 +940,7 @@ __device__ __forceinline__ void front_up(const Block<Z>& B, int node, const Grou
         Z z, t2;
         zset(z, B.zr - site_energy(B.la, B.tab[nd.bsite + tid], B.sg), B.zi);
         zset(t2, B.la.t * B.la.t, 0.0);
-        bt[tid] = zneg(zmul(t2, zinv(z, &m2)));
+        bt[tid] = zneg(zmul(t2, zinv_any(z, &m2)));
       }
       det_mul(m2, mant, expo, B.flags);
     }
@@ -922,7 +965,10 @@ __device__ __forceinline__ void front_up(const Block<Z>& B, int node, const Grou
   f.adj = off(adj);
   f.bt = off(bt);
   f.diag = off(diag);
-  gr.sync();
+  if constexpr (kNarrow<Z>)
+    big = gr.sync_any(big);
+  else
+    gr.sync();
   for (int pa = 0; pa < nd.npan; ++pa) {
     const int o = pa * pw, w = min(pw, p - o), l = m - o, r = l - w;
     const int lda = r + kRows;  // row blocks read up to kRows - 1 entries past r
@@ -939,10 +985,12 @@ __device__ __forceinline__ void front_up(const Block<Z>& B, int node, const Grou
       }
     gr.sync();
     Z* Fo = F + (size_t)o * (m + 1);
-    if (w <= size / w)
-      invert<Z, 1>(gr, w, off(F11), off(rowb), off(colb), off(mag), Fo, m);
+    if (kNarrow<Z> && big)
+      invert<Z, kSlots, true>(gr, w, off(F11), off(rowb), off(colb), off(mag), Fo, m);
+    else if (w <= size / w)
+      invert<Z, 1, false>(gr, w, off(F11), off(rowb), off(colb), off(mag), Fo, m);
     else
-      invert<Z, kSlots>(gr, w, off(F11), off(rowb), off(colb), off(mag), Fo, m);
+      invert<Z, kSlots, false>(gr, w, off(F11), off(rowb), off(colb), off(mag), Fo, m);
     gr.sync();
     if (r > 0)
       times_fit<Z, false, 0>(gr, w, w, r, off(F11), w, off(X), r, (const Z*)F, off(A), lda, 0,
@@ -1070,7 +1118,7 @@ __device__ __forceinline__ void front_down(const Block<Z>& B, int node, const Gr
         Z z, t2;
         zset(z, B.zr - site_energy(B.la, s, B.sg), B.zi);
         zset(t2, B.la.t * B.la.t, 0.0);
-        const Z ai = zinv(z);
+        const Z ai = zinv_any(z);
         const Z g = zadd(ai, zmul(zmul(zmul(ai, t2), ai), sum));
         B.gd[s] = B.la.zshift ? zim(g) : B.sg * zre(g);
       }
@@ -1120,7 +1168,7 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : 1) k_nested(NestArgs<Z> a)
   if (a.range) {
     int big = 0;
     for (int i = tid; i < B.la.N; i += NT)
-      if (!(fabs(B.zr - site_energy(B.la, i, B.sg)) < 0x1p60)) big = 1;
+      if (beyond(B.zr - site_energy(B.la, i, B.sg))) big = 1;
     if (__syncthreads_or(big) != (a.range == 2)) return;  // (alike in all CTAs of a block)
   }
   for (int k = a.k0; k < a.k1; ++k) {
