@@ -29,7 +29,8 @@
 // takes no longer than one of float64 does here: a 20x20 float64 density of states 1013 us in float64,
 // 1004 in these, 11324 in double-double).  They go beside the others, on a stream of their own, in
 // clusters of up to eight CTAs per block: a 20x20 gradient, T = 0.05, 124 blocks in float64 and 4 in
-// these, 1009 us, 1004 with all 128 in float64; 512 blocks, T = 0.1, 2 of them in these, 2291 / 2251.
+// these, 1009 us, 1004 with all 128 in float64; 512 blocks, T = 0.1, 2 of them in these, 2273 / 2264
+// (2296 with clusters of eight where the others take longer than one block's time per SM).
 // On small lattices their dependent chain shows: 8x8 densities of states 287 us, 151 in float64.
 //
 // Work split: a group of threads per front (a warp for the smallest, 256 or 512 threads for the
@@ -1330,7 +1331,8 @@ sca_status launch(Engine& e, const NestArgs<Z>& a, int cnt, size_t smem, cudaStr
 // SMs are for them.
 template <typename Z>
 sca_status run_blocks_of(Engine& e, const Lattice& la, int b0, int cnt, char* mem, size_t bytes,
-                         int free_sms, bool up, bool down, cudaStream_t s, int range = 0) {
+                         int free_sms, bool up, bool down, cudaStream_t s, int max_cluster,
+                         int range = 0) {
   const Nested& ne = *e.nest;
   NestArgs<Z> a;
   a.nodes = ne.d_nodes;
@@ -1410,7 +1412,7 @@ sca_status run_blocks_of(Engine& e, const Lattice& la, int b0, int cnt, char* me
     a.k0 = p0;
     a.k1 = p1;
     a.csize = 1;
-    while (a.csize < 8 && 2 * a.csize * cnt <= free_sms) a.csize *= 2;
+    while (2 * a.csize <= max_cluster && 2 * a.csize * cnt <= free_sms) a.csize *= 2;
     const size_t smem = plan_levels(ne, a);
     st = a.csize > 1 ? launch<Z, 512, true>(e, a, cnt, smem, s)
                      : launch<Z, 512, false>(e, a, cnt, smem, s);
@@ -1426,18 +1428,19 @@ sca_status run_blocks_of(Engine& e, const Lattice& la, int b0, int cnt, char* me
 }
 
 sca_status run_blocks_in(NestedArith ar, Engine& e, const Lattice& la, int b0, int cnt, char* mem,
-                         int free_sms, bool up, bool down, cudaStream_t s) {
+                         int free_sms, bool up, bool down, cudaStream_t s, int max_cluster = 8) {
   const size_t by = e.nest->front_bytes(ar);
+  const int mc = max_cluster;
   if (ar == NestedArith::kFloat2)
-    return run_blocks_of<Zf>(e, la, b0, cnt, mem, by, free_sms, up, down, s);
+    return run_blocks_of<Zf>(e, la, b0, cnt, mem, by, free_sms, up, down, s, mc);
   if (ar == NestedArith::kFloat64)
-    return run_blocks_of<Zd>(e, la, b0, cnt, mem, by, free_sms, up, down, s);
+    return run_blocks_of<Zd>(e, la, b0, cnt, mem, by, free_sms, up, down, s, mc);
   if (ar == NestedArith::kWide32)
-    return run_blocks_of<Zt>(e, la, b0, cnt, mem, by, free_sms, up, down, s);
+    return run_blocks_of<Zt>(e, la, b0, cnt, mem, by, free_sms, up, down, s, mc);
   // a float64 context: entries beyond float32's range take double-double (a launch that ends at
   // once where there are none)
-  sca_status st = run_blocks_of<Zt>(e, la, b0, cnt, mem, by, free_sms, up, down, s, 1);
-  if (st == SCA_OK) st = run_blocks_of<Zw>(e, la, b0, cnt, mem, by, free_sms, up, down, s, 2);
+  sca_status st = run_blocks_of<Zt>(e, la, b0, cnt, mem, by, free_sms, up, down, s, mc, 1);
+  if (st == SCA_OK) st = run_blocks_of<Zw>(e, la, b0, cnt, mem, by, free_sms, up, down, s, mc, 2);
   return st;
 }
 
@@ -1599,15 +1602,18 @@ sca_status run_nested(Engine& e, const Lattice& la, bool up, bool down, cudaStre
     return run_blocks_in(groups[0].ar, e, la, groups[0].first, groups[0].n, ne.fronts, ne.sms, up,
                          down, s);
   // Side by side: the few in wider arithmetic on a stream of their own, with the SMs that the
-  // others leave at one block per SM (all, where those take a launch per level).
+  // others leave at one block per SM.  Where those take a launch per level, over several blocks' time
+  // per SM, clusters are smaller by as much.
   const cudaStream_t ws = ne.wide ? ne.wide : e.side;
   err = cudaEventRecord(ne.ev_wide, s);
   if (err == cudaSuccess) err = cudaStreamWaitEvent(ws, ne.ev_wide, 0);
   if (err != cudaSuccess) return cuda_fail(err, "fork");
   const int others = e.B - nw, free_sms = ne.sms - (others <= ne.sms ? others : 0);
+  const int max_cluster = others <= ne.sms ? 8 : std::max(1, 8 * ne.sms / others);
   int c = 1;
-  while (c < 8 && 2 * c * nw <= free_sms) c *= 2;
-  sca_status st = run_blocks_in(groups[0].ar, e, la, 0, nw, ne.fronts, free_sms, up, down, ws);
+  while (2 * c <= max_cluster && 2 * c * nw <= free_sms) c *= 2;
+  sca_status st =
+      run_blocks_in(groups[0].ar, e, la, 0, nw, ne.fronts, free_sms, up, down, ws, max_cluster);
   if (st == SCA_OK)
     st = run_blocks_in(groups[1].ar, e, la, nw, others, ne.fronts + groups[0].bytes,
                        std::max(1, ne.sms - c * nw), up, down, s);
