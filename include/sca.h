@@ -224,9 +224,10 @@ sca_status sca_solve(const sca_params* params, const sca_adam* adam, const doubl
  * while others run (continuous batching).  Requests whose blocks exceed the
  * fused kernel's size (N > 144; FP64: N > 64) are batched by size bucket: those
  * with the same L and precision share one workspace of up to 256 block slots
- * (counted against the budget while the bucket has requests; then kept up to 10 s,
- * within the budget, for the next one of its size) and one launch sequence per
- * step.  A request's result is the same bit for bit as with sca_solve.  Errors: SCA_EINVAL, SCA_ENOMEM, SCA_ECUDA. */
+ * (counted against the budget while the bucket has requests; then kept up to a second
+ * of real time, within the budget, for the next one of its size, and freed earlier if an
+ * allocation of this library fails) and one launch sequence per step.  A request's result
+ * is the same bit for bit as with sca_solve.  Errors: SCA_EINVAL, SCA_ENOMEM, SCA_ECUDA. */
 sca_status sca_server_create(uint64_t hbm_budget_bytes, int32_t max_slots, sca_server** out);
 
 /* Queues a solve request (parameters and Adam settings are copied; phi0 is

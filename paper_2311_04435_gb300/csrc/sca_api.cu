@@ -75,6 +75,15 @@ sca_status cuda_fail(cudaError_t e, const char* where) {
   return SCA_ECUDA;
 }
 
+cudaError_t device_malloc(void** p, size_t bytes) {
+  cudaError_t err = cudaMalloc(p, bytes);
+  if (err == cudaErrorMemoryAllocation && drop_idle_workspaces()) {
+    (void)cudaGetLastError();
+    err = cudaMalloc(p, bytes);
+  }
+  return err;
+}
+
 static sca_status validate(const sca_params* p) {
   if (!p) { set_error("params is NULL"); return SCA_EINVAL; }
   if (p->L < 2 || p->L > 64 || (p->L & 1)) {
@@ -212,7 +221,7 @@ sca_status plan(const sca_params& p, Engine& e) {
 
 template <typename T>
 static sca_status dev_alloc(T** p, size_t bytes, Engine& e, const char* what) {
-  cudaError_t err = cudaMalloc((void**)p, std::max<size_t>(bytes, 16));
+  cudaError_t err = device_malloc((void**)p, std::max<size_t>(bytes, 16));
   if (err != cudaSuccess) {
     (void)cudaGetLastError();
     release(e);
@@ -505,7 +514,7 @@ sca_status sca_create(const sca_params* params, sca_ctx** out) {
   if (!c) { set_error("host allocation failed"); return SCA_ENOMEM; }
   plan(*params, c->e);
   if ((st = allocate(c->e)) != SCA_OK) { delete c; return st; }
-  cudaError_t err = cudaMalloc((void**)&c->d_in, sizeof(double) * c->e.N);
+  cudaError_t err = device_malloc((void**)&c->d_in, sizeof(double) * c->e.N);
   if (err != cudaSuccess) { release(c->e); delete c; return cuda_fail(err, "cudaMalloc phi"); }
   err = cudaStreamCreateWithFlags(&c->own, cudaStreamNonBlocking);
   c->stream = c->own;
@@ -539,7 +548,7 @@ sca_status sca_set_site_energy(sca_ctx* c, const double* eps_extra_host) {
     return SCA_OK;
   }
   cudaError_t err = cudaSuccess;
-  if (!c->e.eps_extra) err = cudaMalloc((void**)&c->e.eps_extra, sizeof(double) * c->e.N);
+  if (!c->e.eps_extra) err = device_malloc((void**)&c->e.eps_extra, sizeof(double) * c->e.N);
   if (err == cudaSuccess)
     err = cudaMemcpy(c->e.eps_extra, eps_extra_host, sizeof(double) * c->e.N, cudaMemcpyHostToDevice);
   if (err != cudaSuccess) return cuda_fail(err, "site energy upload");

@@ -64,9 +64,9 @@ sca_status ensure_tables(Bucket* b, int passes, int steps) {
   steps = std::max(steps, b->steps);
   free_tables(b);
   const size_t nbd = (size_t)passes * b->cap, nreq = (size_t)passes * steps * b->rmax;
-  err = cudaMalloc((void**)&b->d_bd, sizeof(BlockDesc) * nbd);
-  if (err == cudaSuccess) err = cudaMalloc((void**)&b->d_slots, sizeof(int) * nbd);
-  if (err == cudaSuccess) err = cudaMalloc((void**)&b->d_req, sizeof(ReqDesc) * nreq);
+  err = device_malloc((void**)&b->d_bd, sizeof(BlockDesc) * nbd);
+  if (err == cudaSuccess) err = device_malloc((void**)&b->d_slots, sizeof(int) * nbd);
+  if (err == cudaSuccess) err = device_malloc((void**)&b->d_req, sizeof(ReqDesc) * nreq);
   if (err == cudaSuccess) err = cudaMallocHost((void**)&b->h_bd, sizeof(BlockDesc) * nbd);
   if (err == cudaSuccess) err = cudaMallocHost((void**)&b->h_slots, sizeof(int) * nbd);
   if (err == cudaSuccess) err = cudaMallocHost((void**)&b->h_req, sizeof(ReqDesc) * nreq);
@@ -133,7 +133,7 @@ sca_status bucket_req_init(Bucket* b, BucketReq* r, const sca_params& p, const s
   r->nested = nested_rule(p.t, M_PI * p.T, (2.0 * p.n_omega - 1.0) * M_PI * p.T);
   r->wide = nested_wide_blocks(p.prec == SCA_PREC_FP64, p.L, p.t, p.T, p.n_omega);
   r->delta_eff = (p.ionic == SCA_IONIC_HALF) ? 0.5 * p.delta : p.delta;
-  cudaError_t err = cudaMalloc((void**)&r->d, sizeof(double) * (4 * (size_t)N + 8));
+  cudaError_t err = device_malloc((void**)&r->d, sizeof(double) * (4 * (size_t)N + 8));
   if (err != cudaSuccess) { r->d = nullptr; return cuda_fail(err, "request state"); }
   cudaStream_t s = b->ctx->stream;
   sca_status st = run_seed_phi(r->d, N, a.seed, s);

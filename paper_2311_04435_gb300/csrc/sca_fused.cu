@@ -529,7 +529,7 @@ sca_status fused_prepare(Engine& e) {
   // as long) and for the smallest blocks
   e.fused_grid = std::min(e.B, (e.N <= 16 || e.fp64 ? 1 : per) * sms);
   e.fused_smem = sm;
-  if ((err = cudaMalloc((void**)&e.fused_bar, 2 * sizeof(unsigned))) != cudaSuccess)
+  if ((err = device_malloc((void**)&e.fused_bar, 2 * sizeof(unsigned))) != cudaSuccess)
     return cuda_fail(err, "fused barrier");
   if ((err = cudaMemset(e.fused_bar, 0, 2 * sizeof(unsigned))) != cudaSuccess)
     return cuda_fail(err, "fused barrier");

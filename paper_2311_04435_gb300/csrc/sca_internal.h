@@ -59,6 +59,12 @@ extern std::atomic<uint64_t> g_launches;
 void set_error(const std::string& msg);
 sca_status cuda_fail(cudaError_t e, const char* where);
 
+// Frees the workspaces that the current device's servers keep for requests to come; false if there
+// were none.
+bool drop_idle_workspaces();
+// cudaMalloc; on failure once more after drop_idle_workspaces().
+cudaError_t device_malloc(void** p, size_t bytes);
+
 // Arguments of one Adam update (PyTorch's order and bias corrections).
 struct AdamStep {
   double lr_over_bc1, sqrt_bc2, beta1, beta2, eps, grad_tol;

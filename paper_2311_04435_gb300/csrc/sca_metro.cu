@@ -103,8 +103,8 @@ __global__ void __launch_bounds__(MT)
 
 sca_status ensure_buffers(sca_ctx* c, int32_t trace_steps) {
   cudaError_t err = cudaSuccess;
-  if (!c->d_prop) err = cudaMalloc((void**)&c->d_prop, sizeof(double) * c->e.N);
-  if (err == cudaSuccess && !c->d_metro) err = cudaMalloc((void**)&c->d_metro, 4 * sizeof(double));
+  if (!c->d_prop) err = device_malloc((void**)&c->d_prop, sizeof(double) * c->e.N);
+  if (err == cudaSuccess && !c->d_metro) err = device_malloc((void**)&c->d_metro, 4 * sizeof(double));
   if (err == cudaSuccess && trace_steps > c->mtrace_cap) {
     if (c->d_mtrace) {
       cudaStreamSynchronize(c->stream);
@@ -112,7 +112,7 @@ sca_status ensure_buffers(sca_ctx* c, int32_t trace_steps) {
       c->d_mtrace = nullptr;
       c->mtrace_cap = 0;
     }
-    err = cudaMalloc((void**)&c->d_mtrace, sizeof(double) * 2 * (size_t)trace_steps);
+    err = device_malloc((void**)&c->d_mtrace, sizeof(double) * 2 * (size_t)trace_steps);
     if (err == cudaSuccess) c->mtrace_cap = trace_steps;
   }
   if (err != cudaSuccess) return cuda_fail(err, "Metropolis buffers");

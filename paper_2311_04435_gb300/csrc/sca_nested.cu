@@ -1519,12 +1519,12 @@ sca_status nested_prepare(Engine& e) {
   ne->fronts = static_cast<char*>(e.M);
   ne->room = e.block_room;
   if (need > ne->room) {
-    err = cudaMalloc(&ne->own, need);
+    err = device_malloc(&ne->own, need);
     ne->fronts = static_cast<char*>(ne->own);
     ne->room = need;
   }
-  if (err == cudaSuccess) err = cudaMalloc((void**)&ne->d_nodes, sizeof(Node) * t.nodes.size());
-  if (err == cudaSuccess) err = cudaMalloc((void**)&ne->d_tab, sizeof(int16_t) * t.table.size());
+  if (err == cudaSuccess) err = device_malloc((void**)&ne->d_nodes, sizeof(Node) * t.nodes.size());
+  if (err == cudaSuccess) err = device_malloc((void**)&ne->d_tab, sizeof(int16_t) * t.table.size());
   if (err != cudaSuccess) {
     nested_release(e);
     (void)cudaGetLastError();

@@ -27,6 +27,7 @@
 #include <mutex>
 #include <new>
 #include <string>
+#include <system_error>
 #include <thread>
 #include <unordered_map>
 #include <vector>
@@ -38,10 +39,11 @@ namespace {
 constexpr int32_t kRoundSteps = 8;     // Adam iterations enqueued per request per round
 constexpr int kBucketSlots = 256;      // block slots of a size bucket's workspace
 // How long the workspace of a bucket that has lost its last request waits for another of its
-// size.  Allocating and freeing one takes milliseconds (L = 32, 256 slots: 1.7 and 4.5 ms,
-// against 6.3 ms for all nine evaluations of two requests); in a served mix of 12 requests of
-// six sizes that was 12 of 28 ms.
-constexpr double kIdleSeconds = 10.0;
+// size, in real time.  Allocating and freeing one takes milliseconds (L = 32, 256 slots: 1.7 and
+// 4.5 ms, against 6.3 ms for all nine evaluations of two requests); in a served mix of 12 requests of
+// six sizes that was 12 of 28 ms.  After a second without a request they are less than a hundredth
+// of the time, and the memory is of more use elsewhere.
+constexpr double kIdleSeconds = 1.0;
 
 uint64_t bucket_bytes(int32_t L, int32_t prec, int cap) {
   const sca_params s = sca::bucket_shape(L, prec, cap);
@@ -84,16 +86,26 @@ struct BucketSlot {
   int members = 0;           // admitted requests not yet finished
 };
 
-// The workspace of a bucket without requests: freed after kIdleSeconds, or as soon as it and the
-// admitted requests together would exceed the budget, oldest first.  It counts for nothing in
-// `used`, so admission does not depend on it.
+// The workspace of a bucket without requests: freed after kIdleSeconds (by the worker thread, or
+// on a manual server by a thread of its own, whether or not it is stepped again), as soon as it and
+// the admitted requests together would exceed the budget, oldest first, or when an allocation of
+// this library fails in any thread.  It counts for nothing in `used`, so admission does not depend
+// on it.
 struct IdleBucket {
   std::pair<int32_t, int32_t> key;
   sca::Bucket* b;
   int cap;
   uint64_t bytes;
-  double since;
+  std::chrono::steady_clock::time_point since;
 };
+
+static std::chrono::steady_clock::duration idle_time() {
+  return std::chrono::duration_cast<std::chrono::steady_clock::duration>(
+      std::chrono::duration<double>(kIdleSeconds));
+}
+static bool expired(const IdleBucket& k) {
+  return std::chrono::steady_clock::now() - k.since >= idle_time();
+}
 
 struct sca_server {
   uint64_t budget = 0;
@@ -106,7 +118,11 @@ struct sca_server {
   std::vector<Request*> active;  // worker-owned
   std::unordered_map<uint64_t, Request*> all;
   std::map<std::pair<int32_t, int32_t>, BucketSlot> buckets;  // (L, prec); under the mutex
-  std::vector<IdleBucket> idle;  // oldest first; only the thread that runs the rounds uses it
+  std::mutex idle_mu;            // taken after `mu` where both are held; nothing allocates under it
+  std::vector<IdleBucket> idle;  // oldest first
+  std::condition_variable idle_cv;
+  std::thread reaper;            // manual servers: frees idle workspaces in time
+  bool reaper_stop = false;
   uint64_t next_id = 1;
   bool stop = false;
   std::thread worker;
@@ -123,12 +139,15 @@ struct sca_server {
   sca::Bucket* take_idle(std::pair<int32_t, int32_t> key, int cap);
   void trim_idle();
   bool drop_idle();
+  void keep_idle(const IdleBucket& k);
+  void reap();
   void finish(Request* r, sca_status st);
   void run_buckets(std::vector<Request*>& active, std::vector<Request*>& still);
 };
 
 // The idle workspace of this size and slot count, if there is one.
 sca::Bucket* sca_server::take_idle(std::pair<int32_t, int32_t> key, int cap) {
+  std::lock_guard<std::mutex> lock(idle_mu);
   for (size_t k = 0; k < idle.size(); ++k)
     if (idle[k].key == key && idle[k].cap == cap) {
       sca::Bucket* b = idle[k].b;
@@ -144,8 +163,9 @@ void sca_server::trim_idle() {
     std::lock_guard<std::mutex> lock(mu);
     held = used;
   }
+  std::lock_guard<std::mutex> lock(idle_mu);
   for (const IdleBucket& k : idle) held += k.bytes;
-  while (!idle.empty() && (held > budget || now() - idle.front().since > kIdleSeconds)) {
+  while (!idle.empty() && (held > budget || expired(idle.front()))) {
     held -= idle.front().bytes;
     sca::bucket_destroy(idle.front().b);
     idle.erase(idle.begin());
@@ -154,10 +174,48 @@ void sca_server::trim_idle() {
 
 // Frees every idle workspace; false if there was none.
 bool sca_server::drop_idle() {
+  std::lock_guard<std::mutex> lock(idle_mu);
   if (idle.empty()) return false;
   for (IdleBucket& k : idle) sca::bucket_destroy(k.b);
   idle.clear();
   return true;
+}
+
+void sca_server::keep_idle(const IdleBucket& k) {
+  {
+    std::lock_guard<std::mutex> lock(idle_mu);
+    if (manual && !reaper.joinable()) {
+      try {
+        reaper = std::thread([this] { reap(); });
+      } catch (const std::system_error&) {  // no thread to free it in time: now
+        sca::bucket_destroy(k.b);
+        return;
+      }
+    }
+    idle.push_back(k);
+  }
+  idle_cv.notify_one();
+  trim_idle();
+}
+
+void sca_server::reap() {
+  cudaSetDevice(device);
+  // its frees must not end a stream capture of another thread
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  (void)cudaThreadExchangeStreamCaptureMode(&mode);
+  std::unique_lock<std::mutex> lock(idle_mu);
+  while (!reaper_stop) {
+    if (idle.empty()) {
+      idle_cv.wait(lock);
+      continue;
+    }
+    if (!expired(idle.front())) {
+      idle_cv.wait_until(lock, idle.front().since + idle_time());
+      continue;
+    }
+    sca::bucket_destroy(idle.front().b);
+    idle.erase(idle.begin());
+  }
 }
 
 void sca_server::finish(Request* r, sca_status st) {
@@ -166,7 +224,7 @@ void sca_server::finish(Request* r, sca_status st) {
     sca_destroy(r->ctx);
     r->ctx = nullptr;
   }
-  IdleBucket gone{{r->p.L, r->p.prec}, nullptr, 0, 0, 0.0};
+  IdleBucket gone{{r->p.L, r->p.prec}, nullptr, 0, 0, std::chrono::steady_clock::now()};
   if (r->in_bucket) sca::bucket_req_release(&r->br);
   {
     std::lock_guard<std::mutex> lock(mu);
@@ -180,7 +238,6 @@ void sca_server::finish(Request* r, sca_status st) {
         gone.b = it->second.b;
         gone.cap = it->second.cap;
         gone.bytes = it->second.bytes;
-        gone.since = now();
         used -= it->second.bytes;
         buckets.erase(it);
       }
@@ -188,8 +245,7 @@ void sca_server::finish(Request* r, sca_status st) {
   }
   if (!gone.b) return;
   if (st == SCA_OK) {
-    idle.push_back(gone);
-    trim_idle();
+    keep_idle(gone);
   } else {  // after a failure its state is not trusted
     sca::bucket_destroy(gone.b);
   }
@@ -366,15 +422,10 @@ bool sca_server::round_once(bool idle_wait) {
           std::lock_guard<std::mutex> lock(mu);
           bs = &buckets[{r->p.L, r->p.prec}];
         }
-        if (!bs->b) {
-          st = sca::bucket_create(r->p.L, r->p.prec, bs->cap, &bs->b);
-          if (st != SCA_OK && drop_idle())
-            st = sca::bucket_create(r->p.L, r->p.prec, bs->cap, &bs->b);
-        }
+        if (!bs->b) st = sca::bucket_create(r->p.L, r->p.prec, bs->cap, &bs->b);
         if (st == SCA_OK) st = sca::bucket_req_init(bs->b, &r->br, r->p, r->a);
       } else {
         st = sca_create(&r->p, &r->ctx);
-        if (st != SCA_OK && drop_idle()) st = sca_create(&r->p, &r->ctx);
         if (st == SCA_OK) st = sca_adam_init(r->ctx, &r->a, nullptr);
       }
       if (st != SCA_OK) {
@@ -430,6 +481,25 @@ bool sca_server::round_once(bool idle_wait) {
   return true;
 }
 
+// The servers whose idle workspaces a failed allocation may free.
+static std::mutex g_servers_mu;
+static std::vector<sca_server*> g_servers;
+
+static void register_server(sca_server* s) {
+  std::lock_guard<std::mutex> lock(g_servers_mu);
+  g_servers.push_back(s);
+}
+
+bool sca::drop_idle_workspaces() {
+  int dev = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  std::lock_guard<std::mutex> lock(g_servers_mu);
+  bool any = false;
+  for (sca_server* s : g_servers)
+    if (s->device == dev && s->drop_idle()) any = true;
+  return any;
+}
+
 extern "C" {
 
 sca_status sca_server_create(uint64_t hbm_budget_bytes, int32_t max_slots, sca_server** out) {
@@ -452,6 +522,7 @@ sca_status sca_server_create(uint64_t hbm_budget_bytes, int32_t max_slots, sca_s
     return sca::cuda_fail(err, "cudaGetDevice");
   }
   s->worker = std::thread([s] { s->run(); });
+  register_server(s);
   *out = s;
   return SCA_OK;
 }
@@ -476,6 +547,7 @@ sca_status sca_server_create_manual(uint64_t hbm_budget_bytes, int32_t max_slots
     delete s;
     return sca::cuda_fail(err, "cudaGetDevice");
   }
+  register_server(s);
   *out = s;
   return SCA_OK;
 }
@@ -595,11 +667,21 @@ sca_status sca_request_times(sca_server* s, uint64_t req_id, double* submit_s, d
 void sca_server_destroy(sca_server* s) {
   if (!s) return;
   {
+    std::lock_guard<std::mutex> lock(g_servers_mu);
+    g_servers.erase(std::remove(g_servers.begin(), g_servers.end(), s), g_servers.end());
+  }
+  {
     std::lock_guard<std::mutex> lock(s->mu);
     s->stop = true;
   }
   s->cv.notify_all();
   if (s->worker.joinable()) s->worker.join();
+  {
+    std::lock_guard<std::mutex> lock(s->idle_mu);
+    s->reaper_stop = true;
+  }
+  s->idle_cv.notify_all();
+  if (s->reaper.joinable()) s->reaper.join();
   for (auto& kv : s->all) {
     if (kv.second->ctx) sca_destroy(kv.second->ctx);
     if (kv.second->in_bucket) sca::bucket_req_release(&kv.second->br);

@@ -1258,7 +1258,7 @@ sca_status tc_prepare(Engine& e) {
     delete t;
     return cuda_fail(err, "tcgen05 update set-up");
   }
-  err = cudaMalloc((void**)&e.tc_counters, kCounters * sizeof(int));
+  err = device_malloc((void**)&e.tc_counters, kCounters * sizeof(int));
   if (err == cudaSuccess) err = cudaMemset(e.tc_counters, 0, kCounters * sizeof(int));
   if (err != cudaSuccess) {
     delete t;
