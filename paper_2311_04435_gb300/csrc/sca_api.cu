@@ -283,7 +283,6 @@ sca_status allocate(Engine& e) {
   if (e.tc && (st = tc_prepare(e)) != SCA_OK) { release(e); return st; }
 #undef SCA_ALLOC
   if ((st = fused_prepare(e)) != SCA_OK) { release(e); return st; }
-  if ((st = nested_prepare(e)) != SCA_OK) { release(e); return st; }
   if (e.tc && e.piv_blocks > 0) {
     // SMs kept free for the pivoted group (SCA_SM_RESERVE overrides the default)
     int r = e.N > 2048 ? kLargeNSmReserve : kDefaultSmReserve;
@@ -303,6 +302,7 @@ sca_status allocate(Engine& e) {
   if (err != cudaSuccess) { release(e); return cuda_fail(err, "side stream"); }
   err = cudaEventCreateWithFlags(&e.ev_join2, cudaEventDisableTiming);
   if (err != cudaSuccess) { release(e); return cuda_fail(err, "join event"); }
+  if (e.nest_rule && !e.dense_switch && (st = nested_prepare(e)) != SCA_OK) { release(e); return st; }
   if (e.tc && e.piv_blocks > 0 && e.N >= 1024 && e.N <= 2048 && e.B - e.piv_blocks >= 64) {
     // merged pairs: one partition of 16 SMs (8 if refused); otherwise two dominant partitions
     // (mode 3), one if the driver refuses the second; ordinary streams if it refuses both
@@ -661,6 +661,8 @@ sca_status sca_dos(sca_ctx* c, const double* phi_host, const double* w_host, int
   if (st != SCA_OK) return st;
   Engine& e = c->e;
   c->kept = false;
+  if (!e.dense_switch && nested_rule(e.p.t, eta, eta) && (st = nested_prepare(e)) != SCA_OK)
+    return st;
   const int half = e.B / 2;
   std::vector<double> hz((size_t)e.B), htr((size_t)e.B);
   // Every resolvent has Im z = eta: columns are strictly diagonally dominant (and the

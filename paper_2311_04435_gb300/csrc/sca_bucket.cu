@@ -212,6 +212,7 @@ sca_status bucket_run(Bucket* b, BucketReq* const* requests, int n, int nsteps, 
       if (range == 1) npiv[p] = next;
     }
     ntot[p] = next;
+    if (wide[p] > 0 && (st = nested_wide_stream(e)) != SCA_OK) return st;
     for (int sidx = 0; sidx < nsteps; ++sidx) {
       ReqDesc* rq = b->h_req + ((size_t)p * b->steps + sidx) * b->rmax;
       for (int k = 0; k < count[p]; ++k) {

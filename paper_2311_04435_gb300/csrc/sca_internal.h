@@ -272,7 +272,10 @@ constexpr double kFloat2EnoughSmall = 0.3, kFloat2Enough = 0.15;  // up to 10x10
 enum class NestedArith { kFloat2, kFloat64, kWide32, kWide64 };  // the last: of a float64 context
 bool nested_wide(bool fp64, int L, double t, double imag);
 int nested_wide_blocks(bool fp64, int L, double t, double T, int n_omega);  // leading blocks
-sca_status nested_prepare(Engine& e);  // tables (leaves e.nest null where it does not apply)
+// Tables, streams and memory of a context that takes it (at creation, or on the first density of
+// states that does).
+sca_status nested_prepare(Engine& e);
+sca_status nested_wide_stream(Engine& e);  // for passes beside which blocks take wider arithmetic
 void nested_release(Engine& e);
 bool nested_now(const Engine& e);      // whether the next evaluation takes it
 // up: eliminate (ld); down: diag(G) from the fronts left in M by a preceding `up`.

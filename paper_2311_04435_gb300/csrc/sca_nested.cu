@@ -56,6 +56,9 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstring>
+#include <memory>
+#include <mutex>
 #include <new>
 #include <type_traits>
 #include <vector>
@@ -1238,10 +1241,9 @@ size_t down_smem(const nested::Node& n, size_t z) {
 
 }  // namespace
 
-// Per-context state: the tree's tables on the device and the shapes that the launch plans follow.
-struct Nested {
-  Node* d_nodes = nullptr;
-  int16_t* d_tab = nullptr;
+// The two forms of one lattice size's tree, as every context of that size takes them: the tables in
+// one piece (nodes, then indices) and the shapes that the launch plans follow.
+struct NestedForms {
   struct Shape {
     int first, count, group;  // group: the fewest threads for a front
     int bytes[3];             // shared memory of a front with entries of 16, 24 and 32 bytes
@@ -1249,16 +1251,10 @@ struct Nested {
     int smem() const { return bytes[sizeof(Z) / 8 - 2]; }
   };
   std::vector<Shape> levels[2];
+  std::vector<char> tables;
+  size_t index_at = 0;    // offset of the indices
   int nnodes = 0;
   long long stride = 0;   // entries per block
-  char* fronts = nullptr; // where they are kept: the context's blocks, or `own`
-  size_t room = 0;
-  void* own = nullptr;    // their own memory where the blocks' is too small
-  int sms = 1;
-  // more blocks than SMs: the second half of a pass that takes a launch per level, and the blocks
-  // in wider arithmetic (which otherwise take the side stream)
-  cudaStream_t half = nullptr, wide = nullptr;
-  cudaEvent_t ev_half = nullptr, ev_wide = nullptr;
 
   // A block's fronts, and with its shares of |det A|^2.  (A float64 context's wider blocks have
   // room for double-double, at the same place for both arithmetics that they may take.)
@@ -1266,6 +1262,31 @@ struct Nested {
     return (a == NestedArith::kWide64 ? 32 : a == NestedArith::kWide32 ? 24 : 16) * (size_t)stride;
   }
   size_t block_bytes(NestedArith a) const { return front_bytes(a) + sizeof(Det) * nnodes; }
+  // Room for all blocks in their arithmetic where all are to be resident, and for one block of the
+  // wider one in any case.  From 10 x 10 sites up the dense blocks take more than either.
+  size_t room_for(const Engine& e) const {
+    const size_t base = block_bytes(e.fp64 ? NestedArith::kFloat64 : NestedArith::kFloat2);
+    const size_t wide = block_bytes(e.fp64 ? NestedArith::kWide64 : NestedArith::kWide32);
+    if (e.chunk < e.B) return wide;
+    return std::max(wide, e.nest_wide * wide + (e.B - e.nest_wide) * base + 256);
+  }
+};
+
+// Per-context state: the tables on the device, memory, streams.
+struct Nested {
+  const NestedForms& f;
+  explicit Nested(const NestedForms& forms) : f(forms) {}
+  char* d_tables = nullptr;
+  char* fronts = nullptr; // where they are kept: the context's blocks, or `own`
+  size_t room = 0;
+  void* own = nullptr;    // their own memory where the blocks' is too small
+  int sms = 1;
+  // more blocks than SMs: the second half of a pass that takes a launch per level (a stream of its
+  // own only where there is no second stream of the dense elimination), and the blocks in wider
+  // arithmetic (which otherwise take the side stream)
+  cudaStream_t half = nullptr, wide = nullptr;
+  bool half_own = false;
+  cudaEvent_t ev_half = nullptr, ev_wide = nullptr;
 };
 
 namespace {
@@ -1280,8 +1301,8 @@ size_t plan_levels(const Nested& ne, NestArgs<Z>& a) {
   static_assert(nt / 64 < 16, "a group above a warp needs one of the 15 barriers left");
   size_t need = 0;
   for (int form = 0; form < 2; ++form)
-    for (size_t k = 0; k < ne.levels[form].size(); ++k) {
-      const Nested::Shape& s = ne.levels[form][k];
+    for (size_t k = 0; k < ne.f.levels[form].size(); ++k) {
+      const NestedForms::Shape& s = ne.f.levels[form][k];
       const int smem = s.smem<Z>();
       int g = s.group;
       while (2 * g <= nt && ((nt / (2 * g)) * a.csize >= s.count || nt / g * smem > room)) g *= 2;
@@ -1335,12 +1356,12 @@ sca_status run_blocks_of(Engine& e, const Lattice& la, int b0, int cnt, char* me
                          int range = 0) {
   const Nested& ne = *e.nest;
   NestArgs<Z> a;
-  a.nodes = ne.d_nodes;
-  a.tab = ne.d_tab;
+  a.nodes = reinterpret_cast<const Node*>(ne.d_tables);
+  a.tab = reinterpret_cast<const int16_t*>(ne.d_tables + ne.f.index_at);
   a.fronts = reinterpret_cast<Z*>(mem);
   a.stride = (long long)(bytes / sizeof(Z));
-  a.nnodes = ne.nnodes;
-  a.nlevels = (int)ne.levels[0].size();
+  a.nnodes = ne.f.nnodes;
+  a.nlevels = (int)ne.f.levels[0].size();
   a.la = la;
   a.ld = e.ld;
   a.gd = e.gd;
@@ -1389,7 +1410,7 @@ sca_status run_blocks_of(Engine& e, const Lattice& la, int b0, int cnt, char* me
         const int level = k < nl ? nl - 1 - k : k - nl;
         f.k0 = k;
         f.k1 = k + 1;
-        const Nested::Shape& sh = ne.levels[pt.form][level];
+        const NestedForms::Shape& sh = ne.f.levels[pt.form][level];
         const int smem = sh.smem<Z>();
         int g = sh.group;  // the fewest threads while they fill the SMs; four CTAs per SM
         while (2 * g <= 256 && ((long long)sh.count * pt.all * g < 1024ll * ne.sms ||
@@ -1429,7 +1450,7 @@ sca_status run_blocks_of(Engine& e, const Lattice& la, int b0, int cnt, char* me
 
 sca_status run_blocks_in(NestedArith ar, Engine& e, const Lattice& la, int b0, int cnt, char* mem,
                          int free_sms, bool up, bool down, cudaStream_t s, int max_cluster = 8) {
-  const size_t by = e.nest->front_bytes(ar);
+  const size_t by = e.nest->f.front_bytes(ar);
   const int mc = max_cluster;
   if (ar == NestedArith::kFloat2)
     return run_blocks_of<Zf>(e, la, b0, cnt, mem, by, free_sms, up, down, s, mc);
@@ -1462,60 +1483,90 @@ int nested_wide_blocks(bool fp64, int L, double t, double T, int n_omega) {
   return 2 * n;
 }
 
+// The forms of lattice size L: constant data, built by the first context of that size (64x64: 0.6 ms)
+// and kept, 0.3 MB at most each.  Null where host memory is short.
+static const NestedForms* nested_forms(int L) {
+  static std::mutex mu;
+  static std::unique_ptr<const NestedForms> built[33];
+  if (L < nested::kMinL || L > 64) return nullptr;
+  std::lock_guard<std::mutex> lock(mu);
+  std::unique_ptr<const NestedForms>& slot = built[L / 2];
+  if (slot) return slot.get();
+  try {
+    std::unique_ptr<NestedForms> f(new NestedForms());
+    nested::Tree t[2] = {nested::Builder(L).build(false), nested::Builder(L).build(true)};
+    f->nnodes = (int)t[0].nodes.size();
+    // whole entries of 16, 24 and 32 bytes
+    f->stride = (std::max(t[0].entries, t[1].entries) + 5) / 6 * 6;
+    std::vector<Node> nodes;
+    std::vector<int16_t> table;
+    for (int form = 0; form < 2; ++form) {
+      for (const nested::Level& lv : t[form].levels) {
+        NestedForms::Shape sh{lv.first, lv.count, 32, {0, 0, 0}};
+        for (int k = lv.first; k < lv.first + lv.count; ++k) {
+          const nested::Node& n = t[form].nodes[k];
+          while (10 * sh.group < 9 * (n.p + n.q) || n.pw > kSlots * (sh.group / n.pw)) sh.group *= 2;
+          for (int z = 16; z <= 32; z += 8) {
+            int& by = sh.bytes[z / 8 - 2];
+            by = std::max(by, ((int)std::max(up_smem(n, z), down_smem(n, z)) + 15) / 16 * 16);
+          }
+        }
+        f->levels[form].push_back(sh);
+      }
+      // one table: a form's offsets follow the entries before it
+      const int at = (int)table.size();
+      table.insert(table.end(), t[form].table.begin(), t[form].table.end());
+      for (nested::Node n : t[form].nodes) {
+        for (int* o : {&n.sites, &n.cmap[0], &n.cmap[1], &n.pmap, &n.bsite, &n.bnbr, &n.adj}) *o += at;
+        nodes.push_back(n);
+      }
+    }
+    f->index_at = (sizeof(Node) * nodes.size() + 15) / 16 * 16;
+    f->tables.resize(f->index_at + sizeof(int16_t) * table.size());
+    std::memcpy(f->tables.data(), nodes.data(), sizeof(Node) * nodes.size());
+    std::memcpy(f->tables.data() + f->index_at, table.data(), sizeof(int16_t) * table.size());
+    slot = std::move(f);
+  } catch (const std::bad_alloc&) {
+    return nullptr;
+  }
+  return slot.get();
+}
+
+sca_status nested_wide_stream(Engine& e) {
+  Nested* ne = e.nest;
+  if (!ne || ne->wide || e.B <= ne->sms) return SCA_OK;
+  int least = 0, greatest = 0;
+  cudaError_t err = cudaDeviceGetStreamPriorityRange(&least, &greatest);
+  if (err == cudaSuccess)
+    err = cudaStreamCreateWithPriority(&ne->wide, cudaStreamNonBlocking, greatest);
+  return err == cudaSuccess ? SCA_OK : cuda_fail(err, "nested elimination set-up");
+}
+
 sca_status nested_prepare(Engine& e) {
-  e.nest = nullptr;
-  if (e.L < nested::kMinL) return SCA_OK;
-  nested::Tree t = nested::Builder(e.L).build(false);
-  const nested::Tree td = nested::Builder(e.L).build(true);
-  Nested* ne = new (std::nothrow) Nested();
+  if (e.nest || e.L < nested::kMinL) return SCA_OK;
+  const NestedForms* forms = nested_forms(e.L);
+  Nested* ne = forms ? new (std::nothrow) Nested(*forms) : nullptr;
   if (!ne) { set_error("host allocation failed"); return SCA_ENOMEM; }
   e.nest = ne;
-  ne->nnodes = (int)td.nodes.size();
-  ne->stride = (std::max(t.entries, td.entries) + 5) / 6 * 6;  // whole entries of 16, 24, 32 bytes
-  const nested::Tree* forms[2] = {&t, &td};
-  for (int form = 0; form < 2; ++form)
-    for (const nested::Level& lv : forms[form]->levels) {
-      Nested::Shape sh{lv.first, lv.count, 32, {0, 0, 0}};
-      for (int k = lv.first; k < lv.first + lv.count; ++k) {
-        const nested::Node& n = forms[form]->nodes[k];
-        while (10 * sh.group < 9 * (n.p + n.q) || n.pw > kSlots * (sh.group / n.pw)) sh.group *= 2;
-        for (int z = 16; z <= 32; z += 8) {
-          int& by = sh.bytes[z / 8 - 2];
-          by = std::max(by, ((int)std::max(up_smem(n, z), down_smem(n, z)) + 15) / 16 * 16);
-        }
-      }
-      ne->levels[form].push_back(sh);
-    }
-  // both forms in one table: the second's offsets follow the first's entries
-  const int toff = (int)t.table.size();
-  t.table.insert(t.table.end(), td.table.begin(), td.table.end());
-  for (nested::Node n : td.nodes) {
-    for (int* o : {&n.sites, &n.cmap[0], &n.cmap[1], &n.pmap, &n.bsite, &n.bnbr, &n.adj}) *o += toff;
-    t.nodes.push_back(n);
-  }
   int dev = 0;
   cudaError_t err = cudaGetDevice(&dev);
   if (err == cudaSuccess)
     err = cudaDeviceGetAttribute(&ne->sms, cudaDevAttrMultiProcessorCount, dev);
-  if (err != cudaSuccess) { nested_release(e); return cuda_fail(err, "nested elimination set-up"); }
-  err = cudaEventCreateWithFlags(&ne->ev_wide, cudaEventDisableTiming);
+  if (err == cudaSuccess) err = cudaEventCreateWithFlags(&ne->ev_wide, cudaEventDisableTiming);
   if (err == cudaSuccess && e.B > ne->sms) {
-    int least = 0, greatest = 0;
-    err = cudaDeviceGetStreamPriorityRange(&least, &greatest);
-    if (err == cudaSuccess)
-      err = cudaStreamCreateWithPriority(&ne->wide, cudaStreamNonBlocking, greatest);
-    if (err == cudaSuccess) err = cudaStreamCreateWithFlags(&ne->half, cudaStreamNonBlocking);
+    ne->half = e.aux;
+    if (!ne->half) {
+      err = cudaStreamCreateWithFlags(&ne->half, cudaStreamNonBlocking);
+      ne->half_own = err == cudaSuccess;
+    }
     if (err == cudaSuccess) err = cudaEventCreateWithFlags(&ne->ev_half, cudaEventDisableTiming);
   }
   if (err != cudaSuccess) { nested_release(e); return cuda_fail(err, "nested elimination set-up"); }
-  // Room for all blocks in their arithmetic where all are to be resident, and for one block of the
-  // wider one in any case.  From 10 x 10 sites up the dense blocks take more than either.
-  const NestedArith base = e.fp64 ? NestedArith::kFloat64 : NestedArith::kFloat2;
-  const NestedArith wide = e.fp64 ? NestedArith::kWide64 : NestedArith::kWide32;
-  size_t need = ne->block_bytes(wide);
-  if (e.chunk == e.B)
-    need = std::max(need, e.nest_wide * ne->block_bytes(wide) +
-                              (e.B - e.nest_wide) * ne->block_bytes(base) + 256);
+  if (e.nest_wide > 0) {
+    const sca_status st = nested_wide_stream(e);
+    if (st != SCA_OK) { nested_release(e); return st; }
+  }
+  const size_t need = forms->room_for(e);
   ne->fronts = static_cast<char*>(e.M);
   ne->room = e.block_room;
   if (need > ne->room) {
@@ -1523,24 +1574,24 @@ sca_status nested_prepare(Engine& e) {
     ne->fronts = static_cast<char*>(ne->own);
     ne->room = need;
   }
-  if (err == cudaSuccess) err = device_malloc((void**)&ne->d_nodes, sizeof(Node) * t.nodes.size());
-  if (err == cudaSuccess) err = device_malloc((void**)&ne->d_tab, sizeof(int16_t) * t.table.size());
+  if (err == cudaSuccess) err = device_malloc((void**)&ne->d_tables, forms->tables.size());
   if (err != cudaSuccess) {
     nested_release(e);
     (void)cudaGetLastError();
     set_error("cudaMalloc failed for the elimination tree or its fronts");
     return SCA_ENOMEM;
   }
-  err = cudaMemcpy(ne->d_nodes, t.nodes.data(), sizeof(Node) * t.nodes.size(), cudaMemcpyHostToDevice);
-  if (err == cudaSuccess)
-    err = cudaMemcpy(ne->d_tab, t.table.data(), sizeof(int16_t) * t.table.size(), cudaMemcpyHostToDevice);
+  err = cudaMemcpy(ne->d_tables, forms->tables.data(), forms->tables.size(), cudaMemcpyHostToDevice);
+  // (a copy from pageable memory may still be under way, and the context's streams do not wait for
+  // the default one)
+  if (err == cudaSuccess) err = cudaStreamSynchronize(cudaStreamLegacy);
   if (err != cudaSuccess) { nested_release(e); return cuda_fail(err, "elimination tree upload"); }
   return SCA_OK;
 }
 
 void nested_release(Engine& e) {
   if (!e.nest) return;
-  if (e.nest->half) {
+  if (e.nest->half_own) {
     cudaStreamSynchronize(e.nest->half);
     cudaStreamDestroy(e.nest->half);
   }
@@ -1551,8 +1602,7 @@ void nested_release(Engine& e) {
   if (e.nest->ev_half) cudaEventDestroy(e.nest->ev_half);
   if (e.nest->ev_wide) cudaEventDestroy(e.nest->ev_wide);
   if (e.nest->own) cudaFree(e.nest->own);
-  if (e.nest->d_nodes) cudaFree(e.nest->d_nodes);
-  if (e.nest->d_tab) cudaFree(e.nest->d_tab);
+  if (e.nest->d_tables) cudaFree(e.nest->d_tables);
   delete e.nest;
   e.nest = nullptr;
 }
@@ -1578,8 +1628,8 @@ sca_status run_nested(Engine& e, const Lattice& la, bool up, bool down, cudaStre
   size_t total = 0;
   for (int k = 0; k < 2; ++k)
     if (const int n = ends[k + 1] - ends[k]) {
-      groups[ng] = {kinds[k], ends[k], n, (n * ne.block_bytes(kinds[k]) + 255) / 256 * 256};
-      total += k == 0 && nw < e.B ? groups[ng].bytes : n * ne.block_bytes(kinds[k]);
+      groups[ng] = {kinds[k], ends[k], n, (n * ne.f.block_bytes(kinds[k]) + 255) / 256 * 256};
+      total += k == 0 && nw < e.B ? groups[ng].bytes : n * ne.f.block_bytes(kinds[k]);
       ++ng;
     }
   if (total > ne.room) {  // one after another, in passes that fit
@@ -1588,7 +1638,7 @@ sca_status run_nested(Engine& e, const Lattice& la, bool up, bool down, cudaStre
       return SCA_ENOSTATE;
     }
     for (int g = 0; g < ng; ++g) {
-      const int cap = (int)std::min<size_t>(ne.room / ne.block_bytes(groups[g].ar), groups[g].n);
+      const int cap = (int)std::min<size_t>(ne.room / ne.f.block_bytes(groups[g].ar), groups[g].n);
       for (int b = 0; b < groups[g].n; b += cap) {
         const sca_status st = run_blocks_in(groups[g].ar, e, la, groups[g].first + b,
                                             std::min(cap, groups[g].n - b), ne.fronts, ne.sms, up,
