@@ -125,7 +125,8 @@ sca_status sca_create(const sca_params* params, sca_ctx** out);
 /* Frees the context and its workspace.  NULL is ignored. */
 void sca_destroy(sca_ctx* ctx);
 
-/* Bytes of device memory a context with these parameters allocates. */
+/* Bytes of device memory a context with these parameters allocates, for site energies and densities
+ * of states too; not the arrays of sca_metropolis_init. */
 sca_status sca_workspace_bytes(const sca_params* params, uint64_t* bytes);
 
 /* Adds a per-site energy eps_extra[i] (N host doubles) to H_sigma, e.g. the

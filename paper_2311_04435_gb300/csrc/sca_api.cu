@@ -205,16 +205,22 @@ sca_status plan(const sca_params& p, Engine& e) {
   e.nest_rule = nested_rule(p.t, M_PI * p.T, (2.0 * p.n_omega - 1.0) * M_PI * p.T);
   e.nest_wide = nested_wide_blocks(e.fp64, p.L, p.t, p.T, p.n_omega);
   e.dense_switch = dense_switch_set();
-  size_t bytes = 0;
-  bytes += (size_t)e.chunk * e.mat_stride * S;           // blocks
-  bytes += 2 * (size_t)e.chunk * e.fw_mat * S;            // F, W
+  // Blocks, F and W are one allocation.  The nested elimination's fronts take the blocks' place;
+  // up to 8 x 8 sites they need more than the float32 blocks and run into F and W, which hold no
+  // zero padding there (one elimination step: the whole block is its pivot block).
+  e.m_bytes = round_up((size_t)e.chunk * e.mat_stride * S, 1024);
+  e.fw_bytes = round_up((size_t)e.chunk * e.fw_mat * S, 1024);
+  e.block_room = e.N <= e.nb ? e.m_bytes + 2 * e.fw_bytes : e.m_bytes;
+  size_t bytes = e.m_bytes + 2 * e.fw_bytes;
   if (e.pair) bytes += 2 * (size_t)e.chunk * e.fw_mat * S;  // F2, W2
   bytes += (size_t)e.chunk * 2 * e.nb * e.nb * 2 * C;     // Tinv
   if (e.tc) bytes += (size_t)e.chunk * kTtPlanes * e.nb * e.nb * 4;  // -T^T split planes
   bytes += (size_t)e.chunk * e.N * 2 * sizeof(float);     // Re A_jj as double-float
   bytes += 2 * (size_t)e.chunk * e.N * sizeof(int);       // piv, perm
   bytes += (size_t)e.B * sizeof(double) * (3 + e.N);      // ld, d_z, tr, gd
-  bytes += (size_t)e.N * sizeof(double) * 7 + 256;        // eps, phi, m, v, g, in, misc
+  bytes += (size_t)e.N * sizeof(double) * 6;              // eps, phi, m, v, g, in
+  bytes += 2 * 64 + 16 + 16;                              // status, Omega, flags, fused barrier
+  if (e.tc) bytes += kTcCounters * sizeof(int);           // tile counters
   e.bytes = bytes;
   return SCA_OK;
 }
@@ -237,15 +243,9 @@ sca_status allocate(Engine& e) {
   sca_status st;
 #define SCA_ALLOC(ptr, bytes, what) \
   if ((st = dev_alloc(&(ptr), (bytes), e, what)) != SCA_OK) return st;
-  // Blocks, F and W in one allocation.  The nested elimination's fronts take the blocks' place;
-  // up to 8 x 8 sites they need more than the float32 blocks and run into F and W, which hold no
-  // zero padding there (one elimination step: the whole block is its pivot block).
-  const size_t mbytes = round_up((size_t)e.chunk * e.mat_stride * S, 1024);
-  const size_t fbytes = round_up((size_t)e.chunk * e.fw_mat * S, 1024);
-  e.block_room = e.N <= e.nb ? mbytes + 2 * fbytes : mbytes;
-  SCA_ALLOC(e.M, mbytes + 2 * fbytes, "blocks, F and W");
-  e.F = static_cast<char*>(e.M) + mbytes;
-  e.W = static_cast<char*>(e.F) + fbytes;
+  SCA_ALLOC(e.M, e.m_bytes + 2 * e.fw_bytes, "blocks, F and W");
+  e.F = static_cast<char*>(e.M) + e.m_bytes;
+  e.W = static_cast<char*>(e.F) + e.fw_bytes;
   SCA_ALLOC(e.Tinv, (size_t)e.chunk * 2 * e.nb * e.nb * 2 * S, "Tinv");
   SCA_ALLOC(e.adiag, (size_t)e.chunk * e.N * 2 * sizeof(float), "diagonal table");
   SCA_ALLOC(e.piv, (size_t)e.chunk * e.N * sizeof(int), "piv");
@@ -501,7 +501,7 @@ sca_status sca_workspace_bytes(const sca_params* params, uint64_t* bytes) {
   if (!bytes) { set_error("bytes is NULL"); return SCA_EINVAL; }
   Engine e;
   plan(*params, e);
-  *bytes = e.bytes;
+  *bytes = e.bytes + nested_bytes(e);
   return SCA_OK;
 }
 

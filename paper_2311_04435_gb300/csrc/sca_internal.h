@@ -107,6 +107,7 @@ struct Engine {
   size_t plane_stride = 0, mat_stride = 0;  // elements
   size_t fw_plane = 0, fw_mat = 0;          // F / W panel strides (elements)
 
+  size_t m_bytes = 0, fw_bytes = 0;  // the blocks' part of the allocation at M, F's and W's
   size_t block_room = 0;    // bytes from M on that the nested elimination's fronts may use
   void* M = nullptr;        // chunk blocks
   void* F = nullptr;        // chunk x 2 planes x N x nb (x2 hi/lo for tc)
@@ -184,6 +185,7 @@ struct Engine {
 // Float-plane slots per block of the -T^T split planes (re_hi, im_hi, re_lo, im_lo; a bf16
 // plane fills the first half of its slot).
 constexpr int kTtPlanes = 4;
+constexpr int kTcCounters = 1024;  // tile counters per pass (one per tensor-core launch)
 
 // Kernel kinds for per-launch timing.
 enum KernelKind {
@@ -275,6 +277,7 @@ int nested_wide_blocks(bool fp64, int L, double t, double T, int n_omega);  // l
 // Tables, streams and memory of a context that takes it (at creation, or on the first density of
 // states that does).
 sca_status nested_prepare(Engine& e);
+size_t nested_bytes(const Engine& e);  // device memory that this may allocate
 sca_status nested_wide_stream(Engine& e);  // for passes beside which blocks take wider arithmetic
 void nested_release(Engine& e);
 bool nested_now(const Engine& e);      // whether the next evaluation takes it

@@ -1532,6 +1532,13 @@ static const NestedForms* nested_forms(int L) {
   return slot.get();
 }
 
+size_t nested_bytes(const Engine& e) {
+  const NestedForms* f = e.dense_switch ? nullptr : nested_forms(e.L);
+  if (!f) return 0;
+  const size_t need = f->room_for(e);
+  return f->tables.size() + (need > e.block_room ? need : 0);
+}
+
 sca_status nested_wide_stream(Engine& e) {
   Nested* ne = e.nest;
   if (!ne || ne->wide || e.B <= ne->sms) return SCA_OK;

@@ -37,9 +37,6 @@
 namespace sca {
 namespace {
 
-}  // namespace
-constexpr int kCounters = 1024;    // tile counters per pass (one per tensor-core launch)
-namespace {
 constexpr int kBM = 128;           // F rows per tile
 constexpr int kBNc = 128;          // complex W columns per tile (real MMA N = 256)
 constexpr int kKS = 16;            // K per pipeline stage (SWIZZLE_64B rows of 64 bytes)
@@ -1184,7 +1181,7 @@ bool make_m_map(CUtensorMap* m, void* base, int N, int ldm, long long plane_stri
 sca_status tc_reset_counters(Engine& e, cudaStream_t s) {
   e.tc_next = 0;
   if (!e.tc_counters) return SCA_OK;
-  cudaError_t err = cudaMemsetAsync(e.tc_counters, 0, kCounters * sizeof(int), s);
+  cudaError_t err = cudaMemsetAsync(e.tc_counters, 0, kTcCounters * sizeof(int), s);
   if (err != cudaSuccess) return cuda_fail(err, "tile counters");
   return SCA_OK;
 }
@@ -1258,8 +1255,8 @@ sca_status tc_prepare(Engine& e) {
     delete t;
     return cuda_fail(err, "tcgen05 update set-up");
   }
-  err = device_malloc((void**)&e.tc_counters, kCounters * sizeof(int));
-  if (err == cudaSuccess) err = cudaMemset(e.tc_counters, 0, kCounters * sizeof(int));
+  err = device_malloc((void**)&e.tc_counters, kTcCounters * sizeof(int));
+  if (err == cudaSuccess) err = cudaMemset(e.tc_counters, 0, kTcCounters * sizeof(int));
   if (err != cudaSuccess) {
     delete t;
     return cuda_fail(err, "tile counters");
@@ -1318,7 +1315,7 @@ sca_status tc_update(Engine& e, int m0, int cnt, int k0, int kb, int r0, int c0,
   a.cross_t = -1;
   a.kc0 = a.kcb = 0;
   if (a.tiles <= 0) return SCA_OK;
-  if (e.tc_next >= kCounters) {
+  if (e.tc_next >= kTcCounters) {
     set_error("too many tensor-core launches in one pass");
     return SCA_EINVAL;
   }
@@ -1370,7 +1367,7 @@ sca_status tc_update_pair(Engine& e, int m0, int cnt, int k1, int kb1, int k2, i
   a.T = nullptr;
   a.t_mat = 0;
   if (a.tiles <= 0) return SCA_OK;
-  if (e.tc_next >= kCounters) {
+  if (e.tc_next >= kTcCounters) {
     set_error("too many tensor-core launches in one pass");
     return SCA_EINVAL;
   }
@@ -1422,7 +1419,7 @@ sca_status tc_prep(Engine& e, int m0, int cnt, int r0, cudaStream_t s) {
   a.cross_t = -1;
   a.kc0 = a.kcb = 0;
   if (a.tiles <= 0) return SCA_OK;
-  if (e.tc_next >= kCounters) {
+  if (e.tc_next >= kTcCounters) {
     set_error("too many tensor-core launches in one pass");
     return SCA_EINVAL;
   }
@@ -1473,7 +1470,7 @@ sca_status tc_prep_split(Engine& e, int m0, int cnt, int r0, int k0, int kb, boo
   a.cross_t = -1;
   a.kc0 = a.kcb = 0;
   if (a.tiles <= 0) return SCA_OK;
-  if (e.tc_next >= kCounters) {
+  if (e.tc_next >= kTcCounters) {
     set_error("too many tensor-core launches in one pass");
     return SCA_EINVAL;
   }
@@ -1533,7 +1530,7 @@ sca_status tc_prep_piv(Engine& e, int m0, int cnt, int r0, int k0, int kb, bool 
     a.merge = 0;
     a.cross_t = -1;
     a.kc0 = a.kcb = 0;
-    if (e.tc_next >= kCounters) {
+    if (e.tc_next >= kTcCounters) {
       set_error("too many tensor-core launches in one pass");
       return SCA_EINVAL;
     }

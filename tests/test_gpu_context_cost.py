@@ -1,5 +1,6 @@
-"""What creating a context costs beside the memory it asks for: contexts that never take the nested
-elimination upload no tables for it, and those whose densities of states do get them then."""
+"""What creating a context costs: contexts that never take the nested elimination upload no tables
+for it, and those whose densities of states do get them then; the memory that a context takes is
+what sca_workspace_bytes says, which the server's admission goes by."""
 import os
 import subprocess
 import sys
@@ -14,6 +15,9 @@ _SHIM = r"""
 #include <dlfcn.h>
 #include <stddef.h>
 static long copies, streams;
+static unsigned long long allocated;
+unsigned long long shim_allocated(void) { return allocated; }
+int cudaMalloc(void** p, size_t n);
 long shim_copies(void) { return copies; }
 long shim_streams(void) { return streams; }
 static void* real_fn(const char* name) {
@@ -23,6 +27,11 @@ static void* real_fn(const char* name) {
     if (h) fn = dlsym(h, name);
   }
   return fn;
+}
+int cudaMalloc(void** p, size_t n) {
+  const int err = ((int (*)(void**, size_t))real_fn("cudaMalloc"))(p, n);
+  if (!err) allocated += n;
+  return err;
 }
 int cudaMemcpy(void* d, const void* s, size_t n, int k) {
   ++copies;
@@ -77,11 +86,38 @@ print("context cost ok")
 """
 
 
-def test_tables_and_streams_of_a_context(tmp_path):
+_MEMORY_CHILD = r"""
+import ctypes, os, sys
+import numpy as np
+sys.path.insert(0, sys.argv[1])
+from paper_2311_04435_gb300 import api, inputs
+shim = ctypes.CDLL(sys.argv[2])
+shim.shim_allocated.restype = ctypes.c_ulonglong
+api.Context(api.Params(4, 1, U=4.0, T=0.1)).close()
+for resident in (None, "3"):
+    if resident:
+        os.environ["SCA_MAX_BLOCKS_RESIDENT"] = resident
+    for L, nw, T, prec in ((4, 64, 0.1, "fp64"), (6, 40, 0.012, "fp64"), (8, 40, 0.05, "fp64"),
+                           (8, 20, 0.02, "fp32"), (14, 20, 0.1, "fp32"), (16, 30, 0.005, "bf16x3"),
+                           (20, 100, 0.1, "3xtf32"), (40, 8, 0.1, "bf16x3"), (64, 2, 0.1, "bf16x3")):
+        p = api.Params(L, nw, U=4.0, T=T, delta=0.5, prec=prec)
+        said, a0 = api.workspace_bytes(p), shim.shim_allocated()
+        with api.Context(p) as c:
+            c.set_site_energy(np.zeros(p.N))
+            c.blocks(inputs.seed_phi(1, p.N))
+            c.dos(inputs.seed_phi(1, p.N), np.array([0.1, 0.2]), 0.2)
+        took = shim.shim_allocated() - a0
+        assert 0 <= said - took <= 64, (L, nw, T, prec, resident, said, took)
+print("context cost ok")
+"""
+
+
+@pytest.mark.parametrize("child", [_CHILD, _MEMORY_CHILD], ids=["tables", "memory"])
+def test_cost_of_a_context(tmp_path, child):
     src, shim = tmp_path / "shim.c", tmp_path / "libshim.so"
     src.write_text(_SHIM)
     subprocess.run(["gcc", "-O1", "-shared", "-fPIC", "-o", str(shim), str(src), "-ldl"], check=True)
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
-    r = subprocess.run([sys.executable, "-c", _CHILD, root, str(shim)], capture_output=True,
+    r = subprocess.run([sys.executable, "-c", child, root, str(shim)], capture_output=True,
                        text=True, timeout=300, env=dict(os.environ, LD_PRELOAD=str(shim)))
     assert r.returncode == 0 and "context cost ok" in r.stdout, r.stdout + r.stderr
