@@ -39,10 +39,11 @@
  *    through the lattice's sparsity: nested dissection of the torus, then the entries of
  *    A^{-1} inside the fronts, in float64 (SCA_PREC_FP64) or double-float (48 bits, the other
  *    three); blocks of small omega_n, and float64 densities of states of small eta, in sums of
- *    three float32 (72 bits), as rounding grows there on weak fields.  Below that line, for smaller lattices, and where the caller asks for it
- *    (sca_set_pivoting, sca_set_panel_precision, sca_profile_enable(ctx, 1), or one of the
- *    dense elimination's environment switches set when the context is created), every block is
- *    eliminated as a dense matrix in the context's precision ("the dense elimination" below).
+ *    three float32 (72 bits), as rounding grows there on weak fields.  Below that line, for smaller
+ *    lattices, and where the caller asks for it (sca_set_pivoting, sca_set_panel_precision,
+ *    sca_profile_enable(ctx, 1), or one of the dense elimination's environment switches set when
+ *    the context is created), every block is eliminated as a dense matrix in the context's
+ *    precision ("the dense elimination" below).
  *  - Blocks are numbered b = 2n + s with s = 0 for sigma = +1 (up) and s = 1
  *    for sigma = -1 (down).
  */
@@ -316,8 +317,9 @@ sca_status sca_set_wait_limit(sca_ctx* ctx, int64_t cycles);
  * [n_w, 2 n_w).  The resolvents go through the same batched elimination as the gradient, in
  * batches of n_omega frequencies (the context's block slots), with partial pivoting unless
  * eta > 4|t| or the context is set to SCA_PIVOT_NONE (dense elimination, eta < 0.03 |t|: the
- * mixed precisions take Im G_ii from the float32 inverse without refinement).  Invalidates the inverses kept for
- * sca_backward_dev.  SCA_EINVAL for bad arguments, SCA_ENONFINITE for a singular resolvent. */
+ * mixed precisions take Im G_ii from the float32 inverse without refinement).  Invalidates the
+ * inverses kept for sca_backward_dev.  SCA_EINVAL for bad arguments, SCA_ENONFINITE for a singular
+ * resolvent. */
 sca_status sca_dos(sca_ctx* ctx, const double* phi_host, const double* w_host, int32_t n_w,
                    double eta, double* rho_out);
 
@@ -352,8 +354,9 @@ sca_status sca_metropolis_step(sca_ctx* ctx, int32_t n_steps, double* omega_trac
  *     elsewhere as a dense complex-symmetric (LDL^T-type) elimination that updates one
  *     triangle on the tensor-core path.  The paper has no such variant.  -i A_{n,sigma} has
  *     Hermitian part omega_n I > 0, so every leading principal minor is nonzero and the
- *     elimination exists; its growth has no a-priori bound and rises as omega_n falls (the largest growth met in tests is below 10, down to
- *     T = 0.02).  The fused small-block path (N <= 144) always pivots.
+ *     elimination exists; its growth has no a-priori bound and rises as omega_n falls (the largest
+ *     growth met in tests is below 10, down to T = 0.02).  The fused small-block path (N <= 144)
+ *     always pivots.
  * Applies from the next call on the context; any other mode is SCA_EINVAL. */
 typedef enum { SCA_PIVOT_PARTIAL = 0, SCA_PIVOT_NONE = 1, SCA_PIVOT_AUTO = 2 } sca_pivot;
 sca_status sca_set_pivoting(sca_ctx* ctx, int32_t mode);
@@ -363,8 +366,8 @@ sca_status sca_set_pivoting(sca_ctx* ctx, int32_t mode);
  * SCA_PREC_FP32 (default: the blocks' compute type) or SCA_PREC_FP64 (float64 arithmetic on
  * the float32 blocks; the doubled shared-memory panel narrows the sub-panels, e.g. to 4
  * columns at N = 1600).  While SCA_PREC_FP64 is set on them, the context takes the dense
- * elimination.  The pivot-block inverses and the contractions are unchanged.  Float64 contexts accept only SCA_PREC_FP64.  Applies from the
- * next call; SCA_EINVAL otherwise. */
+ * elimination.  The pivot-block inverses and the contractions are unchanged.  Float64 contexts
+ * accept only SCA_PREC_FP64.  Applies from the next call; SCA_EINVAL otherwise. */
 sca_status sca_set_panel_precision(sca_ctx* ctx, int32_t prec);
 
 /* SM partitions for the two block groups of the dense elimination (driver green contexts; the
@@ -406,12 +409,12 @@ sca_status sca_sm_partition(sca_ctx* ctx, int32_t* pivoted_sms, int32_t* dominan
  * kernels above, so they are not part of any sum), 13 update of the rest of a pivoted outer
  * panel after each sub-panel, 14 rank-nb factors of the pivoted group, 15 the first update of a
  * merged pair of elimination steps of the dominant blocks (only the second step's row and column
- * strips; the merged update of the rest is kind 5), 16 the nested elimination (with its diag(G) where one
- * launch does both), 17 its diag(G) from resident fronts.  enable = 1 times the dense elimination, which the context then
- * takes (kinds 0 to 15 are its kernels); enable = 2 times whatever the context takes without
- * profiling.  Enabling resets the counters.  Timing adds a small host overhead per launch; keep it off when measuring
- * throughput.  With the environment variable SCA_PROFILE_TRACE set to a file name, each
- * synchronisation also appends the launches it collected to that file, one line each:
+ * strips; the merged update of the rest is kind 5), 16 the nested elimination (with its diag(G)
+ * where one launch does both), 17 its diag(G) from resident fronts.  enable = 1 times the dense
+ * elimination, which the context then takes (kinds 0 to 15 are its kernels); enable = 2 times
+ * whatever the context takes without profiling.  Enabling resets the counters.  Timing adds a
+ * small host overhead per launch; keep it off when measuring throughput.  With the environment
+ * variable SCA_PROFILE_TRACE set to a file name, each synchronisation also appends the launches it collected to that file, one line each:
  * kind name, stream index (order of first use), start and duration in ms from the first. */
 sca_status sca_profile_enable(sca_ctx* ctx, int32_t enable);
 sca_status sca_profile_read(sca_ctx* ctx, int32_t kind, double* total_ms, uint64_t* launches);

@@ -97,7 +97,9 @@ sca_params bucket_shape(int32_t L, int32_t prec, int cap) {
 
 bool bucketed(const sca_params& p) {
   const int N = p.L * p.L;
-  return N > (p.prec == SCA_PREC_FP64 ? 64 : 144);  // smaller sizes use the fused kernel
+  // smaller requests have a context of their own: the fused kernel's sizes (4 x 4, and below the
+  // nested elimination's line all of them)
+  return N > (p.prec == SCA_PREC_FP64 ? 64 : 144);
 }
 
 sca_status bucket_create(int32_t L, int32_t prec, int cap, Bucket** out) {

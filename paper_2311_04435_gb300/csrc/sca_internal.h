@@ -198,8 +198,8 @@ enum KernelKind {
   kPanelUpd,   // pivoted group: update of the rest of the outer panel after a sub-panel
   kPrepPiv,    // pivoted group: rank-nb factors
   kUpdateCross,  // merged two-step update: the first step's update of the second step's strips
-  kNestUp,     // nested elimination, one level of fronts
-  kNestDown,   // nested elimination, one level of diag(G)
+  kNestUp,     // nested elimination: all of it in one launch, or one level on the way up
+  kNestDown,   // its diag(G) from resident fronts, or one level of it
   kKinds
 };
 

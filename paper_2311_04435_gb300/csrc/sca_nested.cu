@@ -26,10 +26,10 @@
 // This GPU does 64 float32 FMAs in the time of one float64 FMA, so double-float is 5 times as
 // fast as float64 and keeps 24 bits more than the float32 blocks of the dense paths.  The few
 // blocks of small Im z: sums of three float32 (72 bits, 46 operations per real multiply-add, which
-// takes no longer than one of float64 does here: a 20x20 float64 density of states 1013 us in float64,
-// 1004 in these, 11324 in double-double).  They go beside the others, on a stream of their own, in
-// clusters of up to eight CTAs per block: a 20x20 gradient, T = 0.05, 124 blocks in float64 and 4 in
-// these, 1009 us, 1004 with all 128 in float64; 512 blocks, T = 0.1, 2 of them in these, 2273 / 2264
+// takes no longer than one of float64 does here: a 20x20 float64 density of states 1013 us in
+// float64, 1004 in these, 11324 in double-double).  They go beside the others, on a stream of their
+// own, in clusters of up to eight CTAs per block: a 20x20 gradient, T = 0.05, 124 blocks in float64
+// and 4 in these, 1009 us, 1004 with all 128 in float64; 512 blocks, T = 0.1, 2 of them in these, 2273 / 2264
 // (2296 with clusters of eight where the others take longer than one block's time per SM).
 // On small lattices their dependent chain shows: 8x8 densities of states 287 us, 151 in float64.
 //
@@ -687,7 +687,9 @@ struct Block {
 };
 
 // The functions below are calls of their own, with offsets into shared memory instead of pointers:
-// inlined into one kernel they spill, and through a call a pointer would lose its address space.
+// inlined into one kernel their registers add up (as calls, the forms of 128 registers spill 124
+// bytes or less in float64 and double-float, those of 64 registers up to 292), and through a call a
+// pointer would lose its address space.
 // Their inner loops have no branch per row, which would split them into blocks of two dependent
 // chains each; rows past the end repeat the last one and are dropped.
 
@@ -1064,9 +1066,11 @@ __device__ __forceinline__ void front_down(const Block<Z>& B, int node, const Gr
       for (int j = tid & 31; j < r; j += 32) X[i * ldx + j] = F[(o + i) * m + o + w + j];
     gr.sync();
     if (direct)
-      times_fit<Z, true, NT == 512 ? 4 : 2>(gr, w, r, r, off(X), ldx, off(Y), ldx, G, 0, mp, off(map), (Z*)nullptr, 0);
+      times_fit<Z, true, NT == 512 ? 4 : 2>(gr, w, r, r, off(X), ldx, off(Y), ldx, G, 0, mp,
+                                            off(map), (Z*)nullptr, 0);
     else if (r > 0)
-      times_fit<Z, false, NT == 512 ? 4 : 2>(gr, w, r, r, off(X), ldx, off(Y), ldx, R, 0, m, 0, (Z*)nullptr, 0);
+      times_fit<Z, false, NT == 512 ? 4 : 2>(gr, w, r, r, off(X), ldx, off(Y), ldx, R, 0, m, 0,
+                                             (Z*)nullptr, 0);
     gr.sync();
     // ---- G_pp = P + Y (-X)^T, lower triangle; ks threads share an entry's sum (by the front's
     // shape alone: the order of a sum must not depend on how many threads there are)
@@ -1206,7 +1210,7 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : 1) k_nested(NestArgs<Z> a)
   }
 }
 
-// Im Tr G per block for a density of states: fixed-order sum of the row that k_nest_down wrote.
+// Im Tr G per block for a density of states: fixed-order sum of the row that k_nested wrote.
 __global__ void __launch_bounds__(256) k_nest_trace(int N, int b0, const double* gd, double* tr) {
   __shared__ double part[256];
   const int b = b0 + blockIdx.x;

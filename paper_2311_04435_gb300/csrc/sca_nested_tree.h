@@ -64,7 +64,6 @@ struct Node {
 
 struct Level {
   int first, count;    // nodes [first, first + count), all at one depth
-  int mmax, wmax, qmax;
 };
 
 struct Tree {
@@ -90,7 +89,7 @@ class Builder {
     root.parent = -1;
     cur.push_back(root);
     while (!cur.empty()) {
-      Level lv{(int)t.nodes.size(), (int)cur.size(), 0, 0, 0};
+      const Level lv{(int)t.nodes.size(), (int)cur.size()};
       next.clear();
       for (const Region& r : cur) {
         const int id = (int)t.nodes.size();
@@ -144,9 +143,6 @@ class Builder {
           const int c = par.child[0] < 0 ? 0 : 1;
           par.child[c] = id;
         }
-        lv.mmax = std::max(lv.mmax, m);
-        lv.wmax = std::max(lv.wmax, n.pw);
-        lv.qmax = std::max(lv.qmax, n.q);
         t.nodes.push_back(n);
         for (int k = 0; k < nch; ++k) {
           ch[k].parent = id;

@@ -6,8 +6,9 @@
 // cudaMalloc / cudaFree can synchronise the whole device.  sca_grad_noalloc_dev serves them:
 // its workspace is the file-scope device array below, which every GPU that loads this library
 // holds until the process exits, and the call makes no cudaMalloc, cudaFree or other
-// allocating call.  It runs the same kernels as sca_grad_dev, on float64 or float32 blocks
-// with CUDA-core contractions, and processes the blocks in as many chunks as the array needs.
+// allocating call.  It runs the dense elimination's kernels (sca_grad_dev takes the nested one
+// where that applies), on float64 or float32 blocks with CUDA-core contractions, and processes the
+// blocks in as many chunks as the array needs.
 #include <cuda_runtime.h>
 
 #include <algorithm>

@@ -3,7 +3,7 @@
 //
 // One worker thread owns every device object.  Each round it
 //   1. admits queued requests in arrival order while a slot is free and the request's memory
-//      fits the remaining budget.  Small requests (blocks that the fused kernel holds) get a
+//      fits the remaining budget.  Small requests (of the fused kernel's sizes) get a
 //      context and stream of their own; larger ones join the size bucket of their lattice
 //      size and precision (one shared workspace of kBucketSlots block slots, created with the
 //      bucket's first request and counted against the budget until its last one leaves; then
