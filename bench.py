@@ -442,10 +442,13 @@ def run_ours(args):
                 "timed_steps": args.fp64_steps, "warmup": 1,
                 "mixed_over_fp64": round(ms64 / ms_per_step, 2)}
 
-    # ---------------- the same step without interchanges in any block (the nested elimination
-    # has none; on the dense path a variant beside the paper's pivoted LU, not the headline)
-    nopiv = None
-    if args.variant_steps > 0 and rank == 0 and api.pivoted_blocks(params) > 0:
+    # ---------------- the same step without interchanges in any block, and in the other split
+    # precision: variants of the dense path.  On the nested path both are the headline's kernels
+    # and arithmetic (no interchanges, double-float), so they are not timed again.
+    same = {"same_as": "headline", "why": "the nested elimination has no interchanges and computes "
+            "every reduced precision in double-float"} if nested else None
+    nopiv = same
+    if not nested and args.variant_steps > 0 and rank == 0 and api.pivoted_blocks(params) > 0:
         cn = api.Context(params)
         cn.set_stream(stream)
         cn.set_pivoting("none")
@@ -463,9 +466,8 @@ def run_ours(args):
                  "timed_steps": args.variant_steps, "warmup": 1, "final_omega": omn,
                  "final_gmax": gmn}
 
-    # ---------------- the other split precision beside it (same workload, same path)
-    other = None
-    if args.variant_steps > 0 and rank == 0 and prec in ("3xtf32", "bf16x3"):
+    other = same
+    if not nested and args.variant_steps > 0 and rank == 0 and prec in ("3xtf32", "bf16x3"):
         oprec = "3xtf32" if prec == "bf16x3" else "bf16x3"
         po = api.Params(wl.L, wl.n_omega, U=wl.U, T=wl.T, delta=wl.delta, t=wl.t, mu=wl.mu,
                         prec=oprec)
@@ -554,6 +556,9 @@ def run_ours(args):
             mixed_vs_oracle[prec + "_fp64_panel"] = block_errors(blk_p64, sample, o_ld, o_gd, npb)
         if blk_64 is not None:
             mixed_vs_oracle["fp64"] = block_errors(blk_64, sample, o_ld, o_gd, npb)
+        mixed_vs_oracle["arithmetic"] = {
+            prec: "double-float, 48 bits (nested elimination)" if nested else "as named (dense)",
+            prec + "_fp64_panel": "as named (dense)"}
         mixed_vs_oracle["note"] = ("per-block ln|det A_b| and sigma Re G_b,ii at the seeded "
                                    "start field against the FP64 oracle on the CPU baseline's "
                                    "sample of blocks")
