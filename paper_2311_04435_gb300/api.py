@@ -288,7 +288,8 @@ class Context:
     def profile(self, enable: bool | int = True):
         """True: time the dense elimination's kernels, which the context then takes; 2: time
         whatever it takes without profiling; False: off."""
-        check(_lib.lib().sca_profile_enable(self._h, int(enable)))
+        mode = 2 if not isinstance(enable, bool) and enable == 2 else int(bool(enable))
+        check(_lib.lib().sca_profile_enable(self._h, mode))
 
     def profile_read(self) -> dict:
         out = {}

@@ -58,6 +58,19 @@ def test_auto_below_the_line_pivots():
         assert _same(c.blocks(phi), new) and not _same(none, new)
 
 
+def test_profile_takes_any_truth_value():
+    p = api.Params(8, 2, U=4.0, T=0.3, delta=0.4, prec="fp32")
+    phi = inputs.random_phi(4, p.N, 1.0)
+    with api.Context(p) as c:
+        for enable, dense, nested in ((None, 0, 0), ("", 0, 0), ("on", 1, 0), (True, 1, 0), (2, 0, 1),
+                                      (5, 1, 0), (0, 0, 0)):
+            c.profile(enable)
+            c.blocks(phi)
+            prof = c.profile_read()
+            assert (prof["panel"][1] > 0) == bool(dense), enable
+            assert (prof["nest_up"][1] > 0) == bool(nested), enable
+
+
 def test_environment_switch_counts_at_creation(monkeypatch):
     p = api.Params(14, 3, U=4.0, T=0.3, delta=0.4, prec="bf16x3")
     phi = inputs.random_phi(3, p.N, 1.0)

@@ -38,3 +38,28 @@ def test_served_requests_equal_the_same_alone(prec):
         mixed = [srv.poll(rid, 256) for rid in ids]
     for x, y in zip(alone, mixed):
         assert x.steps == y.steps and x.omega == y.omega and np.array_equal(x.phi, y.phi)
+
+
+@pytest.mark.parametrize("L,nw,T,prec", [(14, 20, 0.05, "fp64"), (14, 100, 0.05, "fp64"),
+                                         (8, 90, 0.03, "fp32"), (20, 30, 0.1, "bf16x3")])
+def test_captured_gradient_replays_to_the_bit(L, nw, T, prec):
+    """Blocks of one and two arithmetics, one launch or one per level: every stream that an
+    evaluation uses forks from the caller's and joins it again."""
+    torch = pytest.importorskip("torch")
+    p = api.Params(L, nw, U=4.0, T=T, delta=0.3, prec=prec)
+    fields = [inputs.random_phi(7 + k, p.N, 0.4) for k in range(2)]
+    with api.Context(p) as c:
+        want = [c.grad(f) for f in fields]
+        x = torch.tensor(fields[0], dtype=torch.float64, device="cuda")
+        s = torch.cuda.Stream()
+        with torch.cuda.stream(s):
+            c.grad_dev(x)
+            s.synchronize()
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph, stream=s):
+                om, g = c.grad_dev(x)
+            for f, (om_ref, g_ref) in zip(fields, want):
+                x.copy_(torch.tensor(f, dtype=torch.float64))
+                graph.replay()
+                s.synchronize()
+                assert float(om) == om_ref and np.array_equal(g.cpu().numpy(), g_ref)
