@@ -491,32 +491,29 @@ __device__ __forceinline__ Zw zinv(Zw z, double* mag2 = nullptr) {
   return r;
 }
 
-// 1 / z for any z.  The float32 forms above square z within float32's range (no pivot is too
-// small: each is at least Im z >= 1e-9 in modulus); a larger one, which a site term makes, goes
-// through float64 (53 bits are enough there: what it couples with is 2^-60 of it or less).
+// The float32 forms square numbers within float32's range, so site terms of 2^60 and more come in as
+// 2^60: what such a site couples with changes by 2^-60 t^2 or less, and its own G_ii, 1 / a, is as
+// far below rounding either way.  Its share of |det A|^2 is put right where it is read: `far`.
+// (No pivot is too small: each is at least Im z >= 1e-9 in modulus.)
 template <typename Z>
 constexpr bool kNarrow = std::is_same<Z, Zf>::value || std::is_same<Z, Zt>::value;
-__device__ __forceinline__ bool beyond(double x) {  // |x| >= 2^60, without the slow pipe
+__device__ __forceinline__ bool beyond(double x) {  // |x| >= 2^60 or not finite, off the slow pipe
   return (__double2hiint(x) & 0x7fffffff) >= 0x43b00000;
 }
-__device__ __forceinline__ bool beyond(Zf z) { return fmaxf(fabsf(z.rh), fabsf(z.ih)) >= 0x1p60f; }
+__device__ __forceinline__ bool beyond(Zf z) { return fabsf(z.rh) >= 0x1p60f; }
 __device__ __forceinline__ bool beyond(Zt z) {
   float r, i;
   f2_get(z.h, r, i);
-  return fmaxf(fabsf(r), fabsf(i)) >= 0x1p60f;
+  return fabsf(r) >= 0x1p60f;
 }
 __device__ __forceinline__ bool beyond(Zd) { return false; }
 __device__ __forceinline__ bool beyond(Zw) { return false; }
 template <typename Z>
-__device__ __forceinline__ Z zinv_any(Z z, double* mag2 = nullptr) {
-  if (!beyond(z)) return zinv(z, mag2);
-  const double re = zre(z), im = zim(z);
-  const double m = fma(im, im, __dmul_rn(re, re)), d = 1.0 / m;
-  if (mag2) *mag2 = m;
-  Z r;
-  zset(r, re * d, -im * d);
-  return r;
+__device__ __forceinline__ double near_term(double re) {
+  return kNarrow<Z> && beyond(re) ? copysign(0x1p60, re) : re;
 }
+// (|a| / 2^60)^2 of a site term beyond 2^60, not finite where it is not.
+__device__ __forceinline__ double far(double re) { return (re * 0x1p-60) * (re * 0x1p-60); }
 
 // A product of moduli squared as mantissa in [1, 2) and exponent: a node's share of |det A|^2.
 // One logarithm per node at the root instead of one per pivot (a float64 logarithm costs about
@@ -652,18 +649,6 @@ struct Group {
     else
       asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(size) : "memory");
   }
-  // The same, and whether q holds in any of the threads.
-  __device__ __forceinline__ bool sync_any(bool q) const {
-    if (size == 32) return __any_sync(0xffffffffu, q);
-    int r;
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\tsetp.ne.s32 p, %3, 0;\n\tbar.red.or.pred q, %1, %2, p;\n\t"
-        "selp.s32 %0, 1, 0, q;\n\t}"
-        : "=r"(r)
-        : "r"(bar), "r"(size), "r"((int)q)
-        : "memory");
-    return r != 0;
-  }
 };
 
 // Offset of a pointer into the CTA's dynamic shared memory.
@@ -687,8 +672,8 @@ struct Block {
 };
 
 // The functions below are calls of their own, with offsets into shared memory instead of pointers:
-// inlined into one kernel their registers add up (as calls, the forms of 128 registers spill 124
-// bytes or less in float64 and double-float, those of 64 registers up to 292), and through a call a
+// inlined into one kernel their registers add up (as calls, the forms of 128 registers spill 72
+// bytes or less in float64 and double-float, those of 64 registers up to 296), and through a call a
 // pointer would lose its address space.
 // Their inner loops have no branch per row, which would split them into blocks of two dependent
 // chains each; rows past the end repeat the last one and are dropped.
@@ -697,9 +682,8 @@ struct Block {
 // (g, j), (g + G, j), ... of the w x w block, S of them, G = size / w.  A step needs the pivot's
 // row, its column and its reciprocal; their owners write them to shared memory as soon as they
 // have them (two buffers, one barrier per step).  The result replaces F11, negated, and goes to
-// the front.  kAny: a pivot may be beyond 2^60 (a check inside the chain of pivots costs 2 to 4 %,
-// so fronts without such a site term take the form without).
-template <typename Z, int S, bool kAny>
+// the front.
+template <typename Z, int S>
 __device__ __noinline__ void invert(const Group gr, int w, int F11o, int rowo, int colo,
                                     int mago, Z* Fo, int m) {
   using Acc = typename AccOf<Z>::type;
@@ -723,7 +707,7 @@ __device__ __noinline__ void invert(const Group gr, int w, int F11o, int rowo, i
 #pragma unroll
       for (int s = 0; s < S; ++s) colb[row[s]] = zneg(reg[s]);
     }
-    if (gr.tid == 0) colb[w] = kAny ? zinv_any(reg[0], mag) : zinv(reg[0], mag);
+    if (gr.tid == 0) colb[w] = zinv(reg[0], mag);
   }
 #pragma unroll 1
   for (int c = 0; c < w; ++c) {
@@ -750,7 +734,7 @@ __device__ __noinline__ void invert(const Group gr, int w, int F11o, int rowo, i
 #pragma unroll
         for (int s = 1; s < S; ++s) nr = zsel(row[s] == c + 1, reg[s], nr);
         rn[j] = nr;
-        if (j == c + 1) cn[w] = kAny ? zinv_any(nr, mag + j) : zinv(nr, mag + j);
+        if (j == c + 1) cn[w] = zinv(nr, mag + j);
       }
       if (j == c + 1) {
 #pragma unroll
@@ -932,21 +916,21 @@ __device__ __forceinline__ void front_up(const Block<Z>& B, int node, const Grou
     cm0[i] = nd.child[0] >= 0 ? B.tab[nd.cmap[0] + i] : (int16_t)-1;
     cm1[i] = nd.child[1] >= 0 ? B.tab[nd.cmap[1] + i] : (int16_t)-1;
   }
-  bool big = false;
-  for (int i = tid; i <= p; i += size) {
-    const double re = i < p ? B.zr - site_energy(B.la, B.tab[nd.sites + i], B.sg) : B.la.t;
-    zset(diag[i], re, i < p ? B.zi : 0.0);
-    big |= beyond(re);
-  }
+  for (int i = tid; i <= p; i += size)
+    zset(diag[i],
+         i < p ? near_term<Z>(B.zr - site_energy(B.la, B.tab[nd.sites + i], B.sg)) : B.la.t,
+         i < p ? B.zi : 0.0);
   if (nd.blacks) {
     for (int i = tid; i < m; i += size) adj[i] = B.tab[nd.adj + i];
     if (tid < 32) {
       double m2 = 1.0;
       if (tid < nd.blacks) {
         Z z, t2;
-        zset(z, B.zr - site_energy(B.la, B.tab[nd.bsite + tid], B.sg), B.zi);
+        const double re = B.zr - site_energy(B.la, B.tab[nd.bsite + tid], B.sg);
+        zset(z, near_term<Z>(re), B.zi);
         zset(t2, B.la.t * B.la.t, 0.0);
-        bt[tid] = zneg(zmul(t2, zinv_any(z, &m2)));
+        bt[tid] = zneg(zmul(t2, zinv(z, &m2)));
+        if (kNarrow<Z> && beyond(re)) m2 *= far(re);
       }
       det_mul(m2, mant, expo, B.flags);
     }
@@ -971,10 +955,7 @@ __device__ __forceinline__ void front_up(const Block<Z>& B, int node, const Grou
   f.adj = off(adj);
   f.bt = off(bt);
   f.diag = off(diag);
-  if constexpr (kNarrow<Z>)
-    big = gr.sync_any(big);
-  else
-    gr.sync();
+  gr.sync();
   for (int pa = 0; pa < nd.npan; ++pa) {
     const int o = pa * pw, w = min(pw, p - o), l = m - o, r = l - w;
     const int lda = r + kRows;  // row blocks read up to kRows - 1 entries past r
@@ -991,18 +972,21 @@ __device__ __forceinline__ void front_up(const Block<Z>& B, int node, const Grou
       }
     gr.sync();
     Z* Fo = F + (size_t)o * (m + 1);
-    if (kNarrow<Z> && big)
-      invert<Z, kSlots, true>(gr, w, off(F11), off(rowb), off(colb), off(mag), Fo, m);
-    else if (w <= size / w)
-      invert<Z, 1, false>(gr, w, off(F11), off(rowb), off(colb), off(mag), Fo, m);
+    if (w <= size / w)
+      invert<Z, 1>(gr, w, off(F11), off(rowb), off(colb), off(mag), Fo, m);
     else
-      invert<Z, kSlots, false>(gr, w, off(F11), off(rowb), off(colb), off(mag), Fo, m);
+      invert<Z, kSlots>(gr, w, off(F11), off(rowb), off(colb), off(mag), Fo, m);
     gr.sync();
     if (r > 0)
       times_fit<Z, false, 0>(gr, w, w, r, off(F11), w, off(X), r, (const Z*)F, off(A), lda, 0,
                                  Fo + w, m);
     gr.sync();
-    if (tid < 32) det_mul(tid < w ? mag[tid] : 1.0, mant, expo, B.flags);
+    if (tid < 32) {
+      double m2 = tid < w ? mag[tid] : 1.0;
+      if (kNarrow<Z> && tid < w && beyond(diag[o + tid]))
+        m2 *= far(B.zr - site_energy(B.la, B.tab[nd.sites + o + tid], B.sg));
+      det_mul(m2, mant, expo, B.flags);
+    }
     // ---- the rest; fewer rows per thread where more would leave threads idle
     Z* R = F + (size_t)(o + w) * (m + 1);
     auto cost = [&](int kr) {
@@ -1124,9 +1108,9 @@ __device__ __forceinline__ void front_down(const Block<Z>& B, int node, const Gr
       sum = zadd(sum, zshfl_xor(sum, 2));
       if (u == 0 && b0 + tid / 4 < nd.blacks) {
         Z z, t2;
-        zset(z, B.zr - site_energy(B.la, s, B.sg), B.zi);
+        zset(z, near_term<Z>(B.zr - site_energy(B.la, s, B.sg)), B.zi);
         zset(t2, B.la.t * B.la.t, 0.0);
-        const Z ai = zinv_any(z);
+        const Z ai = zinv(z);
         const Z g = zadd(ai, zmul(zmul(zmul(ai, t2), ai), sum));
         B.gd[s] = B.la.zshift ? zim(g) : B.sg * zre(g);
       }
